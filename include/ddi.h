@@ -104,7 +104,10 @@ typedef struct {
                           (3D), 8 cells in x running along y (2D).  Applies to FP32 plans whose fine grid
                           is a multiple of 8 in x (3D: and in y) and at least w + 7 cells in x (3D: w + 7
                           in y and w in z; 2D: w in y), and not to compensated 2D plans; DDI_ERR_ARG
-                          otherwise; `chunk` = visits per work item */
+                          otherwise; `chunk` = visits per work item.  The automatic choice also gives
+                          columns to FP64 3D plans of 2048 processed nodes and more whose fine grid
+                          fits (at least w + 7 cells in x and y, multiples of 8) and whose `tile` is
+                          left at 0 */
   int check_finite;    /* NaN / Inf in rho: the pad pass of every evaluation records them in a device
                           flag of the plan (at no cost for finite input).  0 => ddi_apply stays
                           asynchronous and the flag is read by ddi_plan_check (and by ddi_apply_host,

@@ -1,0 +1,512 @@
+// Column spread of 3D plans (type 1, Sec. 2.1, Eq. DDI-Trun1), FP32 and FP64.
+//
+// A warp takes a unit: a range of groups of one column and a window of z-planes.  Lane (lx, ly)
+// owns the cells (lx, ly) and (lx, ly + 4) of the column and keeps W planes of both in
+// registers: plane p lives in register p mod W, so the window advances by writing its oldest
+// plane and never moves a register.  For a run of one z class the lane sums
+// g = sum c_q psi_x psi_y over the run's visits and then adds g psi_z to its W planes once.
+// No shared-memory read-modify-write and no atomics: each cell belongs to one lane.  Planes that
+// several units touch go to partial slots (contiguous per plane, in unit order) that
+// k_reduce_col3 sums in order: results are deterministic.
+//
+// What bounds it.  FP64: this part issues a warp's FP64 instruction over 16 cycles of an SM, so
+// the count of FP64 operations is the time.  A tile plane's read-modify-write costs 3 per tap and
+// shares nothing between nodes; here the taps of a ring's nodes are summed before psi_z, so a
+// visit costs 6 per lane (its 64 cells) and a run 4 W.  FP32: instruction issue.  The rows a visit
+// needs do not change between evaluations, so the plan stores them laid out per group
+// (columns.cuh) and the warp copies a group ahead with cp.async instead of gathering and
+// zero-padding each row.  Its inner step takes two visits at once: four shared loads bring their
+// u = c psi_x (real, imaginary) and psi_y (two cells) as pairs, four packed FMAs add them, and no
+// value has to be duplicated into a pair.  Units are cut to equal work (plan.cu), because one
+// warp that walks a sparse column's 256 planes alone outlasts the rest of the launch.
+//
+// Measured (spread + reduction): 128^3 FP32, 524288 nodes: 198 -> 101 us (4 CTAs per SM at up to
+// 128 registers; 5 CTAs at 96 spill and take 118); 192^3 FP32 564 -> 277 us; 128^3 FP64 27.4 ->
+// 2.6 ms (the FP64 operations above take 2.3 ms at this part's rate).
+#include <algorithm>
+#include <cstring>
+#include <mutex>
+
+#include "columns.cuh"
+
+namespace ddi {
+namespace {
+
+constexpr int kColThreads3 = 128;  // 4 warps per CTA, each taking units on its own
+
+template <typename T> using p2_t = cx_t<T>;
+
+// c + a b per component
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
+  return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+}
+template <typename C> __device__ __forceinline__ C both(decltype(C::x) v) { return cmk<C>(v, v); }
+// the sum of a.x b.x + a.y b.y over a run, as a pair (FP32: packed) or a scalar chain (FP64: no
+// addition to close it); dot_sum closes it
+__device__ __forceinline__ float2 dot2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ double2 dot2(double2 a, double2 b, double2 c) {
+  return make_double2(fma(a.y, b.y, fma(a.x, b.x, c.x)), 0.0);
+}
+__device__ __forceinline__ float dot_sum(float2 v) { return v.x + v.y; }
+__device__ __forceinline__ double dot_sum(double2 v) { return v.x; }
+
+// a += x with the rounding error of the sum carried in c (compensated summation, Kahan):
+// y = x - c, t = a + y, c = (t - a) - y, a = t
+__device__ __forceinline__ void kahan_add2(float2& a, float2& c, float2 x) {
+  const float2 y = __fadd2_rn(x, make_float2(-c.x, -c.y));
+  const float2 t = __fadd2_rn(a, y);
+  c = __fadd2_rn(__fadd2_rn(t, make_float2(-a.x, -a.y)), make_float2(-y.x, -y.y));
+  a = t;
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+// a group's image into the warp's shared memory, 16 bytes per lane and step
+template <int BYTES>
+__device__ __forceinline__ void copy_image(unsigned char* dst, const unsigned char* src, int lane) {
+#pragma unroll
+  for (int i = 0; i < (BYTES + 511) / 512; ++i) {
+    const int o = (i * 32 + lane) * 16;
+    if ((i + 1) * 512 <= BYTES || o < BYTES) cp_async16(dst + o, src + o);
+  }
+}
+
+struct ColArgs3 {
+  int nf[3];
+  int ncx;
+  const ColUnit* units;
+  int nunits;
+  int* counter;
+  const unsigned char* image;  // [group][ColImage::BYTES]
+  const int* nodes;            // [group][32] node of each visit, -1: none
+  const void* c;               // [node]
+  void* fine;
+  void* partial;               // [slot][kColY * kColX]
+  const int* dest;             // [unit][kColPlanes]: partial slot of each plane of its window, -1: the fine grid
+};
+
+// per-warp shared memory of the spread: two group images and u = c psi_x of each visit, rows of
+// 32 visits per x cell, real parts, then imaginary parts
+template <typename T, int W>
+struct SpreadSmem {
+  static constexpr int U = 2 * ColImage<T, W>::BYTES;
+  static constexpr int BYTES = (U + 16 * ColImage<T, W>::RS + 127) / 128 * 128;
+};
+
+#define DDI_COL3_CASES(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15)
+
+template <typename T, int W, bool COMP>
+__global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_spread_col3(ColArgs3 a) {
+  using C = cx_t<T>;
+  using I = ColImage<T, W>;
+  using S = SpreadSmem<T, W>;
+  static_assert(W <= 16 && W % 2 == 0, "planes in register pairs 0..W/2-1 of the window");
+  static_assert(!COMP || sizeof(T) == 4, "compensated sums are built for FP32");
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* sm = smem_raw + warp * S::BYTES;
+  unsigned char* su = sm + S::U;
+  const int lx = lane & 7, ly = lane >> 3;
+  const int nfx = a.nf[0], nfz = a.nf[2];
+  const long long plane = (long long)nfx * a.nf[1];
+  const C* __restrict__ cg = static_cast<const C*>(a.c);
+  // units are taken from a counter, the first one by position; the next unit's index, entry and
+  // first group are requested while the current one is being worked on
+  const int nwarps = gridDim.x * (blockDim.x >> 5);
+  int un = warp * gridDim.x + blockIdx.x;
+  int uw = 0;            // word (lane mod 8) of the next unit's entry
+  int n0 = -1, n1 = -1;  // node of this lane in the next unit's first and second group
+  int buf = 0;
+  static_assert(sizeof(ColUnit) == 32, "eight words per unit");
+  auto load_unit = [&]() { uw = __ldg(reinterpret_cast<const int*>(a.units + un) + (lane & 7)); };
+  auto word = [&](int k) { return __shfl_sync(0xffffffffu, uw, k); };
+  auto request_first = [&]() {  // the next unit's first image into the free buffer
+    n0 = n1 = -1;
+    const int lo = word(1), hi = word(2);
+    if (un < a.nunits && lo < hi) {
+      copy_image<I::BYTES>(sm + buf * I::BYTES, a.image + (size_t)lo * I::BYTES, lane);
+      n0 = __ldg(a.nodes + (size_t)lo * 32 + lane);
+      if (lo + 1 < hi) n1 = __ldg(a.nodes + (size_t)(lo + 1) * 32 + lane);
+    }
+    cp_async_commit();
+  };
+  if (un < a.nunits) load_unit();
+  request_first();
+  while (un < a.nunits) {
+    const ColUnit U = {word(0), word(1), word(2), word(3), word(4), word(5), word(6), word(7)};
+    int nx = 0;
+    if (lane == 0) nx = atomicAdd(a.counter, 1);
+    // where each plane of the window goes, one plane per lane
+    static_assert(kColPlanes == 32, "a lane per plane of the window");
+    const int mydest = __ldg(a.dest + (size_t)un * kColPlanes + lane);
+    const int cx = U.col % a.ncx, cy = U.col / a.ncx;
+    const long long cell = (long long)(cy * kColY + ly) * nfx + cx * kColX + lx;
+    // planes 2 q and 2 q + 1 (mod W) of cells 0 and 1, real and imaginary parts; compensations
+    C r0[W / 2], i0[W / 2], r1[W / 2], i1[W / 2];
+    C cr0[COMP ? W / 2 : 1], ci0[COMP ? W / 2 : 1], cr1[COMP ? W / 2 : 1], ci1[COMP ? W / 2 : 1];
+    const C zero = cmk<C>((T)0, (T)0);
+#pragma unroll
+    for (int q = 0; q < W / 2; ++q) {
+      r0[q] = i0[q] = r1[q] = i1[q] = zero;
+      if constexpr (COMP) cr0[q] = ci0[q] = cr1[q] = ci1[q] = zero;
+    }
+    if (U.lo == U.hi) {  // no visits: zeros
+      for (int z = U.z0; z < U.z1; ++z) {
+        C* dst = static_cast<C*>(a.fine) + (z >= nfz ? z - nfz : z) * plane + cell;
+        __stcs(dst, zero);
+        __stcs(dst + 4 * nfx, zero);
+      }
+      un = nwarps + __shfl_sync(0xffffffffu, nx, 0);
+      if (un < a.nunits) load_unit();
+      request_first();
+      continue;
+    }
+    int zb = U.z0, zslot = U.z0 % W;
+    // write plane zb (direct, or a partial slot when other units touch it), clear its registers
+    auto flush = [&]() {
+      C v0 = zero, v1 = zero;
+      switch (zslot) {
+#define DDI_TAKE3(R)                                                      \
+  case R:                                                                 \
+    if constexpr (R < W) {                                                \
+      constexpr int Q = R / 2;                                            \
+      if constexpr (COMP) {                                               \
+        if constexpr (R % 2 == 0) {                                       \
+          v0 = cmk<C>(r0[Q].x - cr0[Q].x, i0[Q].x - ci0[Q].x);            \
+          v1 = cmk<C>(r1[Q].x - cr1[Q].x, i1[Q].x - ci1[Q].x);            \
+          cr0[Q].x = ci0[Q].x = cr1[Q].x = ci1[Q].x = (T)0;               \
+        } else {                                                          \
+          v0 = cmk<C>(r0[Q].y - cr0[Q].y, i0[Q].y - ci0[Q].y);            \
+          v1 = cmk<C>(r1[Q].y - cr1[Q].y, i1[Q].y - ci1[Q].y);            \
+          cr0[Q].y = ci0[Q].y = cr1[Q].y = ci1[Q].y = (T)0;               \
+        }                                                                 \
+      } else if constexpr (R % 2 == 0) {                                  \
+        v0 = cmk<C>(r0[Q].x, i0[Q].x);                                    \
+        v1 = cmk<C>(r1[Q].x, i1[Q].x);                                    \
+      } else {                                                            \
+        v0 = cmk<C>(r0[Q].y, i0[Q].y);                                    \
+        v1 = cmk<C>(r1[Q].y, i1[Q].y);                                    \
+      }                                                                   \
+      if constexpr (R % 2 == 0)                                           \
+        r0[Q].x = i0[Q].x = r1[Q].x = i1[Q].x = (T)0;                     \
+      else                                                                \
+        r0[Q].y = i0[Q].y = r1[Q].y = i1[Q].y = (T)0;                     \
+    }                                                                     \
+    break;
+        DDI_COL3_CASES(DDI_TAKE3)
+#undef DDI_TAKE3
+      }
+      const int d = __shfl_sync(0xffffffffu, mydest, zb - U.z0);
+      if (d >= 0) {
+        C* dst = static_cast<C*>(a.partial) + (size_t)d * (kColX * kColY) + lane;
+        dst[0] = v0;
+        dst[32] = v1;
+      } else {
+        // streaming stores: the partial slots stay in L2 for the reduction
+        C* dst = static_cast<C*>(a.fine) + (zb >= nfz ? zb - nfz : zb) * plane + cell;
+        __stcs(dst, v0);
+        __stcs(dst + 4 * nfx, v1);
+      }
+      ++zb;
+      zslot = zslot + 1 == W ? 0 : zslot + 1;
+    };
+    // group images are copied one ahead, node values read one ahead, node indices two ahead
+    int nnext = n1;
+    C cnext = zero;
+    if (n0 >= 0) cnext = __ldg(cg + n0);
+    // after the last group: one more turn that only writes the planes left up to z1
+    for (int gi = U.lo; gi <= U.hi; ++gi) {
+      const bool end = gi == U.hi;
+      if (gi + 1 == U.hi) {
+        un = nwarps + __shfl_sync(0xffffffffu, nx, 0);
+        if (un < a.nunits) load_unit();
+      }
+      const C c = cnext;
+      cnext = zero;
+      const unsigned char* im = sm + buf * I::BYTES;
+      if (!end) {
+        if (gi + 1 < U.hi) {
+          copy_image<I::BYTES>(sm + (buf ^ 1) * I::BYTES, a.image + (size_t)(gi + 1) * I::BYTES, lane);
+          if (nnext >= 0) cnext = __ldg(cg + nnext);
+          nnext = gi + 2 < U.hi ? __ldg(a.nodes + (size_t)(gi + 2) * 32 + lane) : -1;
+        }
+        cp_async_commit();
+        cp_async_wait<1>();
+        __syncwarp();
+        buf ^= 1;
+      } else {
+        request_first();
+      }
+      // u = c psi_x, lane = visit
+      if (!end) {
+#pragma unroll
+        for (int ch = 0; ch < I::CH; ++ch) {
+          T x[I::EPC];
+          *reinterpret_cast<int4*>(x) = *reinterpret_cast<const int4*>(im + I::X + ch * 512 + lane * 16);
+#pragma unroll
+          for (int k = 0; k < I::EPC; ++k) {
+            T* dst = reinterpret_cast<T*>(su + (ch * I::EPC + k) * I::RS) + lane;
+            dst[0] = c.x * x[k];
+            *reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(dst) + 8 * I::RS) = c.y * x[k];
+          }
+        }
+      }
+      __syncwarp();
+      const int nruns = end ? 1 : *reinterpret_cast<const int*>(im + I::COUNTS + 4);
+      for (int r = 0; r < nruns; ++r) {
+        const int hd = end ? U.z1 << 12 : *reinterpret_cast<const int*>(im + I::HEAD + 4 * r);
+        const int j0 = hd & 63, j1 = (hd >> 6) & 63, sr = hd >> 12;
+        while (zb < sr) flush();
+        if (end) break;
+        // the run's sum of u psi_y, two visits at a time
+        C a0r = zero, a0i = zero, a1r = zero, a1i = zero;
+        const unsigned char* pu = su + lx * I::RS + j0 * (int)sizeof(T);
+        const unsigned char* py = im + I::Y + ly * I::RS + j0 * (int)sizeof(T);
+#pragma unroll 2
+        for (int j = j0; j < j1; j += 2) {
+          const C ur = *reinterpret_cast<const C*>(pu), ui = *reinterpret_cast<const C*>(pu + 8 * I::RS);
+          const C y0 = *reinterpret_cast<const C*>(py), y1 = *reinterpret_cast<const C*>(py + 4 * I::RS);
+          a0r = dot2(ur, y0, a0r);
+          a0i = dot2(ui, y0, a0i);
+          a1r = dot2(ur, y1, a1r);
+          a1i = dot2(ui, y1, a1i);
+          pu += sizeof(C);
+          py += sizeof(C);
+        }
+        const C g0 = cmk<C>(dot_sum(a0r), dot_sum(a0i)), g1 = cmk<C>(dot_sum(a1r), dot_sum(a1i));
+        const C* pz = reinterpret_cast<const C*>(im + I::Z + r * I::ZS);
+#pragma unroll
+        for (int q = 0; q < W / 2; ++q) {
+          const C z = pz[q];
+          if constexpr (COMP) {
+            kahan_add2(r0[q], cr0[q], __fmul2_rn(both<C>(g0.x), z));
+            kahan_add2(i0[q], ci0[q], __fmul2_rn(both<C>(g0.y), z));
+            kahan_add2(r1[q], cr1[q], __fmul2_rn(both<C>(g1.x), z));
+            kahan_add2(i1[q], ci1[q], __fmul2_rn(both<C>(g1.y), z));
+          } else {
+            r0[q] = fma2(both<C>(g0.x), z, r0[q]);
+            i0[q] = fma2(both<C>(g0.y), z, i0[q]);
+            r1[q] = fma2(both<C>(g1.x), z, r1[q]);
+            i1[q] = fma2(both<C>(g1.y), z, i1[q]);
+          }
+        }
+      }
+      __syncwarp();  // the next group overwrites this image and u
+    }
+  }
+  cp_async_wait<0>();
+}
+
+// Planes of a column that several units touch: the entry's partial slots are contiguous (s0 ..
+// s0 + ns - 1, in unit order).  The first `nlong` entries hold many slots (the dense columns
+// around k = 0: hundreds): a CTA's 8 warps sum a contiguous eighth each, then warp 0 adds the
+// eight sums in order.  The others take a warp each.  The order is fixed by the plan
+// (deterministic); a lane sums two cells, eight loads in flight at a time.
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_reduce_col3(const ColRed* __restrict__ red, int nred, int nlong, const cx_t<T>* __restrict__ partial,
+                  cx_t<T>* __restrict__ fine, int nfx, int nfy, int ncx) {
+  using C = cx_t<T>;
+  __shared__ C sh[7][64];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool team = (int)blockIdx.x < nlong;
+  const int e = team ? (int)blockIdx.x : nlong + ((int)blockIdx.x - nlong) * 8 + warp;
+  if (e >= nred) return;
+  const int4 r = __ldg(reinterpret_cast<const int4*>(red) + e);  // col, z, s0, ns
+  const int k0 = team ? r.w * warp / 8 : 0, k1 = team ? r.w * (warp + 1) / 8 : r.w;
+  C v0 = cmk<C>((T)0, (T)0), v1 = v0;  // cells 2 lane and 2 lane + 1 of the slot (row-major 8 x 8)
+  const C* src = partial + (size_t)r.z * (kColX * kColY) + 2 * lane;
+  auto load = [&](int k, C& p, C& q) {
+    const C* at = src + (size_t)k * (kColX * kColY);
+    if constexpr (sizeof(T) == 4) {
+      const float4 f = __ldcs(reinterpret_cast<const float4*>(at));
+      p = make_float2(f.x, f.y);
+      q = make_float2(f.z, f.w);
+    } else {
+      p = __ldcs(at);
+      q = __ldcs(at + 1);
+    }
+  };
+  int k = k0;
+  for (; k + 8 <= k1; k += 8) {
+    C p[8], q[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) load(k + i, p[i], q[i]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      v0 = cadd(v0, p[i]);
+      v1 = cadd(v1, q[i]);
+    }
+  }
+  for (; k < k1; ++k) {
+    C p, q;
+    load(k, p, q);
+    v0 = cadd(v0, p);
+    v1 = cadd(v1, q);
+  }
+  if (team) {
+    if (warp > 0) {
+      sh[warp - 1][2 * lane] = v0;
+      sh[warp - 1][2 * lane + 1] = v1;
+    }
+    __syncthreads();
+    if (warp > 0) return;
+#pragma unroll
+    for (int w = 0; w < 7; ++w) {
+      v0 = cadd(v0, sh[w][2 * lane]);
+      v1 = cadd(v1, sh[w][2 * lane + 1]);
+    }
+  }
+  const int cx = r.x % ncx, cy = r.x / ncx, c0 = 2 * lane;
+  C* dst = fine + (long long)r.y * nfx * nfy + (long long)(cy * kColY + c0 / 8) * nfx + cx * kColX + c0 % 8;
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(dst) = make_float4(v0.x, v0.y, v1.x, v1.y);
+  } else {
+    dst[0] = v0;
+    dst[1] = v1;
+  }
+}
+
+// ---- group images (plan time) -----------------------------------------------------------------
+// one warp per group; vis: (node or -1, (oy + 16) << 6 | (ox + 16)); runs: the head's entries;
+// counts: (visits, runs)
+template <typename T, int W>
+__global__ void __launch_bounds__(128)
+    k_col_image(const int2* __restrict__ vis, const int* __restrict__ runs, const int2* __restrict__ counts,
+                const T* __restrict__ psi, unsigned char* __restrict__ image, int* __restrict__ nodes, int ngroups) {
+  using I = ColImage<T, W>;
+  const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (g >= ngroups) return;
+  unsigned char* im = image + (size_t)g * I::BYTES;
+  for (int i = lane; i < I::BYTES / 16; i += 32) reinterpret_cast<int4*>(im)[i] = make_int4(0, 0, 0, 0);
+  __syncwarp();
+  const int2 v = vis[(size_t)g * 32 + lane];
+  nodes[(size_t)g * 32 + lane] = v.x;
+  if (v.x >= 0) {
+    const int ox = (v.y & 63) - 16, oy = ((v.y >> 6) & 63) - 16;
+    const T* ps = psi + (size_t)v.x * 3 * W;
+    for (int c = 0; c < 8; ++c) {
+      if ((unsigned)(c - ox) < (unsigned)W)
+        *reinterpret_cast<T*>(im + I::X + c / I::EPC * 512 + lane * 16 + c % I::EPC * (int)sizeof(T)) = ps[c - ox];
+      if ((unsigned)(c - oy) < (unsigned)W)
+        *reinterpret_cast<T*>(im + I::Y + c * I::RS + lane * (int)sizeof(T)) = ps[W + c - oy];
+    }
+  }
+  const int2 n = counts[g];
+  if (lane < n.y) {
+    const int hd = runs[(size_t)g * kColRuns + lane];
+    *reinterpret_cast<int*>(im + I::HEAD + 4 * lane) = hd;
+    const int node = vis[(size_t)g * 32 + (hd & 63)].x, rot = (hd >> 12) % W;
+    T* z = reinterpret_cast<T*>(im + I::Z + lane * I::ZS);
+    for (int k = 0; k < W; ++k) z[rot + k < W ? rot + k : rot + k - W] = psi[(size_t)node * 3 * W + 2 * W + k];
+  }
+  if (lane == 0) *reinterpret_cast<int2*>(im + I::COUNTS) = n;
+}
+
+enum class ColOp { ImageBytes, BuildImage, Configure, Spread };
+
+struct ColBuild {
+  const int2* vis;
+  const int* runs;
+  const int2* counts;
+};
+
+template <typename T, int W, bool COMP>
+int col_op(Plan& p, cudaStream_t s, ColOp op, const ColBuild* b, size_t* out) {
+  using I = ColImage<T, W>;
+  if (op == ColOp::ImageBytes) {
+    *out = I::BYTES;
+    return DDI_OK;
+  }
+  if (op == ColOp::BuildImage) {
+    if (p.ngroups == 0) return DDI_OK;
+    k_col_image<T, W><<<(unsigned)((p.ngroups + 3) / 4), 128, 0, s>>>(b->vis, b->runs, b->counts,
+                                                                      static_cast<const T*>(p.d_psi), p.d_cimage,
+                                                                      p.d_cnodes, p.ngroups);
+    DDI_LAUNCH_CHECK();
+    return DDI_OK;
+  }
+  auto kern = k_spread_col3<T, W, COMP>;
+  constexpr size_t smem = (size_t)SpreadSmem<T, W>::BYTES * (kColThreads3 / 32);
+  if (op == ColOp::Configure) {
+    {
+      // the limit belongs to the kernel, shared by every plan (and thread): only raise it
+      static std::mutex mu;
+      std::lock_guard<std::mutex> lock(mu);
+      cudaFuncAttributes fa;
+      DDI_CUDA(cudaFuncGetAttributes(&fa, kern));
+      if ((size_t)fa.maxDynamicSharedSizeBytes < smem)
+        DDI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    }
+    int per_sm = 0, sms = 0;
+    DDI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kColThreads3, smem));
+    DDI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device));
+    p.spread_smem = smem;
+    p.spread_blocks = std::max(1, std::min(per_sm * sms, (p.ncunits + kColThreads3 / 32 - 1) / (kColThreads3 / 32)));
+    return DDI_OK;
+  }
+  ColArgs3 a;
+  for (int d = 0; d < 3; ++d) a.nf[d] = p.nf[d];
+  a.ncx = p.nf[0] / kColX;
+  a.units = p.d_cunits;
+  a.nunits = p.ncunits;
+  a.counter = p.d_counter;
+  a.image = p.d_cimage;
+  a.nodes = p.d_cnodes;
+  a.c = p.d_c;
+  a.fine = p.d_fine;
+  a.partial = p.d_cpart;
+  a.dest = p.d_cslots;
+  DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, sizeof(int), s));
+  kern<<<p.spread_blocks, kColThreads3, p.spread_smem, s>>>(a);
+  DDI_LAUNCH_CHECK();
+  p.mark("spread", s);
+  if (p.ncred > 0) {
+    k_reduce_col3<T><<<(unsigned)(p.ncred_long + (p.ncred - p.ncred_long + 7) / 8), 256, 0, s>>>(
+        p.d_cred, p.ncred, p.ncred_long, static_cast<const cx_t<T>*>(p.d_cpart), static_cast<cx_t<T>*>(p.d_fine),
+        p.nf[0], p.nf[1], a.ncx);
+    DDI_LAUNCH_CHECK();
+    p.mark("spread_reduce", s);
+  }
+  return DDI_OK;
+}
+
+int col_dispatch(Plan& p, cudaStream_t s, ColOp op, const ColBuild* b, size_t* out) {
+  if (p.prec == DDI_FP32) {
+    switch (p.w) {
+      case 6: return p.col_comp ? col_op<float, 6, true>(p, s, op, b, out) : col_op<float, 6, false>(p, s, op, b, out);
+      case 8: return p.col_comp ? col_op<float, 8, true>(p, s, op, b, out) : col_op<float, 8, false>(p, s, op, b, out);
+    }
+  } else {
+    switch (p.w) {
+      case 10: return col_op<double, 10, false>(p, s, op, b, out);
+      case 12: return col_op<double, 12, false>(p, s, op, b, out);
+      case 14: return col_op<double, 14, false>(p, s, op, b, out);
+      case 16: return col_op<double, 16, false>(p, s, op, b, out);
+    }
+  }
+  set_error("column spread: kernel width %d not built", p.w);
+  return DDI_ERR_ARG;
+}
+
+}  // namespace
+
+size_t col_image_bytes(Plan& p) {
+  size_t n = 0;
+  return col_dispatch(p, nullptr, ColOp::ImageBytes, nullptr, &n) == DDI_OK ? n : 0;
+}
+int build_col_images(Plan& p, const int2* vis, const int* runs, const int2* counts, cudaStream_t s) {
+  const ColBuild b{vis, runs, counts};
+  return col_dispatch(p, s, ColOp::BuildImage, &b, nullptr);
+}
+int configure_spread_col3(Plan& p) { return col_dispatch(p, nullptr, ColOp::Configure, nullptr, nullptr); }
+int launch_spread_col3(Plan& p, cudaStream_t s) { return col_dispatch(p, s, ColOp::Spread, nullptr, nullptr); }
+
+}  // namespace ddi

@@ -95,16 +95,19 @@ struct SplitUnit {
   int tile, plane, slot0, nslots;
 };
 
-// ---- column spread work list (FP32 3D) -------------------------------------------------------
-// A column is a kColX x kColY block of fine cells in x-y with all its z-planes.  A work unit
-// takes a range of the column's visits, sorted by their first z tap, and a window of planes.
+// ---- column spread work list -------------------------------------------------------------------
+// A column is a kColX x kColY block of fine cells in x-y with all its z-planes (2D: kColX cells
+// in x with every y line).  A work unit takes a range of the column's visits, sorted by their
+// first tap along the window axis (z; 2D: y), and a window of planes.
 constexpr int kColX = 8, kColY = 8;
-struct ColUnit {
+constexpr int kColRuns = 8;     // 3D: most runs of one z class per group of 32 visits (columns.cuh)
+constexpr int kColPlanes = 32;  // 3D: most planes of a unit's window
+struct alignas(16) ColUnit {
   int col;       // column index cy * (nf_x / kColX) + cx
-  int lo, hi;    // visit range
+  int lo, hi;    // range of groups (3D) or visits (2D)
   int z0, z1;    // planes [z0, z1) the unit writes (plane z mod nf_z; z1 may exceed nf_z)
   int plo, phi;  // leading / trailing planes that other units also touch: go to partial slots
-  int slot0;     // its shared planes (leading, then trailing) are entries slot0 .. of the unit slot map
+  int slot0;     // 2D: its shared rows (leading, then trailing) are entries slot0 .. of the unit slot map
 };
 struct alignas(16) ColRed {  // a plane of a column touched by several units: the sum of their partial slots
   int col, z;
@@ -185,13 +188,17 @@ struct Plan {
   int* d_nonfinite = nullptr; // set by the pad pass when rho holds NaN / Inf (cleared by checks)
   // column spread (spread_kind == DDI_SPREAD_COLUMNS)
   int spread_kind = DDI_SPREAD_TILES;
-  int2* d_cvis = nullptr;     // visits (node, first z tap << 13 | z-class start << 12 | (oy + 16) << 6 | (ox + 16))
+  int2* d_cvis = nullptr;     // 2D visits (node, first y tap << 13 | run start << 12 | (oy + 16) << 6 | (ox + 16))
+  unsigned char* d_cimage = nullptr;  // 3D: the groups' images (columns.cuh)
+  int* d_cnodes = nullptr;    // 3D: [group][32] node of each visit, -1: none
+  int ngroups = 0;            // 3D: groups of visits
   ColUnit* d_cunits = nullptr;
   ColRed* d_cred = nullptr;
-  int* d_cslots = nullptr;    // per unit (from its slot0): the partial slot of each shared plane
-  
+  int* d_cslots = nullptr;    // 2D: per unit (from its slot0) the partial slot of each shared row; 3D: [unit][kColPlanes],
+                              // the partial slot of each plane of its window, -1 where it alone writes the plane
   void* d_cpart = nullptr;    // partial planes: [slot][kColY * kColX] complex
   int ncunits = 0, ncred = 0, ncslots = 0;
+  int ncred_long = 0;         // 3D: the first reduce entries, each summed by a whole CTA
   bool col_comp = false;      // column spread: compensated (Kahan) plane accumulation
   long long visits = 0;       // total visit-list entries
   long long pairs = 0;        // total (node, plane) pairs of all units
@@ -290,6 +297,12 @@ __host__ __device__ inline size_t spread_warp_bytes(size_t plane_bytes, size_t s
   return ((plane_bytes + 15) & ~(size_t)15) + ((stage_bytes + 15) & ~(size_t)15);
 }
 
+// 3D column spread (columns.cu): bytes of a group's image, the images from device lists, the
+// launch geometry, and the spread with its reduction
+size_t col_image_bytes(Plan& p);
+int build_col_images(Plan& p, const int2* vis, const int* runs, const int2* counts, cudaStream_t s);
+int configure_spread_col3(Plan& p);
+int launch_spread_col3(Plan& p, cudaStream_t s);
 int configure_kernels(Plan& p);  // per-plan launch geometry (nufft.cu)
 // reads and clears the plan's non-finite-input record after synchronising s:
 // DDI_ERR_NONFINITE if it was set (plan.cu)

@@ -99,7 +99,7 @@ void free_plan(Plan& p) {
                   p.d_partial,
                   p.d_visits, p.d_units, p.d_split, p.d_counter, p.d_psi1, p.d_rho, p.d_phi, p.d_work,
                   p.d_work2,  p.d_kin,   p.d_red,   p.d_io_in, p.d_io_out, p.d_cvis, p.d_cunits, p.d_cred,
-                  p.d_cslots, p.d_cpart, p.d_nonfinite};
+                  p.d_cslots, p.d_cpart, p.d_nonfinite, p.d_cimage, p.d_cnodes};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (int i = 0; i < 8; ++i)
@@ -256,19 +256,36 @@ int build_spread(Plan& p, cudaStream_t stream) {
   return configure_kernels(p);
 }
 
-// Whether the column spread applies: FP32 plans whose fine grid holds whole columns and is
-// wide enough that a footprint meets a column (or a window) in one contiguous piece.  2D
-// columns carry no compensated variant (compensated 2D plans use the tile spread).
+namespace {
+// the fine grid holds whole columns and is wide enough that a footprint meets a column (or a
+// window) in one contiguous piece
+bool columns_fit(const Plan& p) {
+  if (p.w > 16 || p.nf[0] % kColX != 0 || p.nf[0] < kColX + p.w - 1) return false;
+  if (p.dim == 2) return p.nf[1] >= p.w;
+  return p.nf[1] % kColY == 0 && p.nf[1] >= kColY + p.w - 1 && p.nf[2] >= p.w;
+}
+}  // namespace
+
+// Whether the column spread may be asked for: FP32 plans whose fine grid fits.  2D columns
+// carry no compensated variant (compensated 2D plans use the tile spread).
 bool columns_apply(const Plan& p) {
-  if (p.prec != DDI_FP32 || p.w > 16 || p.nf[0] % kColX != 0 || p.nf[0] < kColX + p.w - 1) return false;
-  if (p.dim == 2) return p.nf[1] >= p.w && p.desc.compensated == 0;
-  return p.dim == 3 && p.nf[1] % kColY == 0 && p.nf[1] >= kColY + p.w - 1 && p.nf[2] >= p.w;
+  return p.prec == DDI_FP32 && columns_fit(p) && (p.dim == 3 || p.desc.compensated == 0);
+}
+
+// Whether a plan spreads by columns on its own choice (desc.spread == DDI_SPREAD_AUTO).  FP32:
+// wherever they apply in 3D.  FP64, 3D, without a tile size of the caller's own: from 2048
+// processed nodes up, where there are enough units to fill the device.
+static bool columns_auto3(const Plan& p) {
+  if (p.dim != 3) return false;
+  if (p.prec == DDI_FP32) return columns_apply(p);
+  return columns_fit(p) && p.Mh >= 2048 && p.desc.tile[0] <= 0 && p.desc.tile[1] <= 0 && p.desc.tile[2] <= 0;
 }
 
 // Frees the spread lists of both schemes (the autotuner switches a 2D plan between them).
 void drop_spread_lists(Plan& p) {
   for (void** q : {(void**)&p.d_visits, (void**)&p.d_units, (void**)&p.d_split, &p.d_partial, (void**)&p.d_cvis,
-                   (void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart})
+                   (void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart, (void**)&p.d_cimage,
+                   (void**)&p.d_cnodes})
     if (*q) {
       cudaFree(*q);
       *q = nullptr;
@@ -288,6 +305,16 @@ void drop_spread_lists(Plan& p) {
 // boundaries, and the last unit of a column wraps onto the first) is a leading or trailing
 // plane of each of them: those go to partial slots and a reduce entry sums them in unit order;
 // every other plane is written by its one unit.  Every fine cell is written once per apply.
+// Visits per unit of a 3D column spread: the fewest units that still keep the device even.
+// Swept over 32 .. 1024 (spread + reduction, us): FP32 (2432 resident warps) 24^3 at 64,
+// 96x64x48 54 at 128 and 256 (60 at 512, 86 at 64), 128^3 101 at 512 (126 at 128), 192^3 277 at
+// 512 (384 at 128); FP64, bound by its arithmetic, 24^3 102 at 64, 64^3 511 at 512 (529 at 256),
+// 128^3 2590 at 512 (2815 at 256).
+static int default_col_chunk(int prec, long long visits) {
+  const long long c = visits / (prec == DDI_FP32 ? 3500 : 900) / 32 * 32;
+  return (int)std::min<long long>(512, std::max<long long>(64, c));
+}
+
 int build_spread_col(Plan& p, cudaStream_t stream) {
   const bool d3 = p.dim == 3;
   const int W = p.w, nfx = p.nf[0], nfy = p.nf[1];
@@ -295,7 +322,8 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
   const int cy_cells = d3 ? kColY : 1;
   const int ncx = nfx / kColX, ncy = d3 ? nfy / kColY : 1, ncol = ncx * ncy;
   DDI_CUDA(cudaStreamSynchronize(stream));
-  for (void** q : {(void**)&p.d_cvis, (void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart})
+  for (void** q : {(void**)&p.d_cvis, (void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart,
+                   (void**)&p.d_cimage, (void**)&p.d_cnodes})
     if (*q) {
       cudaFree(*q);
       *q = nullptr;
@@ -362,8 +390,43 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
       if (it == b || (it->y >> 13) != ((it - 1)->y >> 13) || p.h_zcls[it->x] != p.h_zcls[(it - 1)->x])
         it->y |= 1 << 12;
   }
-  const int cap = p.desc.chunk > 0 ? p.desc.chunk : 256;
-  const int lmax = std::min(64, nfz);
+  const int cap = p.desc.chunk > 0 ? p.desc.chunk : d3 ? default_col_chunk(p.prec, total) : 256;
+  const int lmax = std::min(d3 ? kColPlanes : 64, nfz);
+  // 3D: the column's visits in groups of at most 32 slots and kColRuns runs (columns.cuh).  A
+  // run takes an even number of slots, and is cut only where it is longer than a group or leaves
+  // half a group empty: its second part adds psi_z to the window once more
+  std::vector<int2> gvis;    // [group][32]: node (-1: none), packed x/y start
+  std::vector<int> gruns;    // [group][kColRuns]: first tap << 12 | end slot << 6 | first slot
+  std::vector<int2> gcount;  // slots, runs
+  std::vector<int> gbeg;     // first visit of each group
+  auto add_groups = [&](int b, int e) {
+    const int gcap = std::min(32, cap);
+    for (int pos = b; pos < e;) {
+      const size_t g = gcount.size();
+      gvis.resize((g + 1) * 32, make_int2(-1, 0));
+      gruns.resize((g + 1) * kColRuns, 0);
+      gbeg.push_back(pos);
+      int nv = 0, ns = 0, nr = 0;  // visits, slots, runs
+      while (pos < e && nr < kColRuns && nv < gcap && ns < 32) {
+        // the group's planes fit a unit's window
+        if (nr > 0 && (vis[pos].y >> 13) - (vis[gbeg[g]].y >> 13) + W > kColPlanes) break;
+        int L = 1;
+        while (pos + L < e && !((vis[pos + L].y >> 12) & 1)) ++L;
+        int take = L;
+        const int room = std::min(gcap - nv, 32 - ns);
+        if (L > room) {
+          if (L <= gcap && room < 16 && nr > 0) break;
+          take = room;
+        }
+        gruns[g * kColRuns + nr++] = ((vis[pos].y >> 13) << 12) | ((ns + take + (take & 1)) << 6) | ns;
+        for (int k = 0; k < take; ++k) gvis[g * 32 + ns + k] = make_int2(vis[pos + k].x, vis[pos + k].y & 4095);
+        nv += take;
+        ns += take + (take & 1);
+        pos += take;
+      }
+      gcount.push_back(make_int2(ns, nr));
+    }
+  };
   std::vector<ColUnit> units;
   std::vector<ColRed> red;
   std::vector<int> slots;  // per unit-local shared plane: its partial slot
@@ -389,14 +452,37 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
       }
       const bool needed = in_x && in_y;
       if (needed)
-        for (int z = 0; z < nfz; z += lmax) units.push_back(ColUnit{c, b0, b0, z, std::min(nfz, z + lmax), 0, 0, 0});
+        for (int z = 0; z < nfz; z += lmax) units.push_back(ColUnit{c, 0, 0, z, std::min(nfz, z + lmax), 0, 0, 0});
       continue;
     }
     // visit chunks and their planes [a, b) (b = last first tap + w)
     std::vector<std::array<int, 4>> ch;  // lo, hi, a, b
-    for (int k = b0; k < b1; k += cap) {
-      const int hi = std::min(b1, k + cap);
-      ch.push_back({{k, hi, vis[k].y >> 13, (vis[hi - 1].y >> 13) + W}});
+    if (d3) {
+      // whole groups: at most cap visits, a window of kColPlanes and the work of about cap visits.
+      // (kernel issue slots: 6 a visit, 33 a run, 40 a plane, 130 a group, on average 22 a visit; the
+      // sparse columns' few visits spread over all planes, and one unit for such a column ran
+      // for 90 us where the average took 13)
+      const int g0 = (int)gcount.size();
+      add_groups(b0, b1);
+      const int g1 = (int)gcount.size();
+      auto first = [&](int g) { return g < g1 ? gbeg[g] : b1; };
+      for (int k = g0; k < g1;) {
+        const int a = vis[gbeg[k]].y >> 13;
+        int hi = k;
+        long long work = 40 * W;
+        for (; hi < g1; ++hi) {
+          const int end = (vis[first(hi + 1) - 1].y >> 13) + W;
+          work += 130 + 6 * gcount[hi].x + 33 * gcount[hi].y + 40 * (end - std::max(a + W, (vis[gbeg[hi]].y >> 13) + W));
+          if (hi > k && (first(hi + 1) - gbeg[k] > cap || end - a > kColPlanes || work > 22LL * cap)) break;
+        }
+        ch.push_back({{k, hi, a, (vis[first(hi) - 1].y >> 13) + W}});
+        k = hi;
+      }
+    } else {
+      for (int k = b0; k < b1; k += cap) {
+        const int hi = std::min(b1, k + cap);
+        ch.push_back({{k, hi, vis[k].y >> 13, (vis[hi - 1].y >> 13) + W}});
+      }
     }
     const int nch = (int)ch.size();
     for (int k = 0; k < nch; ++k) {
@@ -404,7 +490,7 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
       const int next = k + 1 < nch ? ch[k + 1][2] : ch[0][2] + nfz;
       const int e = std::max(ch[k][3], std::min(next, a + lmax));
       units.push_back(ColUnit{c, ch[k][0], ch[k][1], a, e, 0, 0, 0});
-      for (int z = e; z < next; z += lmax) units.push_back(ColUnit{c, ch[k][1], ch[k][1], z, std::min(next, z + lmax), 0, 0, 0});
+      for (int z = e; z < next; z += lmax) units.push_back(ColUnit{c, 0, 0, z, std::min(next, z + lmax), 0, 0, 0});
     }
     // planes touched by several units
     std::fill(tc.begin(), tc.end(), 0);
@@ -439,7 +525,7 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
       contrib[z].clear();
     }
   }
-  // costliest units first.  3D: visits plus the planes each writes.  2D: the four lane
+  // costliest units first, those without visits last.  3D: the work above.  2D: the four lane
   // groups share a run (one first y tap), so a run of L visits takes ceil(L / 4) steps; a
   // unit costs about 4 per step, 3 per run and 5 per row it writes (relative instruction
   // counts of the kernel's visit step, run start and row flush)
@@ -448,7 +534,8 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
     for (size_t u = 0; u < units.size(); ++u) {
       const ColUnit& U = units[u];
       if (d3) {
-        cost[u] = (long long)(U.hi - U.lo) + (U.z1 - U.z0);
+        cost[u] = 40LL * (U.z1 - U.z0);
+        for (int k = U.lo; k < U.hi; ++k) cost[u] += 130 + 6 * gcount[k].x + 33 * gcount[k].y;
         continue;
       }
       long long steps = 0, runs = 0;
@@ -469,10 +556,27 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
     }
     std::vector<size_t> ord(units.size());
     std::iota(ord.begin(), ord.end(), (size_t)0);
-    std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b) { return cost[a] > cost[b]; });
+    std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b) {
+      const bool ea = units[a].lo == units[a].hi, eb = units[b].lo == units[b].hi;
+      return ea != eb ? eb : cost[a] > cost[b];
+    });
     std::vector<ColUnit> sorted(units.size());
     for (size_t k = 0; k < ord.size(); ++k) sorted[k] = units[ord[k]];
     units.swap(sorted);
+    if (d3) {  // the kernel's table: the slot of each plane of the window, -1 where the unit alone writes it
+      std::vector<int> dest(units.size() * kColPlanes, -1);
+      for (size_t u = 0; u < units.size(); ++u) {
+        const ColUnit& U = units[u];
+        const int len = U.z1 - U.z0;
+        if (len > kColPlanes) {
+          set_error("column spread: a unit's window has %d planes", len);
+          return DDI_ERR_INTERNAL;
+        }
+        for (int r = 0; r < U.plo; ++r) dest[u * kColPlanes + r] = slots[U.slot0 + r];
+        for (int r = 0; r < U.phi; ++r) dest[u * kColPlanes + len - U.phi + r] = slots[U.slot0 + U.plo + r];
+      }
+      slots.swap(dest);
+    }
   }
   if (units.size() > (size_t)INT32_MAX || slots.size() > (size_t)INT32_MAX) {
     set_error("column spread: work list too long");
@@ -483,8 +587,35 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
   p.chunk = cap;
   p.ncunits = (int)units.size();
   p.ncred = (int)red.size();
+  p.ncred_long = 0;
+  if (d3)  // entries of more than 24 slots first: a CTA sums each of them
+    p.ncred_long = (int)(std::stable_partition(red.begin(), red.end(), [](const ColRed& r) { return r.ns > 24; }) -
+                         red.begin());
   p.ncslots = nslot;
-  DDI_TRY(upload(p, (void**)&p.d_cvis, vis, "column visits", stream));
+  if (d3) {
+    p.ngroups = (int)gcount.size();
+    // the lists the images are made from are needed on the device only while they are made
+    int2 *dv = nullptr, *dc = nullptr;
+    int* dr = nullptr;
+    const size_t kept = p.bytes;
+    int st = upload(p, (void**)&dv, gvis, "column visits", stream);
+    if (st == DDI_OK) st = upload(p, (void**)&dr, gruns, "column runs", stream);
+    if (st == DDI_OK) st = upload(p, (void**)&dc, gcount, "column groups", stream);
+    p.bytes = kept;
+    if (st == DDI_OK) st = dev_alloc(p, (void**)&p.d_cimage, col_image_bytes(p) * gcount.size(), "column group images");
+    if (st == DDI_OK) st = dev_alloc(p, (void**)&p.d_cnodes, sizeof(int) * 32 * gcount.size(), "column group nodes");
+    if (st == DDI_OK) st = build_col_images(p, dv, dr, dc, stream);
+    if (st == DDI_OK && cudaStreamSynchronize(stream) != cudaSuccess) {
+      set_error("column group images: %s", cudaGetErrorString(cudaGetLastError()));
+      st = DDI_ERR_CUDA;
+    }
+    cudaFree(dv);
+    cudaFree(dr);
+    cudaFree(dc);
+    DDI_TRY(st);
+  } else {
+    DDI_TRY(upload(p, (void**)&p.d_cvis, vis, "column visits", stream));
+  }
   DDI_TRY(upload(p, (void**)&p.d_cunits, units, "column units", stream));
   DDI_TRY(upload(p, (void**)&p.d_cred, red, "column reduce entries", stream));
   DDI_TRY(upload(p, (void**)&p.d_cslots, slots, "column slot lists", stream));
@@ -538,15 +669,15 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
   // items' kernels, and the 96-density batch measured 13.3 ms with columns against 15.5 ms
   // with tiles (the faster tiles alone) and 15.2 ms with the size rule
   p.batch_item = batch_item;
-  p.spread_kind = columns_apply(p) && (d.spread == DDI_SPREAD_COLUMNS ||
-                                       (d.spread == DDI_SPREAD_AUTO &&
-                                        (p.dim == 3 || batch_item || (long long)p.nf[0] * p.nf[1] <= 512LL * 512)))
+  const bool columns2 = p.dim == 2 && columns_apply(p) && (batch_item || (long long)p.nf[0] * p.nf[1] <= 512LL * 512);
+  p.Mh = p.M / 2;  // one node of each (k, -k) pair
+  p.spread_kind = d.spread == DDI_SPREAD_COLUMNS || (d.spread == DDI_SPREAD_AUTO && (columns2 || columns_auto3(p)))
                       ? DDI_SPREAD_COLUMNS
                       : DDI_SPREAD_TILES;
   // compensated FP32 arithmetic: head + tail twiddles in the NUFFT's fine-grid passes and
   // compensated (Kahan) plane sums in the column spread
   p.precise_nufft = d.compensated != 0 && d.precision == DDI_FP32;
-  p.col_comp = d.compensated != 0;
+  p.col_comp = d.compensated != 0 && d.precision == DDI_FP32;
 
   // one node of each (k, -k) pair: the first half of the azimuth
   const int nphi = d.nphi, half = nphi / 2;

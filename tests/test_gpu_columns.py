@@ -1,0 +1,57 @@
+"""Column spread of 3D plans (both precisions, every built kernel width) against the tile spread
+of the same plan: the two sum the same taps in another order, so they agree to the path's own
+tolerance (1e-6 FP32, 1e-12 FP64).  Sizes where the lists can go wrong: the smallest fine grid
+that holds a column and a footprint (windows and footprints wrap), ragged grids, units of a
+few visits (most planes shared, groups of one run) and units of whole columns."""
+import math
+
+import numpy as np
+import pytest
+
+from paper_1504_02897_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+TOL = {0: 1e-12, 1: 1e-6}
+
+
+@pytest.fixture(scope="module")
+def D():
+    from paper_1504_02897_gb300 import build, ddi
+    build.build()
+    ddi.load()
+    return ddi
+
+
+CASES = [
+    # precision, nufft_tol, n, rule, chunk
+    (0, 0.0, (12, 12, 12), (16, 16, 16), 0),
+    (0, 0.0, (24, 12, 8), (17, 11, 26), 5),
+    (0, 1e-7, (12, 16, 12), (16, 16, 16), 40),      # w = 10
+    (0, 1e-9, (16, 12, 24), (16, 17, 16), 100000),  # w = 12
+    (0, 1e-14, (12, 12, 16), (16, 16, 18), 64),     # w = 16
+    (0, 0.0, (32, 24, 48), (33, 15, 50), 0),
+    (1, 0.0, (8, 8, 8), (9, 7, 10), 1),
+    (1, 1e-4, (8, 12, 16), (9, 7, 10), 33),         # w = 6
+    (1, 0.0, (48, 24, 32), (49, 23, 46), 0),
+]
+
+
+@pytest.mark.parametrize("prec,tol,n,rule,chunk", CASES)
+def test_columns_match_tiles(D, prec, tol, n, rule, chunk):
+    import torch
+    lo, ln = tuple(-0.25 * v for v in n), tuple(0.5 * v for v in n)
+    X, Y, Z = synth.coords(n, lo, ln)
+    rng = np.random.default_rng(5)
+    rho = np.exp(-0.3 * (X ** 2 + Y ** 2 + Z ** 2)) * (1 + 0.05 * rng.random(X.shape))
+    axis, m = (0.6, 0.0, 0.8), (0.0, math.sqrt(0.5), math.sqrt(0.5))
+    kw = dict(precision=prec, nufft_tol=tol, nr=rule[0], ntheta=rule[1], nphi=rule[2])
+    cols = D.Plan(3, n, lo, ln, axis, m, chunk=chunk, **kw)
+    tiles = D.Plan(3, n, lo, ln, axis, m, spread=1, **kw)
+    small = rule[0] * rule[1] * rule[2] // 2 < 2048
+    assert tiles.info.spread == 1 and cols.info.spread == (1 if prec == 0 and small else 2)
+    x = torch.from_numpy(rho).to("cuda", cols.real_dtype)
+    a, b = cols.apply(x), tiles.apply(x)
+    err = float((a - b).abs().max() / b.abs().max())
+    assert err <= TOL[prec], err
+    assert torch.equal(a, cols.apply(x))  # fixed summation order
