@@ -374,6 +374,182 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// ---- interpolation (type 2) ------------------------------------------------------------------------
+// The spread's transpose over the same groups.  A warp holds W planes of its column in registers
+// (lane (lx, ly): cells (lx, ly) and (lx, ly + 4); plane p in register p mod W), loading each plane
+// of the unit's window once.  Per run of one z class every lane sums H = sum_z psi_z F for its
+// two cells; the group's H blocks (one per run) go to shared memory, and then a lane per visit
+// sums sum_y psi_y sum_x psi_x H over the 8 x 8 cells of its run's block: no reduction across
+// lanes.  The visit's sum is its column's share of f_q; k_node_sum3 adds a node's shares in a
+// fixed order (deterministic) and applies 2 h^d W_q.
+//
+// What bounds it: FP64 operations (4 W per run and lane, 144 per visit, against 2 per tap and 8/7
+// idle lanes of a gather), in FP32 instruction issue; the gather kernel (k_interp) was bound by L1
+// wavefronts, 64-byte pieces of unrelated rows.
+struct InterpArgs3 {
+  int nf[3];
+  int ncx;
+  int xlo, nx, ylo, ny;  // fine x and y lines that hold transformed values (cyclic ranges)
+  const ColUnit* units;  // the units with visits come first
+  int nunits;
+  int* counter;
+  const unsigned char* image;
+  const void* fine;
+  void* share;           // [group][32] each visit's sum
+};
+
+template <typename T, int W>
+struct InterpSmem {
+  static constexpr int HS = kColX * kColY * 2 * (int)sizeof(T) + 16;  // bytes between the runs' H blocks
+  static constexpr int H = 2 * ColImage<T, W>::BYTES;
+  static constexpr int BYTES = (H + kColRuns * HS + 127) / 128 * 128;
+};
+
+template <typename T, int W>
+__global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_interp_col3(InterpArgs3 a) {
+  using C = cx_t<T>;
+  using I = ColImage<T, W>;
+  using S = InterpSmem<T, W>;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* sm = smem_raw + warp * S::BYTES;
+  unsigned char* sh = sm + S::H;
+  const int lx = lane & 7, ly = lane >> 3;
+  const int nfx = a.nf[0], nfy = a.nf[1], nfz = a.nf[2];
+  const long long plane = (long long)nfx * nfy;
+  const C zero = cmk<C>((T)0, (T)0);
+  auto inside = [](int l, int lo, int n, int nf) {
+    int d = l - lo;
+    if (d < 0) d += nf;
+    return d < n;
+  };
+  const int nwarps = gridDim.x * (blockDim.x >> 5);
+  for (int un = warp * gridDim.x + blockIdx.x; un < a.nunits;) {
+    const ColUnit U = a.units[un];
+    int nx = 0;
+    if (lane == 0) nx = atomicAdd(a.counter, 1);
+    int buf = 0;
+    copy_image<I::BYTES>(sm, a.image + (size_t)U.lo * I::BYTES, lane);
+    cp_async_commit();
+    const int x = (U.col % a.ncx) * kColX + lx, y = (U.col / a.ncx) * kColY + ly;
+    // cells off the transformed lines hold no value of this evaluation: they count as zero (no
+    // visit has a tap there)
+    const bool inx = inside(x, a.xlo, a.nx, nfx);
+    const bool ok0 = inx && inside(y, a.ylo, a.ny, nfy), ok1 = inx && inside(y + 4, a.ylo, a.ny, nfy);
+    const C* col = static_cast<const C*>(a.fine) + (long long)y * nfx + x;
+    auto load = [&](int z, C& v0, C& v1) {
+      const C* at = col + (z >= nfz ? z - nfz : z) * plane;
+      v0 = ok0 ? __ldg(at) : zero;
+      v1 = ok1 ? __ldg(at + 4 * nfx) : zero;
+    };
+    C r0[W / 2], i0[W / 2], r1[W / 2], i1[W / 2];  // planes 2 q and 2 q + 1 (mod W)
+    C p0 = zero, p1 = zero;                          // plane zl, requested ahead
+    int zl = U.z0 - W, zslot = 0;                    // planes zl - W .. zl - 1 are in the window
+    for (int gi = U.lo; gi < U.hi; ++gi) {
+      if (gi + 1 < U.hi)
+        copy_image<I::BYTES>(sm + (buf ^ 1) * I::BYTES, a.image + (size_t)(gi + 1) * I::BYTES, lane);
+      cp_async_commit();
+      cp_async_wait<1>();
+      __syncwarp();
+      const unsigned char* im = sm + buf * I::BYTES;
+      buf ^= 1;
+      const int nslots = *reinterpret_cast<const int*>(im + I::COUNTS);
+      const int nruns = *reinterpret_cast<const int*>(im + I::COUNTS + 4);
+      int myrun = 0;
+      for (int r = 0; r < nruns; ++r) {
+        const int hd = *reinterpret_cast<const int*>(im + I::HEAD + 4 * r);
+        const int j0 = hd & 63, sr = hd >> 12;
+        if (lane >= j0) myrun = r;
+        if (sr + W - zl > 3) {
+          // the unit's first run, or a gap: the whole window in one go (all loads in flight)
+          const int rot = sr % W;
+#pragma unroll
+          for (int k = 0; k < W; ++k) {
+            C v0, v1;
+            load(sr + (k >= rot ? k - rot : k - rot + W), v0, v1);
+            if (k % 2 == 0) {
+              r0[k / 2].x = v0.x, i0[k / 2].x = v0.y, r1[k / 2].x = v1.x, i1[k / 2].x = v1.y;
+            } else {
+              r0[k / 2].y = v0.x, i0[k / 2].y = v0.y, r1[k / 2].y = v1.x, i1[k / 2].y = v1.y;
+            }
+          }
+          zl = sr + W;
+          zslot = rot;
+          if (zl < U.z1) load(zl, p0, p1);
+        }
+        while (zl < sr + W) {
+          switch (zslot) {
+#define DDI_PUT3(R)                                                                  case R:                                                                              if constexpr (R < W) {                                                               constexpr int Q = R / 2;                                                           if constexpr (R % 2 == 0)                                                            r0[Q].x = p0.x, i0[Q].x = p0.y, r1[Q].x = p1.x, i1[Q].x = p1.y;                  else                                                                                 r0[Q].y = p0.x, i0[Q].y = p0.y, r1[Q].y = p1.x, i1[Q].y = p1.y;                }                                                                                  break;
+            DDI_COL3_CASES(DDI_PUT3)
+#undef DDI_PUT3
+          }
+          ++zl;
+          zslot = zslot + 1 == W ? 0 : zslot + 1;
+          if (zl < U.z1) load(zl, p0, p1);
+        }
+        C h0r = zero, h0i = zero, h1r = zero, h1i = zero;
+        const C* pz = reinterpret_cast<const C*>(im + I::Z + r * I::ZS);
+#pragma unroll
+        for (int q = 0; q < W / 2; ++q) {
+          const C z = pz[q];
+          h0r = dot2(z, r0[q], h0r);
+          h0i = dot2(z, i0[q], h0i);
+          h1r = dot2(z, r1[q], h1r);
+          h1i = dot2(z, i1[q], h1i);
+        }
+        C* h = reinterpret_cast<C*>(sh + r * S::HS) + lane;  // row-major 8 x 8 cells
+        h[0] = cmk<C>(dot_sum(h0r), dot_sum(h0i));
+        h[32] = cmk<C>(dot_sum(h1r), dot_sum(h1i));
+      }
+      __syncwarp();
+      // lane = visit
+      T wx[8];
+#pragma unroll
+      for (int ch = 0; ch < I::CH; ++ch)
+        *reinterpret_cast<int4*>(wx + ch * I::EPC) = *reinterpret_cast<const int4*>(im + I::X + ch * 512 + lane * 16);
+      const unsigned char* h = sh + myrun * S::HS;
+      C f = zero;
+#pragma unroll
+      for (int yy = 0; yy < 8; ++yy) {
+        const T wy = reinterpret_cast<const T*>(im + I::Y + yy * I::RS)[lane];
+        C t = zero;
+#pragma unroll
+        for (int xx = 0; xx < 8; xx += 16 / (int)sizeof(C)) {
+          C v[16 / sizeof(C)];
+          *reinterpret_cast<int4*>(v) = *reinterpret_cast<const int4*>(h + (yy * 8 + xx) * (int)sizeof(C));
+#pragma unroll
+          for (int k = 0; k < (int)(16 / sizeof(C)); ++k) t = fma2(both<C>(wx[xx + k]), v[k], t);
+        }
+        f = fma2(both<C>(wy), t, f);
+      }
+      if (lane < nslots) static_cast<C*>(a.share)[(size_t)gi * 32 + lane] = f;
+      __syncwarp();  // the next group overwrites this image and the H blocks
+    }
+    un = nwarps + __shfl_sync(0xffffffffu, nx, 0);
+  }
+  cp_async_wait<0>();
+}
+
+// c_q = 2 h^d W_q times the sum of the node's shares, in the order of its columns
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_node_sum3(const int* __restrict__ off, const int* __restrict__ pos, const cx_t<T>* __restrict__ share,
+                const T* __restrict__ scale, cx_t<T>* __restrict__ c, int count) {
+  using C = cx_t<T>;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count) return;
+  const int b = off[i], e = off[i + 1];
+  C sum = cmk<C>((T)0, (T)0);
+  for (int k = b; k < e; k += 4) {
+    C v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = k + q < e ? __ldcs(share + pos[k + q]) : cmk<C>((T)0, (T)0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sum = cadd(sum, v[q]);
+  }
+  c[i] = cscale(sum, scale[i]);
+}
+
 // ---- group images (plan time) -----------------------------------------------------------------
 // one warp per group; vis: (node or -1, (oy + 16) << 6 | (ox + 16)); runs: the head's entries;
 // counts: (visits, runs)
@@ -410,7 +586,19 @@ __global__ void __launch_bounds__(128)
   if (lane == 0) *reinterpret_cast<int2*>(im + I::COUNTS) = n;
 }
 
-enum class ColOp { ImageBytes, BuildImage, Configure, Spread };
+// raises a kernel's dynamic shared memory limit (it belongs to the kernel, shared by every plan
+// and thread: only raised)
+int raise_smem(const void* fn, size_t bytes) {
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
+  cudaFuncAttributes fa;
+  DDI_CUDA(cudaFuncGetAttributes(&fa, fn));
+  if ((size_t)fa.maxDynamicSharedSizeBytes < bytes)
+    DDI_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  return DDI_OK;
+}
+
+enum class ColOp { ImageBytes, BuildImage, Configure, Spread, Interp };
 
 struct ColBuild {
   const int2* vis;
@@ -434,22 +622,43 @@ int col_op(Plan& p, cudaStream_t s, ColOp op, const ColBuild* b, size_t* out) {
     return DDI_OK;
   }
   auto kern = k_spread_col3<T, W, COMP>;
+  auto interp = k_interp_col3<T, W>;
   constexpr size_t smem = (size_t)SpreadSmem<T, W>::BYTES * (kColThreads3 / 32);
+  constexpr size_t ismem = (size_t)InterpSmem<T, W>::BYTES * (kColThreads3 / 32);
+  constexpr int wpc = kColThreads3 / 32;
   if (op == ColOp::Configure) {
-    {
-      // the limit belongs to the kernel, shared by every plan (and thread): only raise it
-      static std::mutex mu;
-      std::lock_guard<std::mutex> lock(mu);
-      cudaFuncAttributes fa;
-      DDI_CUDA(cudaFuncGetAttributes(&fa, kern));
-      if ((size_t)fa.maxDynamicSharedSizeBytes < smem)
-        DDI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
-    int per_sm = 0, sms = 0;
+    DDI_TRY(raise_smem(reinterpret_cast<const void*>(kern), smem));
+    DDI_TRY(raise_smem(reinterpret_cast<const void*>(interp), ismem));
+    int per_sm = 0, iper_sm = 0, sms = 0;
     DDI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kColThreads3, smem));
+    DDI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&iper_sm, interp, kColThreads3, ismem));
     DDI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device));
     p.spread_smem = smem;
-    p.spread_blocks = std::max(1, std::min(per_sm * sms, (p.ncunits + kColThreads3 / 32 - 1) / (kColThreads3 / 32)));
+    p.spread_blocks = std::max(1, std::min(per_sm * sms, (p.ncunits + wpc - 1) / wpc));
+    p.interp_blocks = std::max(1, std::min(iper_sm * sms, (p.ncvunits + wpc - 1) / wpc));
+    return DDI_OK;
+  }
+  if (op == ColOp::Interp) {
+    if (p.Mh == 0) return DDI_OK;
+    InterpArgs3 a;
+    for (int d = 0; d < 3; ++d) a.nf[d] = p.nf[d];
+    a.ncx = p.nf[0] / kColX;
+    a.xlo = p.xr[0], a.nx = p.xr[1], a.ylo = p.yr[0], a.ny = p.yr[1];
+    a.units = p.d_cunits;
+    a.nunits = p.ncvunits;
+    a.counter = p.d_counter + 1;
+    a.image = p.d_cimage;
+    a.fine = p.d_fine;
+    a.share = p.d_cshare;
+    DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, 2 * sizeof(int), s));
+    interp<<<p.interp_blocks, kColThreads3, ismem, s>>>(a);
+    DDI_LAUNCH_CHECK();
+    p.mark("interp", s);
+    k_node_sum3<T><<<(unsigned)((p.Mh + 255) / 256), 256, 0, s>>>(
+        p.d_cnoff, p.d_cnpos, static_cast<const cx_t<T>*>(p.d_cshare), static_cast<const T*>(p.d_scale),
+        static_cast<cx_t<T>*>(p.d_c), (int)p.Mh);
+    DDI_LAUNCH_CHECK();
+    p.mark("node_sum", s);
     return DDI_OK;
   }
   ColArgs3 a;
@@ -507,6 +716,7 @@ int build_col_images(Plan& p, const int2* vis, const int* runs, const int2* coun
   return col_dispatch(p, s, ColOp::BuildImage, &b, nullptr);
 }
 int configure_spread_col3(Plan& p) { return col_dispatch(p, nullptr, ColOp::Configure, nullptr, nullptr); }
+int launch_interp_col3(Plan& p, cudaStream_t s) { return col_dispatch(p, s, ColOp::Interp, nullptr, nullptr); }
 int launch_spread_col3(Plan& p, cudaStream_t s) { return col_dispatch(p, s, ColOp::Spread, nullptr, nullptr); }
 
 }  // namespace ddi

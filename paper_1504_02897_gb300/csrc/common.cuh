@@ -184,7 +184,7 @@ struct Plan {
   int4* d_visits = nullptr;   // spread visit lists: (node, ox, oy, oz) relative to the tile
   SpreadUnit* d_units = nullptr;
   SplitUnit* d_split = nullptr;
-  int* d_counter = nullptr;   // unit counter of the persistent spread
+  int* d_counter = nullptr;   // unit counters of the persistent spread and of the column interpolation
   int* d_nonfinite = nullptr; // set by the pad pass when rho holds NaN / Inf (cleared by checks)
   // column spread (spread_kind == DDI_SPREAD_COLUMNS)
   int spread_kind = DDI_SPREAD_TILES;
@@ -192,6 +192,12 @@ struct Plan {
   unsigned char* d_cimage = nullptr;  // 3D: the groups' images (columns.cuh)
   int* d_cnodes = nullptr;    // 3D: [group][32] node of each visit, -1: none
   int ngroups = 0;            // 3D: groups of visits
+  void* d_cshare = nullptr;   // 3D: [group][32] each visit's share of its node's value (interpolation)
+  int* d_cnoff = nullptr;     // 3D: [Mh + 1] ranges of d_cnpos
+  int* d_cnpos = nullptr;     // 3D: where a node's shares are in d_cshare
+  int ncvunits = 0;           // 3D: units with visits (they come first)
+  int interp_blocks = 1;
+  bool col_interp = false;    // 3D: interpolate by columns too
   ColUnit* d_cunits = nullptr;
   ColRed* d_cred = nullptr;
   int* d_cslots = nullptr;    // 2D: per unit (from its slot0) the partial slot of each shared row; 3D: [unit][kColPlanes],
@@ -303,6 +309,7 @@ size_t col_image_bytes(Plan& p);
 int build_col_images(Plan& p, const int2* vis, const int* runs, const int2* counts, cudaStream_t s);
 int configure_spread_col3(Plan& p);
 int launch_spread_col3(Plan& p, cudaStream_t s);
+int launch_interp_col3(Plan& p, cudaStream_t s);  // fine grid -> d_c
 int configure_kernels(Plan& p);  // per-plan launch geometry (nufft.cu)
 // reads and clears the plan's non-finite-input record after synchronising s:
 // DDI_ERR_NONFINITE if it was set (plan.cu)

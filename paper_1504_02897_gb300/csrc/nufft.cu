@@ -17,6 +17,8 @@
 //
 // Launches (fft_nufft.cu holds the FFT passes):
 //   forward FFT x (pad + deconvolution fused), y, z, pruned to the padded block
+//   3D plans that spread by columns interpolate by columns too (columns.cu) where that is faster;
+//   the others:
 //   k_interp    8 (w <= 8) or 16 lanes per node: f_q = sum over the w^d taps of psi F,
 //               each footprint row read as one contiguous segment; writes
 //               c_q = 2 h^d W_q f_q
@@ -781,6 +783,7 @@ int time_spread(Plan& p, cudaStream_t s, int reps, float* ms) {
 template <typename T>
 int run_type2(Plan& p, const T* rho, cudaStream_t s) {
   DDI_TRY(nufft_forward_fft<T>(p, rho, s));
+  if (p.col_interp) return launch_interp_col3(p, s);
   DDI_TRY((p.dim == 3 ? launch_interp_w<T, 3>(p, s) : launch_interp_w<T, 2>(p, s)));
   p.mark("interp", s);
   return DDI_OK;

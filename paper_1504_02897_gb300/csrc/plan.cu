@@ -99,7 +99,8 @@ void free_plan(Plan& p) {
                   p.d_partial,
                   p.d_visits, p.d_units, p.d_split, p.d_counter, p.d_psi1, p.d_rho, p.d_phi, p.d_work,
                   p.d_work2,  p.d_kin,   p.d_red,   p.d_io_in, p.d_io_out, p.d_cvis, p.d_cunits, p.d_cred,
-                  p.d_cslots, p.d_cpart, p.d_nonfinite, p.d_cimage, p.d_cnodes};
+                  p.d_cslots, p.d_cpart, p.d_nonfinite, p.d_cimage, p.d_cnodes, p.d_cshare,
+                  p.d_cnoff, p.d_cnpos};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (int i = 0; i < 8; ++i)
@@ -283,9 +284,10 @@ static bool columns_auto3(const Plan& p) {
 
 // Frees the spread lists of both schemes (the autotuner switches a 2D plan between them).
 void drop_spread_lists(Plan& p) {
+  p.col_interp = false;
   for (void** q : {(void**)&p.d_visits, (void**)&p.d_units, (void**)&p.d_split, &p.d_partial, (void**)&p.d_cvis,
                    (void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart, (void**)&p.d_cimage,
-                   (void**)&p.d_cnodes})
+                   (void**)&p.d_cnodes, &p.d_cshare, (void**)&p.d_cnoff, (void**)&p.d_cnpos})
     if (*q) {
       cudaFree(*q);
       *q = nullptr;
@@ -308,10 +310,11 @@ void drop_spread_lists(Plan& p) {
 // Visits per unit of a 3D column spread: the fewest units that still keep the device even.
 // Swept over 32 .. 1024 (spread + reduction, us): FP32 (2432 resident warps) 24^3 at 64,
 // 96x64x48 54 at 128 and 256 (60 at 512, 86 at 64), 128^3 101 at 512 (126 at 128), 192^3 277 at
-// 512 (384 at 128); FP64, bound by its arithmetic, 24^3 102 at 64, 64^3 511 at 512 (529 at 256),
-// 128^3 2590 at 512 (2815 at 256).
+// 512 (384 at 128); FP64, bound by its arithmetic, with the interpolation (which prefers small
+// units: 64^3 367 at 128, 523 at 512) 24^3 at 64, 64^3 950 at 256 (1036 at 512), 128^3 5150 at 512
+// (5340 at 256).
 static int default_col_chunk(int prec, long long visits) {
-  const long long c = visits / (prec == DDI_FP32 ? 3500 : 900) / 32 * 32;
+  const long long c = visits / (prec == DDI_FP32 ? 3500 : 1700) / 32 * 32;
   return (int)std::min<long long>(512, std::max<long long>(64, c));
 }
 
@@ -323,7 +326,7 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
   const int ncx = nfx / kColX, ncy = d3 ? nfy / kColY : 1, ncol = ncx * ncy;
   DDI_CUDA(cudaStreamSynchronize(stream));
   for (void** q : {(void**)&p.d_cvis, (void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart,
-                   (void**)&p.d_cimage, (void**)&p.d_cnodes})
+                   (void**)&p.d_cimage, (void**)&p.d_cnodes, &p.d_cshare, (void**)&p.d_cnoff, (void**)&p.d_cnpos})
     if (*q) {
       cudaFree(*q);
       *q = nullptr;
@@ -592,8 +595,34 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
     p.ncred_long = (int)(std::stable_partition(red.begin(), red.end(), [](const ColRed& r) { return r.ns > 24; }) -
                          red.begin());
   p.ncslots = nslot;
+  p.ncvunits = 0;
+  for (const ColUnit& U : units) p.ncvunits += U.lo < U.hi ? 1 : 0;
   if (d3) {
     p.ngroups = (int)gcount.size();
+    if (gvis.size() > (size_t)INT32_MAX) {
+      set_error("column spread: work list too long");
+      return DDI_ERR_ARG;
+    }
+    // FP64: the gather kernel costs twice the FP64 operations (64^3: 748 us against 400, 128^3 5.9 ms
+    // against 2.5).  FP32: below 2^18 processed nodes its one launch is the shorter (24^3 10 us
+    // against 17, 96x64x48 with 221184 nodes 55 against 54, 128^3 with 524288 133 against 112)
+    p.col_interp = p.prec == DDI_FP64 || p.Mh >= (1 << 18);
+    // where each node's visits are: their interpolation shares are summed in this order
+    if (p.col_interp) {
+      std::vector<int> noff((size_t)p.Mh + 1, 0), npos((size_t)total);
+      for (const int2& v : gvis)
+        if (v.x >= 0) ++noff[(size_t)v.x + 1];
+      for (size_t i = 0; i < (size_t)p.Mh; ++i) noff[i + 1] += noff[i];
+      {
+        std::vector<int> fill(noff.begin(), noff.end() - 1);
+        for (size_t q = 0; q < gvis.size(); ++q)
+          if (gvis[q].x >= 0) npos[fill[gvis[q].x]++] = (int)q;
+      }
+      DDI_TRY(upload(p, (void**)&p.d_cnoff, noff, "node share ranges", stream));
+      DDI_TRY(upload(p, (void**)&p.d_cnpos, npos, "node shares", stream));
+      DDI_TRY(dev_alloc(p, &p.d_cshare, p.cx_size() * gvis.size(), "visit shares"));
+      DDI_CUDA(cudaStreamSynchronize(stream));  // noff and npos die with this block
+    }
     // the lists the images are made from are needed on the device only while they are made
     int2 *dv = nullptr, *dc = nullptr;
     int* dr = nullptr;
@@ -829,7 +858,7 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
     DDI_TRY(upload(p, &p.d_ones, ones, "unit factors", stream));
     DDI_TRY(upload(p, &p.d_ones_x2, ones2, "unit factor pairs", stream));
   }
-  DDI_TRY(dev_alloc(p, (void**)&p.d_counter, sizeof(int), "unit counter"));
+  DDI_TRY(dev_alloc(p, (void**)&p.d_counter, 2 * sizeof(int), "unit counters"));
   DDI_TRY(dev_alloc(p, (void**)&p.d_nonfinite, sizeof(int), "non-finite record"));
   DDI_CUDA(cudaMemsetAsync(p.d_nonfinite, 0, sizeof(int), stream));
   DDI_TRY(dev_alloc(p, &p.d_c, cs * p.Mh, "node values"));

@@ -1,4 +1,4 @@
-"""Column spread of 3D plans (both precisions, every built kernel width) against the tile spread
+"""Column spread and interpolation of 3D plans (both precisions, every built kernel width) against the tile spread
 of the same plan: the two sum the same taps in another order, so they agree to the path's own
 tolerance (1e-6 FP32, 1e-12 FP64).  Sizes where the lists can go wrong: the smallest fine grid
 that holds a column and a footprint (windows and footprints wrap), ragged grids, units of a
@@ -34,6 +34,8 @@ CASES = [
     (1, 0.0, (8, 8, 8), (9, 7, 10), 1),
     (1, 1e-4, (8, 12, 16), (9, 7, 10), 33),         # w = 6
     (1, 0.0, (48, 24, 32), (49, 23, 46), 0),
+    (1, 0.0, (24, 16, 12), (128, 64, 64), 0),       # 2^18 processed nodes: FP32 interpolates by columns too
+    (1, 1e-4, (8, 12, 16), (64, 128, 64), 200),
 ]
 
 
