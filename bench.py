@@ -257,6 +257,14 @@ def kernel_bytes(name, info, real=4):
     ball = int(4.0 / 3.0 * math.pi * (radius + w / 2.0) ** 3 * min(1.0, yfrac + w / nf)) * cx
     psi = mh * 3 * w * real + mh * 8        # kernel values and first taps
     table = {
+        # the passes in their order (y first): read rho, write the tap lines' first N cells, ...
+        "pad_fft_y": n3 * real + 2 * n3 * cx * yfrac,
+        "fft_x_fwd": (2 * n3 * cx + 4 * n3 * cx) * yfrac,
+        "fft_x_inv": (4 * n3 * cx + 2 * n3 * cx) * yfrac,
+        "fft_y_inv_crop": 2 * n3 * cx * yfrac + n3 * real,
+        "fft_y_inv_crop_add": 2 * n3 * cx * yfrac + 2 * n3 * real,
+        "node_sum": 2 * mh * cx + mh * real,                 # at least one share per node, scale in, c_q out
+        # the same passes transforming x first
         "pad_fft_x": n3 * real + 2 * n3 * cx,                # read rho, write N^2 rows of 2N
         "fft_y_fwd": 2 * n3 * cx + 4 * n3 * cx * yfrac,      # read the block half, write the tap lines
         "fft_z_fwd": (4 * n3 * cx + 8 * n3 * cx) * yfrac,    # the columns on the tap lines
@@ -268,8 +276,13 @@ def kernel_bytes(name, info, real=4):
         "fft_x_inv_crop": 2 * n3 * cx + n3 * real,
         "fft_x_inv_crop_add": 2 * n3 * cx + 2 * n3 * real,  # also reads phi (split plans)
     }
-    # the split algorithm's smooth part: the same passes without the deconvolution, every line
-    smooth = {"smooth_pad_fft_x": n3 * real + 2 * n3 * cx, "smooth_fft_y_fwd": 6 * n3 * cx,
+    # the split algorithm's smooth part: the same passes without the deconvolution, on the half
+    # spectrum (y lines 0 .. N), its z passes in one; or x first on every line
+    hfrac = (N + 1) / nf
+    smooth = {"smooth_pad_fft_y": n3 * real + 2 * n3 * cx * hfrac, "smooth_fft_x_fwd": 6 * n3 * cx * hfrac,
+              "smooth_fft_z_pair": 8 * n3 * cx * hfrac, "smooth_fft_x_inv": 6 * n3 * cx * hfrac,
+              "smooth_fft_y_inv_crop": 2 * n3 * cx * hfrac + n3 * real,
+              "smooth_pad_fft_x": n3 * real + 2 * n3 * cx, "smooth_fft_y_fwd": 6 * n3 * cx,
               "smooth_fft_z_symbol": 12 * n3 * cx, "smooth_fft_z_inv": 12 * n3 * cx, "smooth_fft_y_inv": 6 * n3 * cx,
               "smooth_fft_x_inv_crop": 2 * n3 * cx + n3 * real}
     return table.get(name, smooth.get(name, 0))
@@ -971,13 +984,13 @@ def bench_gpe(args):
 
 def _kernel_hash():
     """Hash of the sources that determine the spread kernel's DRAM traffic: the kernel
-    (nufft.cu), its work lists and node tables (plan.cu, tables.cpp/.h) and their shared
-    definitions (common.cuh); the tile is checked separately.  A recorded ncu traffic
+    (columns.cu/.cuh, nufft.cu), its work lists and node tables (plan.cu, tables.cpp/.h) and
+    their shared definitions (common.cuh); the tile is checked separately.  A recorded ncu traffic
     figure is only used while these are unchanged."""
     import hashlib
     h = hashlib.sha1()
     d = os.path.join(ROOT, "paper_1504_02897_gb300", "csrc")
-    for f in ("common.cuh", "nufft.cu", "plan.cu", "tables.cpp", "tables.h"):
+    for f in ("columns.cu", "columns.cuh", "common.cuh", "nufft.cu", "plan.cu", "tables.cpp", "tables.h"):
         h.update(f.encode())
         with open(os.path.join(d, f), "rb") as fh:
             h.update(fh.read())

@@ -17,7 +17,8 @@ LIBDIR = os.path.join(HERE, "lib")
 LIB = os.path.join(LIBDIR, "libddi_gb300.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-CU_SOURCES = ["fft.cu", "fft_nufft.cu", "nufft.cu", "columns.cu", "plan.cu", "gpe.cu", "batch.cu", "noalloc.cu"]
+CU_SOURCES = ["fft_nufft_f64.cu", "fft_nufft_f32.cu", "gpe_fft_f64.cu", "gpe_fft_f32.cu", "columns.cu", "nufft.cu", "gpe.cu",
+              "plan.cu", "batch.cu", "noalloc.cu", "fft.cu"]
 CPP_SOURCES = ["tables.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -176,9 +176,10 @@ struct Plan {
   NodeDir* d_dirw = nullptr;  // [Mh]: direction and weight without the symbol (ddi_plan_set_axes)
   void* d_c = nullptr;        // cx [Mh]: node values c_q
   void* d_deconv = nullptr;   // double [n0 + n1 + n2]: 1/psihat per axis, index j (0..n-1)
-  void* d_deconv_x2 = nullptr;  // float2 [n0]: the x factors as FP32 head + tail (FP32 plans)
+  void* d_deconv_x2 = nullptr;  // float2 [n1]: the y factors as FP32 head + tail (FP32 plans)
   void* d_ones = nullptr;     // double [n0 + n1 + n2] of ones: the pad and crop of a split plan's smooth part
-  void* d_ones_x2 = nullptr;  // float2 [n0] of (1, 0)
+  void* d_em1 = nullptr;      // T [nf0 + nf1 + nf2], split plans: e^{-k_d^2/k0^2} - 1 at the fine grid's modes
+  void* d_ones_x2 = nullptr;  // float2 [n1] of (1, 0)
   void* d_fine = nullptr;     // cx [nf0 nf1 nf2]
   void* d_partial = nullptr;  // cx [nslots * tile cells]
   int4* d_visits = nullptr;   // spread visit lists: (node, ox, oy, oz) relative to the tile
@@ -231,7 +232,7 @@ struct Plan {
   void* d_phi = nullptr;      // T [N]
   void* d_work = nullptr;     // cx [N]
   void* d_work2 = nullptr;    // cx [N]
-  void* d_kin = nullptr;      // cx [n0 + n1 + n2]: per-axis kinetic phase factors
+  void* d_kin = nullptr;      // cx [2][n0 + n1 + n2]: per-axis kinetic phase factors for two times
   double* d_red = nullptr;    // reduction partials
   double* h_red = nullptr;    // pinned host copy of reduction results
   void* d_io_in = nullptr;    // staging for ddi_apply_host
@@ -268,16 +269,33 @@ inline const void* twiddles(const Plan& p, int n) {
   return nullptr;
 }
 
-// ---- FFT (fft.cu) ------------------------------------------------------------------
-// In-place batched 1-D FFTs along one axis of a [nz][ny][nx] complex array, unnormalised,
-// dir = -1: e^{-2 pi i jk/n}, dir = +1: e^{+2 pi i jk/n}.  axis 0 = x, 1 = y, 2 = z.
-template <typename T>
-int fft_axis(const Plan& p, cx_t<T>* data, int nx, int ny, int nz, int axis, int dir, cudaStream_t s);
-template <typename T>
-int fft_3d(const Plan& p, cx_t<T>* data, int nx, int ny, int nz, int dir, cudaStream_t s);
+// ---- FFT twiddle tables (fft.cu) -----------------------------------------------------------
 int make_twiddles(Plan& p, int n);
 
-// ---- pruned / fused fine-grid FFTs of the NUFFT (fft_nufft.cu) ----------------------
+// ---- the GPE's Fourier passes on the plan's grid (gpe_fft.cuh) ---------------------------------
+// transforms are unnormalised, dir = -1: e^{-2 pi i jk/n}
+template <typename T> int gpe_forward(Plan& p, cx_t<T>* a, cudaStream_t s);  // a <- F a
+// a <- F^{-1} e^{i f |mu|^2} F a for the per-axis tables tab of e^{i f mu_d^2} - 1 (x, y, z); rho,
+// if not null, <- |a|^2
+template <typename T> int gpe_kinetic(Plan& p, cx_t<T>* a, const cx_t<T>* tab, T* rho, cudaStream_t s);
+// one sweep of the gradient flow's fixed point,
+//   out <- F^{-1}[F(phi/dt + (alpha - W) cur) / (1/dt + alpha + |mu|^2/2)], W = V + beta rho + lambda Phi,
+// and *change <- max |out - cur|^2 (FP64 bits, cleared by the caller); skipped when prev is not
+// null and the FP64 number at *prev is <= tol2
+template <typename T>
+struct GfSweep {
+  const cx_t<T>*phi, *cur;
+  cx_t<T>* out;
+  const T *V, *rho, *dip;  // dip may be null
+  T beta, lam, alpha, inv_dt;
+  double inv_dt_alpha, ks[3];
+  const unsigned long long* prev;
+  double tol2;
+  unsigned long long* change;
+};
+template <typename T> int gpe_gf_sweep(Plan& p, const GfSweep<T>& w, cudaStream_t s);
+
+// ---- pruned / fused fine-grid FFTs of the NUFFT (fft_nufft.cuh) ----------------------
 template <typename T> int nufft_forward_fft(Plan& p, const T* rho, cudaStream_t s);  // rho -> F (fine grid)
 // U (fine grid) -> phi; acc: phi += the result instead of phi = the result
 template <typename T> int nufft_inverse_fft(Plan& p, T* phi, cudaStream_t s, bool acc = false);

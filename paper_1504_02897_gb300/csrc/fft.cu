@@ -1,28 +1,10 @@
-// Plain batched 1-D FFTs along one axis of a [nz][ny][nx] complex grid (GPE grid and
-// tests) and the FP64-built twiddle tables.  The Stockham core is in fft_core.cuh.
+// The FP64-built twiddle tables of the Stockham FFTs (fft_core.cuh).
+#include <cmath>
 #include <cstring>
 
-#include "fft_core.cuh"
+#include "common.cuh"
 
 namespace ddi {
-namespace {
-using namespace fftcore;
-
-template <typename T>
-struct PlainLines {
-  using C = cx_t<T>;
-  C* data;
-  LineGeom g;
-  using Ref = long long;  // offset of the line's first element
-  static constexpr bool kPreciseTwiddles = true;  // the GPE's repeated transforms
-  __host__ __device__ long long nlines() const { return g.nlines; }
-  __device__ bool contig() const { return g.se == 1; }
-  __device__ Ref ref(long long L) const { return line_off(g, L); }
-  __device__ C load(Ref r, int i) const { return __ldg(data + r + (long long)i * g.se); }
-  __device__ void store(Ref r, int i, C v) const { data[r + (long long)i * g.se] = v; }
-};
-
-}  // namespace
 
 int make_twiddles(Plan& p, int n) {
   if (twiddles(p, n)) return DDI_OK;
@@ -65,54 +47,5 @@ int make_twiddles(Plan& p, int n) {
   p.tw_n[b] = n;
   return DDI_OK;
 }
-
-template <typename T>
-int fft_axis(const Plan& p, cx_t<T>* data, int nx, int ny, int nz, int axis, int dir, cudaStream_t s) {
-  LineGeom g{};
-  int n = 1;
-  if (axis == 0) {
-    n = nx;
-    g.nlines = (long long)ny * nz;
-    g.l1 = ny;
-    g.s_hi = (long long)nx * ny;
-    g.s_lo = nx;
-    g.se = 1;
-  } else if (axis == 1) {
-    n = ny;
-    g.nlines = (long long)nx * nz;
-    g.l1 = nx;
-    g.s_hi = (long long)nx * ny;
-    g.s_lo = 1;
-    g.se = nx;
-  } else {
-    n = nz;
-    g.nlines = (long long)nx * ny;
-    g.l1 = nx;
-    g.s_hi = nx;
-    g.s_lo = 1;
-    g.se = (long long)nx * ny;
-  }
-  if (n == 1) return DDI_OK;
-  const void* tw = twiddles(p, n);
-  if (!tw) {
-    set_error("missing twiddle table for FFT length %d", n);
-    return DDI_ERR_ARG;
-  }
-  PlainLines<T> pol{data, g};
-  return dir < 0 ? dispatch_policy<T, -1>(n, pol, tw, s) : dispatch_policy<T, +1>(n, pol, tw, s);
-}
-
-template <typename T>
-int fft_3d(const Plan& p, cx_t<T>* data, int nx, int ny, int nz, int dir, cudaStream_t s) {
-  DDI_TRY(fft_axis<T>(p, data, nx, ny, nz, 0, dir, s));
-  DDI_TRY(fft_axis<T>(p, data, nx, ny, nz, 1, dir, s));
-  DDI_TRY(fft_axis<T>(p, data, nx, ny, nz, 2, dir, s));
-  return DDI_OK;
-}
-
-template int fft_axis<float>(const Plan&, float2*, int, int, int, int, int, cudaStream_t);
-template int fft_axis<double>(const Plan&, double2*, int, int, int, int, int, cudaStream_t);
-template int fft_3d<float>(const Plan&, float2*, int, int, int, int, cudaStream_t);
-template int fft_3d<double>(const Plan&, double2*, int, int, int, int, cudaStream_t);
 
 }  // namespace ddi

@@ -219,21 +219,62 @@ __device__ __forceinline__ long long line_off(const LineGeom& g, long long L) {
   return (L / g.l1) * g.s_hi + (L % g.l1) * g.s_lo;
 }
 
-// Generic batched-line FFT: a policy P supplies nlines(), contig() (element index fastest
-// in memory), ref(L) (the line's addresses, computed once per line by one thread),
-// load(ref, i) / store(ref, i, v) for element i of the line and kPreciseTwiddles.
+// Generic batched-line FFT: a policy P supplies nlines(), ref(L) (the line's addresses,
+// computed once per line by one thread), load(ref, i) /
+// store(ref, i, v, acc) for element i of the line, skip() (the whole pass is not needed), an
+// accumulator Acc with finish(acc), and the constants
+//   kStrided   the lines' elements are strided in memory and neighbouring lines adjacent (else the
+//              element index is fastest)
+//   kPrecise   apply the twiddle tails (FP32)
+//   kBlockIn   only the elements i < N/4 and i >= 3 N/4 are nonzero and loaded (the zero padding
+//              of a twofold oversampled line): the first stage's other inputs are literal zeros,
+//              so their loads and most of their butterfly drop out at compile time
+//   kBlockOut  only those elements are stored (the crop)
 // The first Stockham stage takes its inputs straight from global memory and the last one
 // writes its outputs straight back (both are in natural element order there), so each
 // element crosses shared memory once per middle stage plus once between the first stage
 // and the next.  Threads are (line b, butterfly t) pairs: lines fastest when lines are
 // strided in memory (a warp's accesses then cover adjacent lines), butterflies fastest
 // when lines are contiguous.
+struct PolicyBase {
+  struct Acc {};
+  static constexpr bool kPrecise = false, kBlockIn = false, kBlockOut = false, kStrided = true;
+  __device__ bool skip() const { return false; }
+  __device__ void finish(const Acc&) const {}
+};
+
+__host__ __device__ constexpr bool outside_block(int r, int R) { return r >= R / 4 && r < R - R / 4; }
+
+// first stage: butterfly t's inputs are elements t + r N/R0 (all loads issued before use)
+template <int N, int R0, typename C, typename P, typename Ref>
+__device__ __forceinline__ void load_first(const P& pol, const Ref& ref, bool live, int t, C (&v)[R0]) {
+  static_assert(!P::kBlockIn || R0 % 4 == 0, "the block is whole quarters of the first stage");
+#pragma unroll
+  for (int r = 0; r < R0; ++r) {
+    if (P::kBlockIn && outside_block(r, R0))
+      v[r] = cmk<C>(0, 0);
+    else
+      v[r] = live ? pol.load(ref, t + r * (N / R0)) : cmk<C>(0, 0);
+  }
+}
+// last stage: butterfly j's outputs are elements j + r NSL
+template <int N, int RL, int NSL, typename C, typename P, typename Ref>
+__device__ __forceinline__ void store_last(const P& pol, const Ref& ref, int j, const C (&v)[RL], typename P::Acc& acc) {
+#pragma unroll
+  for (int r = 0; r < RL; ++r) {
+    if (P::kBlockOut && RL % 4 == 0 && outside_block(r, RL)) continue;
+    const int i = j + r * NSL;
+    if (P::kBlockOut && RL % 4 != 0 && i >= N / 4 && i < N - N / 4) continue;
+    pol.store(ref, i, v[r], acc);
+  }
+}
+
 template <typename T, int N, int LPB, int DIR, typename P>
 __global__ void __launch_bounds__(LPB * Shape<N>::TPL)
     k_fft_policy(P pol, const cx_t<T>* __restrict__ tw) {
   using C = cx_t<T>;
   using Ref = typename P::Ref;
-  constexpr bool PR = P::kPreciseTwiddles;
+  constexpr bool PR = P::kPrecise;
   constexpr int LS = Shape<N>::LS;
   constexpr int TPL = Shape<N>::TPL;
   constexpr int RM = Shape<N>::RM;
@@ -244,59 +285,149 @@ __global__ void __launch_bounds__(LPB * Shape<N>::TPL)
   constexpr int GL = (RM + RL - 1) / RL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Ref refs[LPB];
+  if (pol.skip()) return;
   C* sm = reinterpret_cast<C*>(smem_raw);
   const long long L0 = (long long)blockIdx.x * LPB;
   const long long left = pol.nlines() - L0;
   const int nb = left < LPB ? (int)left : LPB;  // lines of this CTA
   if ((int)threadIdx.x < nb) refs[threadIdx.x] = pol.ref(L0 + threadIdx.x);
   __syncthreads();
-  const bool contig = pol.contig();
+  constexpr bool contig = !P::kStrided;
   const int b = contig ? (int)threadIdx.x / TPL : (int)threadIdx.x % LPB;
   const int t = contig ? (int)threadIdx.x % TPL : (int)threadIdx.x / LPB;
   const bool live = b < nb;
   C* line = sm + b * LS;
-  // first stage: butterfly t takes elements t + r N/R0 (all loads issued before use)
+  typename P::Acc acc{};
   C v0[R0];
-#pragma unroll
-  for (int r = 0; r < R0; ++r) v0[r] = live ? pol.load(refs[b], t + r * (N / R0)) : cmk<C>((T)0, (T)0);
+  load_first<N, R0>(pol, refs[b], live, t, v0);
   Dft<R0, DIR, C>::run(v0);
   if constexpr (R0 == N) {
-    // a single stage: outputs in natural order
-#pragma unroll
-    for (int r = 0; r < R0; ++r)
-      if (live) pol.store(refs[b], r, v0[r]);
+    if (live) store_last<N, N, 1>(pol, refs[b], 0, v0, acc);
   } else {
 #pragma unroll
     for (int r = 0; r < R0; ++r) line[pidx(t * R0 + r)] = v0[r];
     __syncthreads();
     MidStages<C, N, DIR, R0, NSL, PR>::run(line, t, tw);
-    // last stage: butterfly j's outputs are elements j + r NSL
     C v[GL][RL];
     stage_compute<C, N, RL, NSL, DIR, PR>(line, t, tw, v);
 #pragma unroll
     for (int g = 0; g < GL; ++g) {
       const int j = t + g * TPL;
-      if (live && (RM % RL == 0 || j < N / RL)) {
-#pragma unroll
-        for (int r = 0; r < RL; ++r) pol.store(refs[b], j + r * NSL, v[g][r]);
-      }
+      if (live && (RM % RL == 0 || j < N / RL)) store_last<N, RL, NSL>(pol, refs[b], j, v[g], acc);
     }
   }
+  pol.finish(acc);
 }
 
-template <typename T, int N>
+// Forward transform, pol.apply(ref, i, v) on every mode, inverse transform of the same line in one
+// pass: the line crosses global memory once each way instead of twice.  Where the last stage has
+// the first stage's radix (N = 16^k), a thread's modes are the inverse's first inputs and stay in
+// registers; otherwise they cross shared memory once.
+template <typename T, int N, int LPB, typename P>
+__global__ void __launch_bounds__(LPB * Shape<N>::TPL)
+    k_fft_pair(P pol, const cx_t<T>* __restrict__ tw) {
+  using C = cx_t<T>;
+  using Ref = typename P::Ref;
+  constexpr bool PR = P::kPrecise;
+  constexpr int LS = Shape<N>::LS;
+  constexpr int TPL = Shape<N>::TPL;
+  constexpr int RM = Shape<N>::RM;
+  constexpr int R0 = radix_for(N, 1);
+  constexpr int NSL = last_ns(N);
+  constexpr int RL = N / NSL;
+  constexpr int GL = (RM + RL - 1) / RL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ Ref refs[LPB];
+  if (pol.skip()) return;
+  C* sm = reinterpret_cast<C*>(smem_raw);
+  const long long L0 = (long long)blockIdx.x * LPB;
+  const long long left = pol.nlines() - L0;
+  const int nb = left < LPB ? (int)left : LPB;
+  if ((int)threadIdx.x < nb) refs[threadIdx.x] = pol.ref(L0 + threadIdx.x);
+  __syncthreads();
+  constexpr bool contig = !P::kStrided;
+  const int b = contig ? (int)threadIdx.x / TPL : (int)threadIdx.x % LPB;
+  const int t = contig ? (int)threadIdx.x % TPL : (int)threadIdx.x / LPB;
+  const bool live = b < nb;
+  C* line = sm + b * LS;
+  typename P::Acc acc{};
+  C v0[R0];
+  load_first<N, R0>(pol, refs[b], live, t, v0);
+  Dft<R0, -1, C>::run(v0);
+  if constexpr (R0 == N) {
+    if (live) {
+#pragma unroll
+      for (int r = 0; r < R0; ++r) v0[r] = pol.apply(refs[b], r, v0[r]);
+    }
+    Dft<R0, 1, C>::run(v0);
+    if (live) store_last<N, N, 1>(pol, refs[b], 0, v0, acc);
+  } else {
+#pragma unroll
+    for (int r = 0; r < R0; ++r) line[pidx(t * R0 + r)] = v0[r];
+    __syncthreads();
+    MidStages<C, N, -1, R0, NSL, PR>::run(line, t, tw);
+    {
+      C v[GL][RL];
+      stage_compute<C, N, RL, NSL, -1, PR>(line, t, tw, v);
+      __syncthreads();  // every input of the stage has been read
+#pragma unroll
+      for (int g = 0; g < GL; ++g) {
+        const int j = t + g * TPL;
+        if (RM % RL == 0 || j < N / RL) {
+#pragma unroll
+          for (int r = 0; r < RL; ++r) {
+            const C m = live ? pol.apply(refs[b], j + r * NSL, v[g][r]) : v[g][r];
+            if constexpr (RL == R0)
+              v0[r] = m;
+            else
+              line[pidx(j + r * NSL)] = m;
+          }
+        }
+      }
+      if constexpr (RL != R0) {
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < R0; ++r) v0[r] = line[pidx(t + r * (N / R0))];
+        __syncthreads();
+      }
+    }
+    Dft<R0, 1, C>::run(v0);
+#pragma unroll
+    for (int r = 0; r < R0; ++r) line[pidx(t * R0 + r)] = v0[r];
+    __syncthreads();
+    MidStages<C, N, 1, R0, NSL, PR>::run(line, t, tw);
+    C v[GL][RL];
+    stage_compute<C, N, RL, NSL, 1, PR>(line, t, tw, v);
+#pragma unroll
+    for (int g = 0; g < GL; ++g) {
+      const int j = t + g * TPL;
+      if (live && (RM % RL == 0 || j < N / RL)) store_last<N, RL, NSL>(pol, refs[b], j, v[g], acc);
+    }
+  }
+  pol.finish(acc);
+}
+
+// Lines per CTA.  Strided lines: a power of two, so that the lines of a CTA are whole 128-byte
+// pieces of memory at every element (10 lines of N = 384 made 80-byte pieces: 192^3 z passes 103
+// -> 76 us; 8 of N = 512 64-byte ones: the 256^3 split's z pass 571 -> 530 us).  Contiguous
+// lines: ~35 KB of shared memory per CTA in FP32.  FP64 takes half the lines.
+template <typename T, int N, bool STRIDED>
 constexpr int lines_per_cta() {
-  // ~35 KB of shared memory per CTA in FP32, the same line count halved in FP64
-  return sizeof(T) == 8 ? (lines_per_cta_base<N>() > 1 ? lines_per_cta_base<N>() / 2 : 1)
-                        : lines_per_cta_base<N>();
+  constexpr int f32 = !STRIDED ? lines_per_cta_base<N>() : N <= 64 ? 32 : N <= 512 ? 16 : N <= 1024 ? 8 : 4;
+  return sizeof(T) == 8 ? (f32 > 1 ? f32 / 2 : 1) : f32;
 }
 
+// DIR = 0: forward and inverse in one pass (k_fft_pair)
 template <typename T, int N, int DIR, typename P>
 int launch_policy(const P& pol, const void* tw, cudaStream_t s) {
-  constexpr int LPB = lines_per_cta<T, N>();
+  constexpr int LPB = lines_per_cta<T, N, P::kStrided>();
   constexpr int threads = LPB * Shape<N>::TPL;
   const size_t smem = (size_t)LPB * Shape<N>::LS * sizeof(cx_t<T>);
-  auto kern = k_fft_policy<T, N, LPB, DIR, P>;
+  void (*kern)(P, const cx_t<T>*);
+  if constexpr (DIR == 0)
+    kern = k_fft_pair<T, N, LPB, P>;
+  else
+    kern = k_fft_policy<T, N, LPB, DIR, P>;
   if (smem > 48 * 1024) {
     DDI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   }
@@ -307,31 +438,22 @@ int launch_policy(const P& pol, const void* tw, cudaStream_t s) {
   return DDI_OK;
 }
 
-// FFT lengths built: 2^a (8..2048) and 3 * 2^a (12..1536)
-template <typename T, int DIR, typename P>
+// FFT lengths built, 2^a and 3 * 2^a: LO and HI bound the lengths a policy is built for (fine-grid
+// lines 16..2048, 3D 1024; grid lines 8..1024)
+template <typename T, int DIR, int LO, int HI, typename P>
 int dispatch_policy(int n, const P& pol, const void* tw, cudaStream_t s) {
+#define DDI_LEN(NN)                                                        \
+  case NN:                                                                 \
+    if constexpr (NN >= LO && NN <= HI) return launch_policy<T, NN, DIR>(pol, tw, s); \
+    break;
   switch (n) {
-    case 8: return launch_policy<T, 8, DIR>(pol, tw, s);
-    case 12: return launch_policy<T, 12, DIR>(pol, tw, s);
-    case 16: return launch_policy<T, 16, DIR>(pol, tw, s);
-    case 24: return launch_policy<T, 24, DIR>(pol, tw, s);
-    case 32: return launch_policy<T, 32, DIR>(pol, tw, s);
-    case 48: return launch_policy<T, 48, DIR>(pol, tw, s);
-    case 64: return launch_policy<T, 64, DIR>(pol, tw, s);
-    case 96: return launch_policy<T, 96, DIR>(pol, tw, s);
-    case 128: return launch_policy<T, 128, DIR>(pol, tw, s);
-    case 192: return launch_policy<T, 192, DIR>(pol, tw, s);
-    case 256: return launch_policy<T, 256, DIR>(pol, tw, s);
-    case 384: return launch_policy<T, 384, DIR>(pol, tw, s);
-    case 512: return launch_policy<T, 512, DIR>(pol, tw, s);
-    case 768: return launch_policy<T, 768, DIR>(pol, tw, s);
-    case 1024: return launch_policy<T, 1024, DIR>(pol, tw, s);
-    case 1536: return launch_policy<T, 1536, DIR>(pol, tw, s);
-    case 2048: return launch_policy<T, 2048, DIR>(pol, tw, s);
-    default:
-      set_error("FFT length %d not supported (2^a or 3 * 2^a, 8..2048)", n);
-      return DDI_ERR_ARG;
+    DDI_LEN(8) DDI_LEN(12) DDI_LEN(16) DDI_LEN(24) DDI_LEN(32) DDI_LEN(48) DDI_LEN(64) DDI_LEN(96) DDI_LEN(128)
+    DDI_LEN(192) DDI_LEN(256) DDI_LEN(384) DDI_LEN(512) DDI_LEN(768) DDI_LEN(1024) DDI_LEN(1536) DDI_LEN(2048)
+    default: break;
   }
+#undef DDI_LEN
+  set_error("FFT length %d not supported (2^a or 3 * 2^a, %d..%d here)", n, LO, HI);
+  return DDI_ERR_ARG;
 }
 
 }  // namespace fftcore

@@ -3,8 +3,8 @@
 // Euler (Sec. 3.1, Eqs. gf-eq2..gffg33) and the adjoint of one TSFP step.
 //
 // Grids are the plan's n[0] x n[1] x n[2] periodic box; Fourier modes are
-// mu_p = 2 pi p / len, p = -n/2..n/2-1 (stored in FFT order).  The FFTs of fft.cu are
-// unnormalised, so every Fourier-space multiplier below carries the 1/N_tot factor.
+// mu_p = 2 pi p / len, p = -n/2..n/2-1 (stored in FFT order).  The transforms and their
+// multipliers are in gpe_fft.cuh.
 // Reductions accumulate in FP64 per thread, per block (fixed order), then one block
 // sums the block partials in a fixed order: results are deterministic.
 #include <algorithm>
@@ -65,11 +65,13 @@ __device__ __forceinline__ cx_t<T> expm1_i(T a) {
   return cmk<cx_t<T>>((T)-2 * s * s, (T)2 * s * c);
 }
 
-// per-axis factors e^{i f mu_d^2} - 1 (FP64 built, rounded once) for separable kinetic phases
+// per-axis factors e^{i f mu_d^2} - 1 (FP64 built, rounded once) for separable kinetic phases, for
+// f = f0 and f = f1
 template <typename T>
-__global__ void k_phase_tables(cx_t<T>* tab, G3 g, double f) {
+__global__ void k_phase_tables(cx_t<T>* tab, G3 g, double f0, double f1) {
   const int total = g.n[0] + g.n[1] + g.n[2];
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 2 * total; k += gridDim.x * blockDim.x) {
+    const int i = k < total ? k : k - total;
     int d = 0, l = i;
     while (l >= g.n[d]) {
       l -= g.n[d];
@@ -77,42 +79,8 @@ __global__ void k_phase_tables(cx_t<T>* tab, G3 g, double f) {
     }
     const double mu = g.n[d] == 1 ? 0.0 : mode_mu(l, g.n[d], g.ks[d]);
     double s, c;
-    sincos(0.5 * f * mu * mu, &s, &c);
-    tab[i] = cmk<cx_t<T>>((T)(-2.0 * s * s), (T)(2.0 * s * c));
-  }
-}
-
-// v * k for a constant known in FP64: head + tail in FP32 (a rounded 1/N would scale the
-// state by the same wrong factor every step)
-template <typename T>
-__device__ __forceinline__ T scale_const(T v, double k) {
-  if constexpr (sizeof(T) == 4) {
-    const float hi = (float)k;
-    return fmaf(v, hi, v * (float)(k - (double)hi));
-  } else {
-    return v * (T)k;
-  }
-}
-
-// psihat <- psihat * e^{i f |mu|^2} / N_tot using the per-axis tables of e - 1:
-// (1+A)(1+B)(1+C) - 1 = P + C + C P with P = A + B + A B
-template <typename T>
-__global__ void k_kinetic(cx_t<T>* __restrict__ a, const cx_t<T>* __restrict__ tab, G3 g, double inv_n) {
-  using C = cx_t<T>;
-  const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-  const C* tx = tab;
-  const C* ty = tab + g.n[0];
-  const C* tz = ty + g.n[1];
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    idx3(i, g, x, y, z);
-    const C A = tx[x], B = ty[y], Cz = tz[z];
-    const C P = cadd(cadd(A, B), cmul(A, B));
-    const C E = cadd(cadd(P, Cz), cmul(Cz, P));
-    const C v = a[i];
-    const C r = cadd(v, cmul(v, E));
-    a[i] = cmk<C>(scale_const(r.x, inv_n), scale_const(r.y, inv_n));
+    sincos(0.5 * (k < total ? f0 : f1) * mu * mu, &s, &c);
+    tab[k] = cmk<cx_t<T>>((T)(-2.0 * s * s), (T)(2.0 * s * c));
   }
 }
 
@@ -210,14 +178,14 @@ __global__ void k_nonlinear_general(cx_t<T>* __restrict__ psi, const T* __restri
   }
 }
 
-// psi <- psi exp(-i dt (V + beta rho + lambda Phi)), rho = |psi|^2 (Case I of Eq. tssp2)
+// psi <- psi exp(-i dt (V + beta |psi|^2 + lambda Phi)) (Case I of Eq. tssp2)
 template <typename T>
-__global__ void k_nonlinear(cx_t<T>* __restrict__ psi, const T* __restrict__ V, const T* __restrict__ rho,
-                            const T* __restrict__ phi, T beta, T lam, T dt, long long total) {
+__global__ void k_nonlinear(cx_t<T>* __restrict__ psi, const T* __restrict__ V, const T* __restrict__ phi, T beta,
+                            T lam, T dt, long long total) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    const T th = V[i] + beta * rho[i] + lam * phi[i];
     const cx_t<T> v = psi[i];
+    const T th = V[i] + beta * (v.x * v.x + v.y * v.y) + lam * phi[i];
     psi[i] = cadd(v, cmul(v, expm1_i(-dt * th)));
   }
 }
@@ -352,48 +320,12 @@ __global__ void __launch_bounds__(256) k_red_final(const double* part, int block
   if (t < k) out[t] = sh[t][0];
 }
 
-// GF: rhs = phi/dt + (alpha - W) cur, W = V + beta rho + lambda Phi
+// b <- s a (b may be a)
 template <typename T>
-__global__ void k_gf_rhs(const cx_t<T>* __restrict__ phi, const cx_t<T>* __restrict__ cur,
-                         const T* __restrict__ V, const T* __restrict__ rho, const T* __restrict__ dip,
-                         cx_t<T>* __restrict__ out, T beta, T lam, T alpha, T inv_dt, long long total) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const T w = V[i] + beta * rho[i] + (dip ? lam * dip[i] : (T)0);
-    const T f = alpha - w;
-    const cx_t<T> a = phi[i], c = cur[i];
-    out[i] = cmk<cx_t<T>>(a.x * inv_dt + f * c.x, a.y * inv_dt + f * c.y);
-  }
-}
-
-// GF: divide by (1/dt + alpha + |mu|^2/2) and by N_tot
-template <typename T>
-__global__ void k_gf_solve(cx_t<T>* __restrict__ a, G3 g, double inv_dt_alpha, double inv_n) {
-  // in the working precision: the fixed point's own tolerance is the plan's (1e-7 in FP32)
-  const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-  const T ks[3] = {(T)g.ks[0], (T)g.ks[1], (T)g.ks[2]};
-  const T c0 = (T)inv_dt_alpha, sc = (T)inv_n;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    int q[3];
-    idx3(i, g, q[0], q[1], q[2]);
-    T m2 = 0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int pp = q[d] < g.n[d] / 2 ? q[d] : q[d] - g.n[d];
-      const T m = (T)pp * ks[d];
-      m2 += g.n[d] > 1 ? m * m : (T)0;
-    }
-    const T f = sc / (c0 + (T)0.5 * m2);
-    a[i] = cscale(a[i], f);
-  }
-}
-
-template <typename T>
-__global__ void k_scale(cx_t<T>* __restrict__ a, T s, long long total) {
+__global__ void k_scale(const cx_t<T>* a, cx_t<T>* b, T s, long long total) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x)
-    a[i] = cscale(a[i], s);
+    b[i] = cscale(a[i], s);
 }
 
 // adjoint, part A: given psi1, rho = |psi1|^2, Phi, g2 (in cot):
@@ -459,6 +391,9 @@ __global__ void k_observable(const cx_t<T>* __restrict__ psi, cx_t<T>* __restric
   block_sum<1>(v, part + (size_t)blockIdx.x * kRedMax);
 }
 
+constexpr int kSweeps = 200;     // most sweeps of the gradient flow's fixed point per step
+constexpr int kSweepBatch = 48;  // most of them launched between two looks at their changes (h_red)
+
 template <typename T>
 struct Gpe {
   using C = cx_t<T>;
@@ -469,17 +404,17 @@ struct Gpe {
 
   Gpe(Plan& pl, cudaStream_t st) : p(pl), s(st), N(pl.grid_points()), g(g3_of(pl)) {}
 
-  int fft(C* a, int dir) { return fft_3d<T>(p, a, p.n[0], p.n[1], p.n[2], dir, s); }
+  // the two tables of kinetic() for e^{i f0 |mu|^2} and e^{i f1 |mu|^2}
+  int phase_tables(double f0, double f1) {
+    k_phase_tables<T><<<8, kThreads, 0, s>>>(static_cast<C*>(p.d_kin), g, f0, f1);
+    DDI_LAUNCH_CHECK();
+    return DDI_OK;
+  }
 
-  // a <- F^{-1} e^{i f |mu|^2} F a
-  int kinetic(C* a, double f) {
-    DDI_TRY(fft(a, -1));
-    C* tab = static_cast<C*>(p.d_kin);
-    k_phase_tables<T><<<4, kThreads, 0, s>>>(tab, g, f);
-    DDI_LAUNCH_CHECK();
-    k_kinetic<T><<<blocks_for(N), kThreads, 0, s>>>(a, tab, g, 1.0 / (double)N);
-    DDI_LAUNCH_CHECK();
-    return fft(a, +1);
+  // a <- F^{-1} e^{i f_k |mu|^2} F a; rho, if not null, <- |a|^2
+  int kinetic(C* a, int k, T* rho = nullptr) {
+    const C* tab = static_cast<const C*>(p.d_kin) + (size_t)k * (p.n[0] + p.n[1] + p.n[2]);
+    return gpe_kinetic<T>(p, a, tab, rho, s);
   }
 
   int abs2(const C* a, T* out) {
@@ -512,7 +447,7 @@ struct Gpe {
     DDI_TRY(reduce(4, 0, sums));
     C* w = static_cast<C*>(p.d_work2);
     DDI_CUDA(cudaMemcpyAsync(w, psi, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
-    DDI_TRY(fft(w, -1));
+    DDI_TRY(gpe_forward<T>(p, w, s));
     k_red_kinetic<T><<<p.red_blocks, kThreads, 0, s>>>(w, g, p.d_red);
     DDI_LAUNCH_CHECK();
     double kin;
@@ -533,7 +468,8 @@ struct Gpe {
     return DDI_OK;
   }
 
-  int normalise(C* a, double* mass_out) {
+  // out <- a / ||a|| (out may be a)
+  int normalise(const C* a, C* out, double* mass_out) {
     k_red_energy<T><<<p.red_blocks, kThreads, 0, s>>>(a, static_cast<const T*>(p.d_rho), nullptr, N, p.d_red);
     DDI_LAUNCH_CHECK();
     double sums[4];
@@ -543,7 +479,7 @@ struct Gpe {
       set_error("state has zero or non-finite mass");
       return DDI_ERR_NONFINITE;
     }
-    k_scale<T><<<blocks_for(N), kThreads, 0, s>>>(a, (T)(1.0 / std::sqrt(m)), N);
+    k_scale<T><<<blocks_for(N), kThreads, 0, s>>>(a, out, (T)(1.0 / std::sqrt(m)), N);
     DDI_LAUNCH_CHECK();
     if (mass_out) *mass_out = m;
     return DDI_OK;
@@ -563,17 +499,18 @@ struct Gpe {
     T* rho = static_cast<T*>(p.d_rho);
     T* phi = static_cast<T*>(p.d_phi);
     // consecutive half kinetic steps merge into one full step between nonlinear steps
-    DDI_TRY(kinetic(psi, -0.25 * dt));
+    DDI_TRY(phase_tables(-0.25 * dt, -0.5 * dt));
+    DDI_TRY(kinetic(psi, 0, rho));
     for (int k = 0; k < nsteps; ++k) {
-      DDI_TRY(abs2(psi, rho));
       if (lam != 0.0) {
         DDI_TRY(run_ddi<T>(p, rho, phi, s));
       } else {
         DDI_CUDA(cudaMemsetAsync(phi, 0, sizeof(T) * N, s));
       }
-      k_nonlinear<T><<<blocks_for(N), kThreads, 0, s>>>(psi, V, rho, phi, (T)beta, (T)lam, (T)dt, N);
+      k_nonlinear<T><<<blocks_for(N), kThreads, 0, s>>>(psi, V, phi, (T)beta, (T)lam, (T)dt, N);
       DDI_LAUNCH_CHECK();
-      DDI_TRY(kinetic(psi, k + 1 < nsteps ? -0.5 * dt : -0.25 * dt));
+      const bool more = k + 1 < nsteps;
+      DDI_TRY(kinetic(psi, more ? 1 : 0, more ? rho : nullptr));
     }
     return DDI_OK;
   }
@@ -582,7 +519,8 @@ struct Gpe {
   int step_general(C* psi, const T* V, double beta, double lam, const NonlinParams& nl, double dt, int nsteps) {
     T* g = static_cast<T*>(p.d_rho);
     T* phi = static_cast<T*>(p.d_phi);
-    DDI_TRY(kinetic(psi, -0.25 * dt));
+    DDI_TRY(phase_tables(-0.25 * dt, -0.5 * dt));
+    DDI_TRY(kinetic(psi, 0));
     for (int k = 0; k < nsteps; ++k) {
       k_step_density<T><<<blocks_for(N), kThreads, 0, s>>>(psi, g, nl, (T)dt, N);
       DDI_LAUNCH_CHECK();
@@ -593,7 +531,7 @@ struct Gpe {
       }
       k_nonlinear_general<T><<<blocks_for(N), kThreads, 0, s>>>(psi, V, phi, (T)beta, (T)lam, (T)dt, nl, N);
       DDI_LAUNCH_CHECK();
-      DDI_TRY(kinetic(psi, k + 1 < nsteps ? -0.5 * dt : -0.25 * dt));
+      DDI_TRY(kinetic(psi, k + 1 < nsteps ? 1 : 0));
     }
     return DDI_OK;
   }
@@ -661,35 +599,34 @@ struct Gpe {
     T* rho = static_cast<T*>(p.d_rho);
     T* phi = static_cast<T*>(p.d_phi);
     DDI_CUDA(cudaMemcpyAsync(psi1, psi_in, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
-    DDI_TRY(kinetic(psi1, -0.25 * dt));
-    DDI_TRY(abs2(psi1, rho));
+    DDI_TRY(phase_tables(-0.25 * dt, +0.25 * dt));
+    DDI_TRY(kinetic(psi1, 0, rho));
     if (lam != 0.0) {
       DDI_TRY(run_ddi<T>(p, rho, phi, s));
     } else {
       DDI_CUDA(cudaMemsetAsync(phi, 0, sizeof(T) * N, s));
     }
-    DDI_TRY(kinetic(cot, +0.25 * dt));
+    DDI_TRY(kinetic(cot, 1));
     k_adj_a<T><<<blocks_for(N), kThreads, 0, s>>>(psi1, V, rho, phi, cot, grad, rho, (T)beta, (T)lam, (T)dt,
                                                   (T)p.dv, N);
     DDI_LAUNCH_CHECK();
     if (lam != 0.0) DDI_TRY(run_ddi<T>(p, rho, phi, s));
     k_adj_b<T><<<blocks_for(N), kThreads, 0, s>>>(psi1, rho, lam != 0.0 ? phi : nullptr, cot, (T)beta, (T)lam, N);
     DDI_LAUNCH_CHECK();
-    return kinetic(cot, +0.25 * dt);
+    return kinetic(cot, 1);
   }
 
   int ground_state(C* phi0, const T* V, double beta, double lam, double dt, double tol, int rule,
                    double inner_tol, int max_steps, int check_every, gpe_stats* out) {
-    C* cur = static_cast<C*>(p.d_psi1);
-    C* nxt = static_cast<C*>(p.d_work);
+    C* const buf[2] = {static_cast<C*>(p.d_work), static_cast<C*>(p.d_psi1)};  // the sweeps' outputs in turn
     C* prev = static_cast<C*>(p.d_work2);
     T* rho = static_cast<T*>(p.d_rho);
     T* dip = static_cast<T*>(p.d_phi);
-    DDI_TRY(normalise(phi0, nullptr));
+    DDI_TRY(normalise(phi0, phi0, nullptr));
     gpe_stats st{};
     DDI_TRY(energy(phi0, V, beta, lam, &st));
     double e_prev = st.E;
-    int inner_max_seen = 0;
+    int inner_max_seen = 0, sweeps_guess = 8;
     double change = INFINITY;
     if (check_every < 1) check_every = 1;
     for (int n = 1; n <= max_steps; ++n) {
@@ -705,34 +642,52 @@ struct Gpe {
         return DDI_ERR_NONFINITE;
       }
       const double alpha = 0.5 * (wr[0] - wr[1]);
-      const double inv_dt_alpha = 1.0 / dt + alpha;
-      DDI_CUDA(cudaMemcpyAsync(cur, phi0, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
-      int it = 0;
-      for (it = 1; it <= 200; ++it) {
-        k_gf_rhs<T><<<blocks_for(N), kThreads, 0, s>>>(phi0, cur, V, rho, lam != 0.0 ? dip : nullptr, nxt, (T)beta,
-                                                       (T)lam, (T)alpha, (T)(1.0 / dt), N);
-        DDI_LAUNCH_CHECK();
-        DDI_TRY(fft(nxt, -1));
-        k_gf_solve<T><<<blocks_for(N), kThreads, 0, s>>>(nxt, g, inv_dt_alpha, 1.0 / (double)N);
-        DDI_LAUNCH_CHECK();
-        DDI_TRY(fft(nxt, +1));
-        double d;
-        DDI_TRY(maxdiff(nxt, cur, &d, nullptr));
-        C* t = cur;
-        cur = nxt;
-        nxt = t;
-        if (!std::isfinite(d)) {
-          set_error("gradient-flow inner iteration diverged at step %d", n);
-          return DDI_ERR_NONFINITE;
+      // the fixed point's sweeps, up to 200, until max|change| <= inner_tol: launched in batches with
+      // one look at their changes per batch; a sweep after the converged one does nothing.  The
+      // first batch is the last step's count (it varies slowly along the flow)
+      GfSweep<T> w{};
+      w.phi = phi0;
+      w.V = V;
+      w.rho = rho;
+      w.dip = lam != 0.0 ? dip : nullptr;
+      w.beta = (T)beta;
+      w.lam = (T)lam;
+      w.alpha = (T)alpha;
+      w.inv_dt = (T)(1.0 / dt);
+      w.inv_dt_alpha = 1.0 / dt + alpha;
+      for (int a = 0; a < 3; ++a) w.ks[a] = g.ks[a];
+      w.tol2 = inner_tol * inner_tol;
+      unsigned long long* change_of = reinterpret_cast<unsigned long long*>(p.d_red + (size_t)(p.red_blocks + 1) * kRedMax);
+      DDI_CUDA(cudaMemsetAsync(change_of, 0, kSweeps * sizeof(double), s));
+      int it = 0, launched = 0;
+      bool converged = false;
+      while (!converged && launched < kSweeps) {
+        const int nb = std::min(std::min(launched ? 2 : sweeps_guess, kSweepBatch), kSweeps - launched);
+        for (int k = launched; k < launched + nb; ++k) {
+          w.cur = k ? buf[(k - 1) & 1] : phi0;
+          w.out = buf[k & 1];
+          w.prev = k ? change_of + k - 1 : nullptr;
+          w.change = change_of + k;
+          DDI_TRY(gpe_gf_sweep<T>(p, w, s));
         }
-        if (d <= inner_tol) break;
+        DDI_CUDA(cudaMemcpyAsync(p.h_red, change_of + launched, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
+        DDI_CUDA(cudaStreamSynchronize(s));
+        for (int k = 0; k < nb && !converged; ++k) {
+          if (!std::isfinite(p.h_red[k])) {
+            set_error("gradient-flow inner iteration diverged at step %d", n);
+            return DDI_ERR_NONFINITE;
+          }
+          it = launched + k + 1;
+          converged = p.h_red[k] <= w.tol2;
+        }
+        launched += nb;
       }
-      if (it > 200) it = 200;
+      sweeps_guess = it;
       inner_max_seen = it > inner_max_seen ? it : inner_max_seen;
-      DDI_TRY(normalise(cur, nullptr));
-      // cur is phi^{n+1}; keep phi^n in prev for the paper's rule
-      DDI_CUDA(cudaMemcpyAsync(prev, phi0, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
-      DDI_CUDA(cudaMemcpyAsync(phi0, cur, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
+      // phi^{n+1} = the last sweep's output, normalised; phi^n is kept for the paper's rule
+      if (rule == GPE_STOP_PAPER)
+        DDI_CUDA(cudaMemcpyAsync(prev, phi0, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
+      DDI_TRY(normalise(buf[(it - 1) & 1], phi0, nullptr));
       if (n % check_every == 0 || n == max_steps) {
         bool done;
         if (rule == GPE_STOP_PAPER) {

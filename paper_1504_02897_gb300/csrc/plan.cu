@@ -100,7 +100,7 @@ void free_plan(Plan& p) {
                   p.d_visits, p.d_units, p.d_split, p.d_counter, p.d_psi1, p.d_rho, p.d_phi, p.d_work,
                   p.d_work2,  p.d_kin,   p.d_red,   p.d_io_in, p.d_io_out, p.d_cvis, p.d_cunits, p.d_cred,
                   p.d_cslots, p.d_cpart, p.d_nonfinite, p.d_cimage, p.d_cnodes, p.d_cshare,
-                  p.d_cnoff, p.d_cnpos};
+                  p.d_cnoff, p.d_cnpos, p.d_em1};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (int i = 0; i < 8; ++i)
@@ -837,26 +837,35 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
     }
     DDI_TRY(upload(p, (void**)&p.d_dirw, dirw, "node directions", stream));
   }
-  // deconvolution factors stay FP64 in both precisions; FP32 plans also get the x factors
+  // deconvolution factors stay FP64 in both precisions; FP32 plans also get the y factors
   // as FP32 head + tail pairs (applied so that only the final product is rounded)
-  auto pairs = [](const std::vector<double>& v, int n) {
-    std::vector<float2> out((size_t)n);
-    for (int j = 0; j < n; ++j) {
-      const float hi = (float)v[j];
-      out[j] = make_float2(hi, (float)(v[j] - (double)hi));
+  auto pairs = [&](const std::vector<double>& v) {
+    std::vector<float2> out((size_t)p.n[1]);
+    for (int j = 0; j < p.n[1]; ++j) {
+      const double f = v[(size_t)p.n[0] + j];
+      const float hi = (float)f;
+      out[j] = make_float2(hi, (float)(f - (double)hi));
     }
     return out;
   };
   DDI_TRY(upload(p, &p.d_deconv, dc, "deconvolution", stream));
-  std::vector<float2> dcx2 = pairs(dc, p.n[0]);
+  std::vector<float2> dcx2 = pairs(dc);
   DDI_TRY(upload(p, &p.d_deconv_x2, dcx2, "deconvolution pairs", stream));
   std::vector<double> ones;
   std::vector<float2> ones2;
+  std::vector<double> em1;
+  std::vector<float> em1f;
   if (p.split()) {
     ones.assign((size_t)p.n[0] + p.n[1] + p.n[2], 1.0);
-    ones2 = pairs(ones, p.n[0]);
+    ones2 = pairs(ones);
     DDI_TRY(upload(p, &p.d_ones, ones, "unit factors", stream));
     DDI_TRY(upload(p, &p.d_ones_x2, ones2, "unit factor pairs", stream));
+    for (int a = 0; a < 3; ++a)
+      for (int l = 0; l < p.nf[a]; ++l) {
+        const double k = (2.0 * M_PI / ((double)p.nf[a] * p.h[a])) * (double)(l < p.nf[a] / 2 ? l : l - p.nf[a]);
+        em1.push_back(std::expm1(-(k * k) / (d.split_k0 * d.split_k0)));
+      }
+    DDI_TRY(upload_real(p, &p.d_em1, em1, "window factors", stream, &em1f));
   }
   DDI_TRY(dev_alloc(p, (void**)&p.d_counter, 2 * sizeof(int), "unit counters"));
   DDI_TRY(dev_alloc(p, (void**)&p.d_nonfinite, sizeof(int), "non-finite record"));
@@ -878,7 +887,7 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
   DDI_TRY(dev_alloc(p, &p.d_phi, rs * N, "gpe phi"));
   DDI_TRY(dev_alloc(p, &p.d_work, cs * N, "gpe work"));
   DDI_TRY(dev_alloc(p, &p.d_work2, cs * N, "gpe work2"));
-  DDI_TRY(dev_alloc(p, &p.d_kin, cs * (p.n[0] + p.n[1] + p.n[2]), "kinetic tables"));
+  DDI_TRY(dev_alloc(p, &p.d_kin, cs * 2 * (p.n[0] + p.n[1] + p.n[2]), "kinetic tables"));
   p.red_blocks = 1024;
   DDI_TRY(dev_alloc(p, (void**)&p.d_red, sizeof(double) * 16 * (p.red_blocks + 1), "reductions"));
   if (cudaMallocHost((void**)&p.h_red, sizeof(double) * 64) != cudaSuccess) {
