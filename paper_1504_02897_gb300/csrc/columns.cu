@@ -1,4 +1,5 @@
-// Column spread of 3D plans (type 1, Sec. 2.1, Eq. DDI-Trun1), FP32 and FP64.
+// Column spread and interpolation of 3D plans (Sec. 2.1, Eq. DDI-Trun1), FP32 and FP64, and the block
+// spread of FP32 2D plans.
 //
 // A warp takes a unit: a range of groups of one column and a window of z-planes.  Lane (lx, ly)
 // owns the cells (lx, ly) and (lx, ly + 4) of the column and keeps W planes of both in
@@ -110,6 +111,7 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_spread
   static_assert(W <= 16 && W % 2 == 0, "planes in register pairs 0..W/2-1 of the window");
   static_assert(!COMP || sizeof(T) == 4, "compensated sums are built for FP32");
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  chain_release();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned char* sm = smem_raw + warp * S::BYTES;
   unsigned char* su = sm + S::U;
@@ -139,6 +141,7 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_spread
   };
   if (un < a.nunits) load_unit();
   request_first();
+  chain_wait();
   while (un < a.nunits) {
     const ColUnit U = {word(0), word(1), word(2), word(3), word(4), word(5), word(6), word(7)};
     int nx = 0;
@@ -304,6 +307,127 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_spread
   cp_async_wait<0>();
 }
 
+// 2D spread (FP32): a warp takes a unit, a range of groups of one 8 x 8 block, and sums
+// c_q psi_x psi_y for its two cells per lane, four visits at a time: four 16-byte shared loads and
+// eight packed FMAs, three issues a visit.  A block of several units goes to partial slots that
+// k_reduce_col3 sums in unit order.
+//
+// The 2N x 2N polar rule puts about 1.3 nodes on every fine cell, so the blocks' visit lists are long
+// and there is nothing to share between nodes (no rings of one k_z).  The kernels this replaces kept
+// windows of rows whose runs were 1-3 visits (columns) or read and wrote each tap in shared memory
+// (tiles).  Bound by issue and by reading the images (72 bytes a visit, 3.5 visits a node).  Spread +
+// reduction, against the tiles: 128^2 39 -> 17 us, 512^2 90 -> 51 us, 1024^2 299 -> 135 us.
+struct BlockArgs {
+  int nfx, ncx;
+  const ColUnit* units;  // col: block index; z0: -1 (the fine grid) or the partial slot
+  int nunits;
+  int* counter;
+  const unsigned char* image;
+  const int* nodes;
+  const float2* c;
+  float2* fine;
+  float2* partial;
+};
+
+struct BlockSmem {
+  static constexpr int U = 2 * BlockImage<float>::BYTES;
+  static constexpr int BYTES = (U + 16 * BlockImage<float>::RS + 127) / 128 * 128;
+};
+
+__global__ void __launch_bounds__(kColThreads3, 8) k_spread_block(BlockArgs a) {
+  using I = BlockImage<float>;
+  using S = BlockSmem;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  chain_release();
+  chain_wait();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* sm = smem_raw + warp * S::BYTES;
+  unsigned char* su = sm + S::U;
+  const int lx = lane & 7, ly = lane >> 3;
+  const int nwarps = gridDim.x * (blockDim.x >> 5);
+  const float2 zero = make_float2(0.f, 0.f);
+  for (int un = warp * gridDim.x + blockIdx.x; un < a.nunits;) {
+    const ColUnit U = a.units[un];
+    int nx = 0;
+    if (lane == 0) nx = atomicAdd(a.counter, 1);
+    float2 s0r = zero, s0i = zero, s1r = zero, s1i = zero;
+    // group images are copied one ahead, node values read one ahead, node indices two ahead
+    int buf = 0, nnext = -1;
+    float2 cnext = zero;
+    if (U.lo < U.hi) {
+      copy_image<I::BYTES>(sm, a.image + (size_t)U.lo * I::BYTES, lane);
+      const int n0 = __ldg(a.nodes + (size_t)U.lo * 32 + lane);
+      if (U.lo + 1 < U.hi) nnext = __ldg(a.nodes + (size_t)(U.lo + 1) * 32 + lane);
+      if (n0 >= 0) cnext = __ldg(a.c + n0);
+    }
+    cp_async_commit();
+    for (int gi = U.lo; gi < U.hi; ++gi) {
+      const float2 c = cnext;
+      cnext = zero;
+      if (gi + 1 < U.hi) {
+        copy_image<I::BYTES>(sm + (buf ^ 1) * I::BYTES, a.image + (size_t)(gi + 1) * I::BYTES, lane);
+        if (nnext >= 0) cnext = __ldg(a.c + nnext);
+        nnext = gi + 2 < U.hi ? __ldg(a.nodes + (size_t)(gi + 2) * 32 + lane) : -1;
+      }
+      cp_async_commit();
+      cp_async_wait<1>();
+      __syncwarp();
+      const unsigned char* im = sm + buf * I::BYTES;
+      buf ^= 1;
+      // u = c psi_x, lane = visit
+#pragma unroll
+      for (int ch = 0; ch < I::CH; ++ch) {
+        const float4 x = *reinterpret_cast<const float4*>(im + I::X + ch * 512 + lane * 16);
+        const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          float* dst = reinterpret_cast<float*>(su + (ch * 4 + k) * I::RS) + lane;
+          dst[0] = c.x * xs[k];
+          *reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(dst) + 8 * I::RS) = c.y * xs[k];
+        }
+      }
+      __syncwarp();
+      // the group's sums, then added to the unit's: a cell takes some hundred terms of the size of its
+      // total, and one running sum of them all lost 1.5 times the accuracy of the result
+      float2 a0r = zero, a0i = zero, a1r = zero, a1i = zero;
+      const float4* ur = reinterpret_cast<const float4*>(su + lx * I::RS);
+      const float4* ui = reinterpret_cast<const float4*>(su + (8 + lx) * I::RS);
+      const float4* y0 = reinterpret_cast<const float4*>(im + I::Y + ly * I::RS);
+      const float4* y1 = reinterpret_cast<const float4*>(im + I::Y + (ly + 4) * I::RS);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float4 r = ur[j], i = ui[j], p = y0[j], q = y1[j];
+        a0r = dot2(make_float2(r.x, r.y), make_float2(p.x, p.y), a0r);
+        a0i = dot2(make_float2(i.x, i.y), make_float2(p.x, p.y), a0i);
+        a1r = dot2(make_float2(r.x, r.y), make_float2(q.x, q.y), a1r);
+        a1i = dot2(make_float2(i.x, i.y), make_float2(q.x, q.y), a1i);
+        a0r = dot2(make_float2(r.z, r.w), make_float2(p.z, p.w), a0r);
+        a0i = dot2(make_float2(i.z, i.w), make_float2(p.z, p.w), a0i);
+        a1r = dot2(make_float2(r.z, r.w), make_float2(q.z, q.w), a1r);
+        a1i = dot2(make_float2(i.z, i.w), make_float2(q.z, q.w), a1i);
+      }
+      s0r = __fadd2_rn(s0r, a0r);
+      s0i = __fadd2_rn(s0i, a0i);
+      s1r = __fadd2_rn(s1r, a1r);
+      s1i = __fadd2_rn(s1i, a1i);
+      __syncwarp();  // the next group overwrites this image and u
+    }
+    const float2 v0 = make_float2(dot_sum(s0r), dot_sum(s0i)), v1 = make_float2(dot_sum(s1r), dot_sum(s1i));
+    if (U.z0 >= 0) {
+      float2* dst = a.partial + (size_t)U.z0 * (kColX * kColY) + lane;
+      dst[0] = v0;
+      dst[32] = v1;
+    } else {
+      const int bx = U.col % a.ncx, by = U.col / a.ncx;
+      float2* dst = a.fine + (long long)(by * kColY + ly) * a.nfx + bx * kColX + lx;
+      dst[0] = v0;
+      dst[4 * a.nfx] = v1;
+    }
+    un = nwarps + __shfl_sync(0xffffffffu, nx, 0);
+  }
+  cp_async_wait<0>();
+}
+
 // Planes of a column that several units touch: the entry's partial slots are contiguous (s0 ..
 // s0 + ns - 1, in unit order).  The first `nlong` entries hold many slots (the dense columns
 // around k = 0: hundreds): a CTA's 8 warps sum a contiguous eighth each, then warp 0 adds the
@@ -315,6 +439,8 @@ __global__ void __launch_bounds__(256)
                   cx_t<T>* __restrict__ fine, int nfx, int nfy, int ncx) {
   using C = cx_t<T>;
   __shared__ C sh[7][64];
+  chain_release();
+  chain_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool team = (int)blockIdx.x < nlong;
   const int e = team ? (int)blockIdx.x : nlong + ((int)blockIdx.x - nlong) * 8 + warp;
@@ -411,6 +537,8 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_interp
   using I = ColImage<T, W>;
   using S = InterpSmem<T, W>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  chain_release();
+  chain_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned char* sm = smem_raw + warp * S::BYTES;
   unsigned char* sh = sm + S::H;
@@ -537,6 +665,8 @@ __global__ void __launch_bounds__(256)
                 const T* __restrict__ scale, cx_t<T>* __restrict__ c, int count) {
   using C = cx_t<T>;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  chain_release();
+  chain_wait();
   if (i >= count) return;
   const int b = off[i], e = off[i + 1];
   C sum = cmk<C>((T)0, (T)0);
@@ -586,16 +716,26 @@ __global__ void __launch_bounds__(128)
   if (lane == 0) *reinterpret_cast<int2*>(im + I::COUNTS) = n;
 }
 
-// raises a kernel's dynamic shared memory limit (it belongs to the kernel, shared by every plan
-// and thread: only raised)
-int raise_smem(const void* fn, size_t bytes) {
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lock(mu);
-  cudaFuncAttributes fa;
-  DDI_CUDA(cudaFuncGetAttributes(&fa, fn));
-  if ((size_t)fa.maxDynamicSharedSizeBytes < bytes)
-    DDI_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  return DDI_OK;
+// the 2D images: vis as in k_col_image
+template <int W>
+__global__ void __launch_bounds__(128)
+    k_block_image(const int2* __restrict__ vis, const float* __restrict__ psi, unsigned char* __restrict__ image,
+                  int* __restrict__ nodes, int ngroups) {
+  using I = BlockImage<float>;
+  const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (g >= ngroups) return;
+  unsigned char* im = image + (size_t)g * I::BYTES;
+  const int2 v = vis[(size_t)g * 32 + lane];
+  nodes[(size_t)g * 32 + lane] = v.x;
+  const int ox = (v.y & 63) - 16, oy = ((v.y >> 6) & 63) - 16;
+  const float* ps = psi + (size_t)(v.x < 0 ? 0 : v.x) * 3 * W;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const bool inx = v.x >= 0 && (unsigned)(c - ox) < (unsigned)W, iny = v.x >= 0 && (unsigned)(c - oy) < (unsigned)W;
+    *reinterpret_cast<float*>(im + I::X + c / I::EPC * 512 + lane * 16 + c % I::EPC * 4) = inx ? ps[c - ox] : 0.f;
+    *reinterpret_cast<float*>(im + I::Y + c * I::RS + lane * 4) = iny ? ps[W + c - oy] : 0.f;
+  }
+  if (lane < 8) *reinterpret_cast<int4*>(im + I::Y + lane * I::RS + 128) = make_int4(0, 0, 0, 0);  // row padding
 }
 
 enum class ColOp { ImageBytes, BuildImage, Configure, Spread, Interp };
@@ -627,8 +767,8 @@ int col_op(Plan& p, cudaStream_t s, ColOp op, const ColBuild* b, size_t* out) {
   constexpr size_t ismem = (size_t)InterpSmem<T, W>::BYTES * (kColThreads3 / 32);
   constexpr int wpc = kColThreads3 / 32;
   if (op == ColOp::Configure) {
-    DDI_TRY(raise_smem(reinterpret_cast<const void*>(kern), smem));
-    DDI_TRY(raise_smem(reinterpret_cast<const void*>(interp), ismem));
+    DDI_TRY(prepare_kernel(reinterpret_cast<const void*>(kern), smem));
+    DDI_TRY(prepare_kernel(reinterpret_cast<const void*>(interp), ismem));
     int per_sm = 0, iper_sm = 0, sms = 0;
     DDI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kColThreads3, smem));
     DDI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&iper_sm, interp, kColThreads3, ismem));
@@ -650,14 +790,11 @@ int col_op(Plan& p, cudaStream_t s, ColOp op, const ColBuild* b, size_t* out) {
     a.image = p.d_cimage;
     a.fine = p.d_fine;
     a.share = p.d_cshare;
-    DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, 2 * sizeof(int), s));
-    interp<<<p.interp_blocks, kColThreads3, ismem, s>>>(a);
-    DDI_LAUNCH_CHECK();
+    DDI_TRY(launch_chain(p, interp, p.interp_blocks, kColThreads3, ismem, s, a));
     p.mark("interp", s);
-    k_node_sum3<T><<<(unsigned)((p.Mh + 255) / 256), 256, 0, s>>>(
-        p.d_cnoff, p.d_cnpos, static_cast<const cx_t<T>*>(p.d_cshare), static_cast<const T*>(p.d_scale),
-        static_cast<cx_t<T>*>(p.d_c), (int)p.Mh);
-    DDI_LAUNCH_CHECK();
+    DDI_TRY(launch_chain(p, k_node_sum3<T>, (unsigned)((p.Mh + 255) / 256), 256, 0, s, p.d_cnoff, p.d_cnpos,
+                         static_cast<const cx_t<T>*>(p.d_cshare), static_cast<const T*>(p.d_scale),
+                         static_cast<cx_t<T>*>(p.d_c), (int)p.Mh));
     p.mark("node_sum", s);
     return DDI_OK;
   }
@@ -673,22 +810,71 @@ int col_op(Plan& p, cudaStream_t s, ColOp op, const ColBuild* b, size_t* out) {
   a.fine = p.d_fine;
   a.partial = p.d_cpart;
   a.dest = p.d_cslots;
-  DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, sizeof(int), s));
-  kern<<<p.spread_blocks, kColThreads3, p.spread_smem, s>>>(a);
-  DDI_LAUNCH_CHECK();
+  DDI_TRY(launch_chain(p, kern, p.spread_blocks, kColThreads3, p.spread_smem, s, a));
   p.mark("spread", s);
   if (p.ncred > 0) {
-    k_reduce_col3<T><<<(unsigned)(p.ncred_long + (p.ncred - p.ncred_long + 7) / 8), 256, 0, s>>>(
-        p.d_cred, p.ncred, p.ncred_long, static_cast<const cx_t<T>*>(p.d_cpart), static_cast<cx_t<T>*>(p.d_fine),
-        p.nf[0], p.nf[1], a.ncx);
+    DDI_TRY(launch_chain(p, k_reduce_col3<T>, (unsigned)(p.ncred_long + (p.ncred - p.ncred_long + 7) / 8), 256, 0, s,
+                         p.d_cred, p.ncred, p.ncred_long, static_cast<const cx_t<T>*>(p.d_cpart), static_cast<cx_t<T>*>(p.d_fine), p.nf[0], p.nf[1], a.ncx));
+    p.mark("spread_reduce", s);
+  }
+  return DDI_OK;
+}
+
+template <int W>
+int block_op(Plan& p, cudaStream_t s, ColOp op, const ColBuild* b, size_t* out) {
+  using I = BlockImage<float>;
+  constexpr int wpc = kColThreads3 / 32;
+  constexpr size_t smem = (size_t)BlockSmem::BYTES * wpc;
+  if (op == ColOp::ImageBytes) {
+    *out = I::BYTES;
+    return DDI_OK;
+  }
+  if (op == ColOp::BuildImage) {
+    if (p.ngroups == 0) return DDI_OK;
+    k_block_image<W><<<(unsigned)((p.ngroups + 3) / 4), 128, 0, s>>>(b->vis, static_cast<const float*>(p.d_psi),
+                                                                     p.d_cimage, p.d_cnodes, p.ngroups);
     DDI_LAUNCH_CHECK();
+    return DDI_OK;
+  }
+  if (op == ColOp::Configure) {
+    DDI_TRY(prepare_kernel(reinterpret_cast<const void*>(k_spread_block), smem));
+    int per_sm = 0, sms = 0;
+    DDI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread_block, kColThreads3, smem));
+    DDI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device));
+    p.spread_smem = smem;
+    p.spread_blocks = std::max(1, std::min(per_sm * sms, (p.ncunits + wpc - 1) / wpc));
+    return DDI_OK;
+  }
+  if (op != ColOp::Spread) {
+    set_error("column interpolation: not built in 2D");
+    return DDI_ERR_INTERNAL;
+  }
+  BlockArgs a;
+  a.nfx = p.nf[0];
+  a.ncx = p.nf[0] / kColX;
+  a.units = p.d_cunits;
+  a.nunits = p.ncunits;
+  a.counter = p.d_counter;
+  a.image = p.d_cimage;
+  a.nodes = p.d_cnodes;
+  a.c = static_cast<const float2*>(p.d_c);
+  a.fine = static_cast<float2*>(p.d_fine);
+  a.partial = static_cast<float2*>(p.d_cpart);
+  DDI_TRY(launch_chain(p, k_spread_block, p.spread_blocks, kColThreads3, p.spread_smem, s, a));
+  p.mark("spread", s);
+  if (p.ncred > 0) {
+    DDI_TRY(launch_chain(p, k_reduce_col3<float>, (unsigned)(p.ncred_long + (p.ncred - p.ncred_long + 7) / 8), 256, 0, s,
+                         p.d_cred, p.ncred, p.ncred_long, static_cast<const float2*>(p.d_cpart), static_cast<float2*>(p.d_fine), p.nf[0], p.nf[1], a.ncx));
     p.mark("spread_reduce", s);
   }
   return DDI_OK;
 }
 
 int col_dispatch(Plan& p, cudaStream_t s, ColOp op, const ColBuild* b, size_t* out) {
-  if (p.prec == DDI_FP32) {
+  if (p.dim == 2) {
+    if (p.w == 6) return block_op<6>(p, s, op, b, out);
+    if (p.w == 8) return block_op<8>(p, s, op, b, out);
+  } else if (p.prec == DDI_FP32) {
     switch (p.w) {
       case 6: return p.col_comp ? col_op<float, 6, true>(p, s, op, b, out) : col_op<float, 6, false>(p, s, op, b, out);
       case 8: return p.col_comp ? col_op<float, 8, true>(p, s, op, b, out) : col_op<float, 8, false>(p, s, op, b, out);
@@ -715,8 +901,8 @@ int build_col_images(Plan& p, const int2* vis, const int* runs, const int2* coun
   const ColBuild b{vis, runs, counts};
   return col_dispatch(p, s, ColOp::BuildImage, &b, nullptr);
 }
-int configure_spread_col3(Plan& p) { return col_dispatch(p, nullptr, ColOp::Configure, nullptr, nullptr); }
-int launch_interp_col3(Plan& p, cudaStream_t s) { return col_dispatch(p, s, ColOp::Interp, nullptr, nullptr); }
-int launch_spread_col3(Plan& p, cudaStream_t s) { return col_dispatch(p, s, ColOp::Spread, nullptr, nullptr); }
+int configure_spread_col(Plan& p) { return col_dispatch(p, nullptr, ColOp::Configure, nullptr, nullptr); }
+int launch_interp_col(Plan& p, cudaStream_t s) { return col_dispatch(p, s, ColOp::Interp, nullptr, nullptr); }
+int launch_spread_col(Plan& p, cudaStream_t s) { return col_dispatch(p, s, ColOp::Spread, nullptr, nullptr); }
 
 }  // namespace ddi

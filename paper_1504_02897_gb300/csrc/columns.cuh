@@ -31,4 +31,15 @@ struct ColImage {
   static constexpr int BYTES = (COUNTS + 8 + 15) / 16 * 16;
 };
 
+// 2D: blocks of kColX x kColY cells; a group is 32 visits of one block and its image the X rows and
+// Y rows alone.
+template <typename T>
+struct BlockImage {
+  static constexpr int EPC = 16 / (int)sizeof(T);
+  static constexpr int CH = 8 / EPC;
+  static constexpr int RS = 32 * (int)sizeof(T) + 16;
+  static constexpr int X = 0, Y = CH * 512;
+  static constexpr int BYTES = Y + 8 * RS;
+};
+
 }  // namespace ddi

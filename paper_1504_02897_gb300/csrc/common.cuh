@@ -96,18 +96,19 @@ struct SplitUnit {
 };
 
 // ---- column spread work list -------------------------------------------------------------------
-// A column is a kColX x kColY block of fine cells in x-y with all its z-planes (2D: kColX cells
-// in x with every y line).  A work unit takes a range of the column's visits, sorted by their
-// first tap along the window axis (z; 2D: y), and a window of planes.
+// 3D: a column is a kColX x kColY block of fine cells in x-y with all its z-planes.  A work unit
+// takes a range of the column's visits, sorted by their first z tap, and a window of planes.
+// 2D: a block is kColX x kColY cells; a unit takes a range of its visits.
 constexpr int kColX = 8, kColY = 8;
 constexpr int kColRuns = 8;     // 3D: most runs of one z class per group of 32 visits (columns.cuh)
 constexpr int kColPlanes = 32;  // 3D: most planes of a unit's window
 struct alignas(16) ColUnit {
-  int col;       // column index cy * (nf_x / kColX) + cx
-  int lo, hi;    // range of groups (3D) or visits (2D)
-  int z0, z1;    // planes [z0, z1) the unit writes (plane z mod nf_z; z1 may exceed nf_z)
-  int plo, phi;  // leading / trailing planes that other units also touch: go to partial slots
-  int slot0;     // 2D: its shared rows (leading, then trailing) are entries slot0 .. of the unit slot map
+  int col;       // column or block index cy * (nf_x / kColX) + cx
+  int lo, hi;    // range of groups
+  int z0, z1;    // 3D: planes [z0, z1) the unit writes (plane z mod nf_z; z1 may exceed nf_z);
+                 // 2D: z0 = -1 (the unit writes the block) or its partial slot
+  int plo, phi;  // 3D: leading / trailing planes that other units also touch: go to partial slots
+  int slot0;     // 3D, plan time: its shared planes (leading, then trailing) count from slot0
 };
 struct alignas(16) ColRed {  // a plane of a column touched by several units: the sum of their partial slots
   int col, z;
@@ -176,7 +177,7 @@ struct Plan {
   NodeDir* d_dirw = nullptr;  // [Mh]: direction and weight without the symbol (ddi_plan_set_axes)
   void* d_c = nullptr;        // cx [Mh]: node values c_q
   void* d_deconv = nullptr;   // double [n0 + n1 + n2]: 1/psihat per axis, index j (0..n-1)
-  void* d_deconv_x2 = nullptr;  // float2 [n1]: the y factors as FP32 head + tail (FP32 plans)
+  void* d_deconv_x2 = nullptr;  // float2 [n1] (2D: [n0]): the y (x) factors as FP32 head + tail (FP32 plans)
   void* d_ones = nullptr;     // double [n0 + n1 + n2] of ones: the pad and crop of a split plan's smooth part
   void* d_em1 = nullptr;      // T [nf0 + nf1 + nf2], split plans: e^{-k_d^2/k0^2} - 1 at the fine grid's modes
   void* d_ones_x2 = nullptr;  // float2 [n1] of (1, 0)
@@ -189,10 +190,9 @@ struct Plan {
   int* d_nonfinite = nullptr; // set by the pad pass when rho holds NaN / Inf (cleared by checks)
   // column spread (spread_kind == DDI_SPREAD_COLUMNS)
   int spread_kind = DDI_SPREAD_TILES;
-  int2* d_cvis = nullptr;     // 2D visits (node, first y tap << 13 | run start << 12 | (oy + 16) << 6 | (ox + 16))
-  unsigned char* d_cimage = nullptr;  // 3D: the groups' images (columns.cuh)
-  int* d_cnodes = nullptr;    // 3D: [group][32] node of each visit, -1: none
-  int ngroups = 0;            // 3D: groups of visits
+  unsigned char* d_cimage = nullptr;  // the groups' images (columns.cuh)
+  int* d_cnodes = nullptr;    // [group][32] node of each visit, -1: none
+  int ngroups = 0;            // groups of visits
   void* d_cshare = nullptr;   // 3D: [group][32] each visit's share of its node's value (interpolation)
   int* d_cnoff = nullptr;     // 3D: [Mh + 1] ranges of d_cnpos
   int* d_cnpos = nullptr;     // 3D: where a node's shares are in d_cshare
@@ -201,11 +201,11 @@ struct Plan {
   bool col_interp = false;    // 3D: interpolate by columns too
   ColUnit* d_cunits = nullptr;
   ColRed* d_cred = nullptr;
-  int* d_cslots = nullptr;    // 2D: per unit (from its slot0) the partial slot of each shared row; 3D: [unit][kColPlanes],
-                              // the partial slot of each plane of its window, -1 where it alone writes the plane
+  int* d_cslots = nullptr;    // 3D: [unit][kColPlanes], the partial slot of each plane of its window, -1 where it
+                              // alone writes the plane
   void* d_cpart = nullptr;    // partial planes: [slot][kColY * kColX] complex
   int ncunits = 0, ncred = 0, ncslots = 0;
-  int ncred_long = 0;         // 3D: the first reduce entries, each summed by a whole CTA
+  int ncred_long = 0;         // the first reduce entries, each summed by a whole CTA
   bool col_comp = false;      // column spread: compensated (Kahan) plane accumulation
   long long visits = 0;       // total visit-list entries
   long long pairs = 0;        // total (node, plane) pairs of all units
@@ -223,7 +223,7 @@ struct Plan {
   // fine-grid x lines that hold node taps (every line, except for split plans' ball band)
   int xr[2] = {0, 1};
   bool precise_nufft = false;  // NUFFT passes apply FP32 twiddles as head + tail
-  bool batch_item = false;     // built by ddi_batch_create (2D items spread by columns, see create_plan)
+  bool batch_item = false;     // built by ddi_batch_create
   int tw_n[8] = {};           // lengths of the twiddle tables below
   void* d_tw[8] = {};         // cx twiddle tables e^{-2 pi i k / n} (FP32: n heads, then n tails)
   // GPE workspace
@@ -262,6 +262,41 @@ struct Plan {
   size_t real_size() const { return prec == DDI_FP64 ? 8 : 4; }
   size_t cx_size() const { return prec == DDI_FP64 ? 16 : 8; }
 };
+
+// ---- launches of the DDI's chain of kernels ------------------------------------------------------
+// The kernels of an evaluation follow one another on one stream, each needing all of the one before.
+// They are launched programmatically dependent: a kernel's CTAs may be placed, and do what needs only
+// the plan's constants, while the last CTAs of the one before are still running; chain_wait() then
+// holds them until that kernel has completed and its writes are visible.  Every such kernel calls
+// chain_wait() in all its threads before it touches what an evaluation writes (or anything a
+// caller's work on the stream may still use), so completion carries over along the chain.  Saves
+// the launch gap of each of the 9-14 kernels: 24^3 50 -> 40 us, 128^3 304 -> 281 us, four 128^3 steps
+// 1525 -> 1385 us.  Not used inside batches, whose side streams fill the gaps, nor in FP64, whose
+// kernels are long (128^3 6.73 against 6.75 ms; rotating 64^3 steps were slower with it, 2.95
+// against 2.72 ms).
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Once per kernel and device: raises the kernel's dynamic shared memory limit to `smem` (the limit
+// belongs to the kernel, shared by every plan and thread: only raised).
+int prepare_kernel(const void* fn, size_t smem);
+
+template <typename... P, typename... A>
+int launch_chain(const Plan& p, void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                 A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = p.batch_item || p.prec == DDI_FP64 ? 0 : 1;
+  DDI_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...));
+  return DDI_OK;
+}
 
 inline const void* twiddles(const Plan& p, int n) {
   for (int i = 0; i < 8; ++i)
@@ -325,9 +360,9 @@ __host__ __device__ inline size_t spread_warp_bytes(size_t plane_bytes, size_t s
 // launch geometry, and the spread with its reduction
 size_t col_image_bytes(Plan& p);
 int build_col_images(Plan& p, const int2* vis, const int* runs, const int2* counts, cudaStream_t s);
-int configure_spread_col3(Plan& p);
-int launch_spread_col3(Plan& p, cudaStream_t s);
-int launch_interp_col3(Plan& p, cudaStream_t s);  // fine grid -> d_c
+int configure_spread_col(Plan& p);
+int launch_spread_col(Plan& p, cudaStream_t s);
+int launch_interp_col(Plan& p, cudaStream_t s);  // fine grid -> d_c
 int configure_kernels(Plan& p);  // per-plan launch geometry (nufft.cu)
 // reads and clears the plan's non-finite-input record after synchronising s:
 // DDI_ERR_NONFINITE if it was set (plan.cu)
@@ -337,9 +372,8 @@ int take_nonfinite(Plan& p, cudaStream_t s);
 int create_plan(Plan& p, const ddi_plan_desc* desc, cudaStream_t stream, bool gpe = true, bool batch_item = false);
 void set_tile(Plan& p, const int want[3]);         // tile rounded as for ddi_plan_desc.tile
 int build_spread(Plan& p, cudaStream_t stream);     // spread lists for the current tile
-int build_spread_col(Plan& p, cudaStream_t stream); // column spread lists for desc.chunk (plan.cu)
+int build_spread_col(Plan& p, cudaStream_t stream); // column (2D: block) spread lists for desc.chunk (plan.cu)
 bool columns_apply(const Plan& p);                   // the column spread fits the plan (plan.cu)
-void drop_spread_lists(Plan& p);                    // frees both schemes' spread lists (plan.cu)
 int time_spread(Plan& p, cudaStream_t s, int reps, float* ms);  // best of reps (nufft.cu)
 int tune_spread_tile(Plan& p, cudaStream_t s);      // autotuner (batch.cu)
 void destroy_plan(Plan& p);

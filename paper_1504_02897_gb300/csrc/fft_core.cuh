@@ -101,21 +101,62 @@ struct Dft<3, DIR, C> {
   }
 };
 
-__device__ __forceinline__ int pidx(int i) { return i + (i >> 4); }
+// 12 = 3 x 4 points by the prime-factor map (no twiddles between the factors): with
+// n = (4 n1 + 3 n2) mod 12 and k = (4 k1 + 9 k2) mod 12, n k = 4 n1 k1 + 3 n2 k2 (mod 12)
+template <int DIR, typename C>
+struct Dft<12, DIR, C> {
+  __device__ __forceinline__ static void run(C* v) {
+    C a[4][3];
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) {
+#pragma unroll
+      for (int n1 = 0; n1 < 3; ++n1) a[n2][n1] = v[(4 * n1 + 3 * n2) % 12];
+      Dft<3, DIR, C>::run(a[n2]);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+      C u[4];
+#pragma unroll
+      for (int n2 = 0; n2 < 4; ++n2) u[n2] = a[n2][k1];
+      Dft<4, DIR, C>::run(u);
+#pragma unroll
+      for (int k2 = 0; k2 < 4; ++k2) v[(4 * k1 + 9 * k2) % 12] = u[k2];
+    }
+  }
+};
 
-// radix of the stage that follows sub-transform length NS (16, then 8/4/2, then 3)
+__device__ __forceinline__ int pidx(int i) { return i + (i >> 4); }
+// pidx(i + r STEP) given pi = pidx(i): one constant offset where STEP is a multiple of 16 (the
+// compiler cannot split the shift of a sum)
+template <int STEP>
+__device__ __forceinline__ int pidx_at(int i, int pi, int r) {
+  return STEP % 16 == 0 ? pi + r * (STEP + STEP / 16) : pidx(i + r * STEP);
+}
+
+// Radix of the stage that follows sub-transform length NS: 16, then what is left (8, 4, 2 and 3).
+// Lengths 3 * 2^a up to 192 take 12 first and 32 takes 8 and 4: two stages for 96 and 192 where 16, 2
+// or 4 and 3 made three (96^3 gradient-flow sweep 51 -> 46 us).  384 and 512 stay with 16 first:
+// 12 or 16, 8 and 4 took their passes from 76 to 96 and from 110 to 160 us.
 __host__ __device__ constexpr int pow2_part(int n) { return n & (-n); }
 __host__ __device__ constexpr int radix_for(int N, int NS) {
-  return pow2_part(N / NS) >= 16 ? 16 : (pow2_part(N / NS) > 1 ? pow2_part(N / NS) : 3);
+  const int left = N / NS;
+  if (N <= 192 && left % 3 == 0) return 12;
+  if (left == 32 && N == 32) return 8;
+  return pow2_part(left) >= 16 ? 16 : (pow2_part(left) > 1 ? pow2_part(left) : 3);
 }
-__host__ __device__ constexpr int max_radix(int N) { return pow2_part(N) >= 16 ? 16 : (pow2_part(N) > 3 ? pow2_part(N) : 3); }
 
 template <int N>
 struct Shape {
-  static constexpr int RM = max_radix(N);      // largest radix
+  static constexpr int RM = radix_for(N, 1);   // the first radix: elements per thread
   static constexpr int TPL = N / RM;           // threads per line
   static constexpr int LS = N + N / 16 + 1;    // padded line stride in shared memory
 };
+
+// shared-memory index of the first stage's output r of butterfly t, element t R0 + r
+template <int R0>
+__device__ __forceinline__ int first_out(int t, int r) {
+  return R0 == 16 ? t * 17 + r : pidx(t * R0 + r);
+}
 
 // One Stockham stage of radix R with sub-transform length NS; each thread owns
 // G = ceil(RM / R) butterflies of its line (the last ones masked when R does not divide RM).
@@ -133,8 +174,9 @@ __device__ __forceinline__ void stage_compute(const C* line, int t, const C* __r
   for (int g = 0; g < G; ++g) {
     const int j = t + g * TPL;  // butterfly index in [0, N/R)
     if (RM % R == 0 || j < NB) {
+      const int pj = pidx(j);
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[g][r] = line[pidx(j + r * NB)];
+      for (int r = 0; r < R; ++r) v[g][r] = line[pidx_at<NB>(j, pj, r)];
       if (NS > 1) {
         const int jm = j % NS;
         constexpr int STRIDE = N / (NS * R);
@@ -175,9 +217,9 @@ __device__ __forceinline__ void stage(C* line, int t, const C* __restrict__ tw) 
     const int j = t + g * TPL;
     if (RM % R == 0 || j < NB) {
       const int jm = j % NS;
-      const int idxD = (j - jm) * R + jm;
+      const int idxD = (j - jm) * R + jm, pD = pidx(idxD);
 #pragma unroll
-      for (int r = 0; r < R; ++r) line[pidx(idxD + r * NS)] = v[g][r];
+      for (int r = 0; r < R; ++r) line[pidx_at<NS>(idxD, pD, r)] = v[g][r];
     }
   }
   __syncthreads();
@@ -222,7 +264,7 @@ __device__ __forceinline__ long long line_off(const LineGeom& g, long long L) {
 // Generic batched-line FFT: a policy P supplies nlines(), ref(L) (the line's addresses,
 // computed once per line by one thread), load(ref, i) /
 // store(ref, i, v, acc) for element i of the line, skip() (the whole pass is not needed), an
-// accumulator Acc with finish(acc), and the constants
+// accumulator Acc with finish(acc), begin() (once per thread, before the lines), and the constants
 //   kStrided   the lines' elements are strided in memory and neighbouring lines adjacent (else the
 //              element index is fastest)
 //   kPrecise   apply the twiddle tails (FP32)
@@ -240,6 +282,7 @@ struct PolicyBase {
   struct Acc {};
   static constexpr bool kPrecise = false, kBlockIn = false, kBlockOut = false, kStrided = true;
   __device__ bool skip() const { return false; }
+  __device__ void begin() const {}
   __device__ void finish(const Acc&) const {}
 };
 
@@ -279,13 +322,15 @@ __global__ void __launch_bounds__(LPB * Shape<N>::TPL)
   constexpr int TPL = Shape<N>::TPL;
   constexpr int RM = Shape<N>::RM;
   constexpr int R0 = radix_for(N, 1);
-  static_assert(R0 == RM, "the first stage has one butterfly per thread");
   constexpr int NSL = last_ns(N);      // the last stage's sub-transform length
   constexpr int RL = N / NSL;          // and its radix
   constexpr int GL = (RM + RL - 1) / RL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Ref refs[LPB];
+  chain_release();
+  chain_wait();
   if (pol.skip()) return;
+  pol.begin();
   C* sm = reinterpret_cast<C*>(smem_raw);
   const long long L0 = (long long)blockIdx.x * LPB;
   const long long left = pol.nlines() - L0;
@@ -305,7 +350,7 @@ __global__ void __launch_bounds__(LPB * Shape<N>::TPL)
     if (live) store_last<N, N, 1>(pol, refs[b], 0, v0, acc);
   } else {
 #pragma unroll
-    for (int r = 0; r < R0; ++r) line[pidx(t * R0 + r)] = v0[r];
+    for (int r = 0; r < R0; ++r) line[first_out<R0>(t, r)] = v0[r];
     __syncthreads();
     MidStages<C, N, DIR, R0, NSL, PR>::run(line, t, tw);
     C v[GL][RL];
@@ -338,7 +383,10 @@ __global__ void __launch_bounds__(LPB * Shape<N>::TPL)
   constexpr int GL = (RM + RL - 1) / RL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Ref refs[LPB];
+  chain_release();
+  chain_wait();
   if (pol.skip()) return;
+  pol.begin();
   C* sm = reinterpret_cast<C*>(smem_raw);
   const long long L0 = (long long)blockIdx.x * LPB;
   const long long left = pol.nlines() - L0;
@@ -363,7 +411,7 @@ __global__ void __launch_bounds__(LPB * Shape<N>::TPL)
     if (live) store_last<N, N, 1>(pol, refs[b], 0, v0, acc);
   } else {
 #pragma unroll
-    for (int r = 0; r < R0; ++r) line[pidx(t * R0 + r)] = v0[r];
+    for (int r = 0; r < R0; ++r) line[first_out<R0>(t, r)] = v0[r];
     __syncthreads();
     MidStages<C, N, -1, R0, NSL, PR>::run(line, t, tw);
     {
@@ -380,20 +428,20 @@ __global__ void __launch_bounds__(LPB * Shape<N>::TPL)
             if constexpr (RL == R0)
               v0[r] = m;
             else
-              line[pidx(j + r * NSL)] = m;
+              line[pidx_at<NSL>(j, pidx(j), r)] = m;
           }
         }
       }
       if constexpr (RL != R0) {
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < R0; ++r) v0[r] = line[pidx(t + r * (N / R0))];
+        for (int r = 0; r < R0; ++r) v0[r] = line[pidx_at<N / R0>(t, pidx(t), r)];
         __syncthreads();
       }
     }
     Dft<R0, 1, C>::run(v0);
 #pragma unroll
-    for (int r = 0; r < R0; ++r) line[pidx(t * R0 + r)] = v0[r];
+    for (int r = 0; r < R0; ++r) line[first_out<R0>(t, r)] = v0[r];
     __syncthreads();
     MidStages<C, N, 1, R0, NSL, PR>::run(line, t, tw);
     C v[GL][RL];
@@ -419,7 +467,7 @@ constexpr int lines_per_cta() {
 
 // DIR = 0: forward and inverse in one pass (k_fft_pair)
 template <typename T, int N, int DIR, typename P>
-int launch_policy(const P& pol, const void* tw, cudaStream_t s) {
+int launch_policy(const Plan& p, const P& pol, cudaStream_t s) {
   constexpr int LPB = lines_per_cta<T, N, P::kStrided>();
   constexpr int threads = LPB * Shape<N>::TPL;
   const size_t smem = (size_t)LPB * Shape<N>::LS * sizeof(cx_t<T>);
@@ -428,23 +476,23 @@ int launch_policy(const P& pol, const void* tw, cudaStream_t s) {
     kern = k_fft_pair<T, N, LPB, P>;
   else
     kern = k_fft_policy<T, N, LPB, DIR, P>;
-  if (smem > 48 * 1024) {
-    DDI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  DDI_TRY(prepare_kernel(reinterpret_cast<const void*>(kern), smem));
+  if (!twiddles(p, N)) {
+    set_error("missing twiddle table for FFT length %d", N);
+    return DDI_ERR_ARG;
   }
   const long long blocks = (pol.nlines() + LPB - 1) / LPB;
   if (blocks <= 0) return DDI_OK;
-  kern<<<(unsigned)blocks, threads, smem, s>>>(pol, static_cast<const cx_t<T>*>(tw));
-  DDI_LAUNCH_CHECK();
-  return DDI_OK;
+  return launch_chain(p, kern, (unsigned)blocks, threads, smem, s, pol, static_cast<const cx_t<T>*>(twiddles(p, N)));
 }
 
 // FFT lengths built, 2^a and 3 * 2^a: LO and HI bound the lengths a policy is built for (fine-grid
 // lines 16..2048, 3D 1024; grid lines 8..1024)
 template <typename T, int DIR, int LO, int HI, typename P>
-int dispatch_policy(int n, const P& pol, const void* tw, cudaStream_t s) {
+int dispatch_policy(const Plan& p, int n, const P& pol, cudaStream_t s) {
 #define DDI_LEN(NN)                                                        \
   case NN:                                                                 \
-    if constexpr (NN >= LO && NN <= HI) return launch_policy<T, NN, DIR>(pol, tw, s); \
+    if constexpr (NN >= LO && NN <= HI) return launch_policy<T, NN, DIR>(p, pol, s); \
     break;
   switch (n) {
     DDI_LEN(8) DDI_LEN(12) DDI_LEN(16) DDI_LEN(24) DDI_LEN(32) DDI_LEN(48) DDI_LEN(64) DDI_LEN(96) DDI_LEN(128)

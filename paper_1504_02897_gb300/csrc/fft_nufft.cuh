@@ -5,7 +5,7 @@
 // 2n-oversampled grid and the type-1 output is read back at the same positions.  The density is
 // real, so one half of the spectrum holds all of it, and one node of each (k, -k) pair is
 // processed, the one with k_y >= 0 (the first half of the azimuth): its taps lie on about half of
-// the fine y lines (the plan finds the shortest cyclic range holding all of them).  So y is
+// the fine y lines (the plan finds the shortest cyclic range holding all of them).  So in 3D y is
 // transformed first and returned last, and every other pass works on the lines of that range only:
 //   forward  y: the n_x n_z lines of the density (read straight from rho: pad and deconvolution
 //               fused); only the y lines of the range are stored, in the first n_x cells of
@@ -51,7 +51,7 @@ struct Geo {
   using C = cx_t<T>;
   Axis ax, ay, az;
   // deconvolution factors 1 / psihat, FP64 (x: [0, n0), y: [n0, n0 + n1), z: after), and for
-  // FP32 plans the y factors as FP32 head + tail pairs (the FP64 value to ~2^-48)
+  // FP32 plans the y factors (2D: x) as FP32 head + tail pairs (the FP64 value to ~2^-48)
   const double* dc;
   const float2* dcx2;
   C* fine;
@@ -60,9 +60,10 @@ struct Geo {
   int ylo, nyr;
   int xlo, nxr;
   int* nonfinite;  // set when the pad pass reads a NaN / Inf
-  __device__ long long fidx(int lz, int ly, int lx) const {
-    return ((long long)lz * ay.nf + ly) * ax.nf + lx;
-  }
+  int* counters;   // the work counters of the spread and the interpolation, cleared by the pad pass
+  int sz;  // fine cells per plane
+  // offsets into the fine grid (at most 1024^3 cells) and into rho / phi fit 32 bits
+  __device__ int fidx(int lz, int ly, int lx) const { return lz * sz + ly * ax.nf + lx; }
   __host__ __device__ bool in_yr(int l) const {
     int d = l - ylo;
     if (d < 0) d += ay.nf;
@@ -83,39 +84,53 @@ struct Geo {
   }
 };
 
-// y lines of the density and the potential, one per (x, z) of the grid
+// lines of the density and the potential: along y, one per (x, z) of the grid (3D), or rows (2D)
 template <typename T>
 struct YRef {
-  long long grid;  // offset of the line's first element in rho / phi
-  long long fine;  // the same in the fine grid: row y of plane z, cell x
-  T hi, lo;        // the line's deconvolution factor dx dz (FP64 product): FP64 value, or FP32 head + tail
+  int grid;        // offset of the line's first element in rho / phi
+  int fine;        // the same in the fine grid (3D: row y of plane z, cell x)
+  T hi, lo;        // the line's deconvolution factor (FP64 product of the other axes'): FP64 value, or FP32
+                   // head + tail
 };
 
 template <typename T>
-__device__ __forceinline__ YRef<T> y_ref(const Geo<T>& g, long long L) {
-  const int jx = (int)(L % g.ax.n), jz = (int)(L / g.ax.n);
-  const double f = g.dc[jx] * g.dc[g.ax.n + g.ay.n + jz];
+__device__ __forceinline__ YRef<T> line_ref(int grid, int fine, double f) {
   YRef<T> r;
-  r.grid = (long long)jz * g.ay.n * g.ax.n + jx;
-  r.fine = g.fidx(g.az.fine_of(jz), 0, jx);
+  r.grid = grid;
+  r.fine = fine;
   r.hi = (T)f;
   r.lo = sizeof(T) == 4 ? (T)(f - (double)r.hi) : (T)0;
   return r;
 }
 
-// v times the deconvolution factor of element jy of line r, rounded once: in FP64 directly;
-// in FP32 the factor dx dy dz is formed as a head + tail pair (the exact product error of the
-// heads by an FMA plus the cross terms), so only the final product is rounded
 template <typename T>
-__device__ __forceinline__ T deconv(const Geo<T>& g, const YRef<T>& r, int jy, T v) {
+__device__ __forceinline__ YRef<T> y_ref(const Geo<T>& g, long long L) {
+  const int jz = (int)((unsigned)L / (unsigned)g.ax.n), jx = (int)L - jz * g.ax.n;
+  return line_ref<T>(jz * g.ay.n * g.ax.n + jx, g.fidx(g.az.fine_of(jz), 0, jx),
+                     g.dc[jx] * g.dc[g.ax.n + g.ay.n + jz]);
+}
+
+// v times the deconvolution factor of element j of line r (d: the FP64 factors along the line),
+// rounded once: in FP64 directly; in FP32 the factor dx dy dz is formed as a head + tail pair (the
+// exact product error of the heads by an FMA plus the cross terms), so only the final product is
+// rounded
+template <typename T>
+__device__ __forceinline__ T deconv(const Geo<T>& g, const double* d, const YRef<T>& r, int j, T v) {
   if constexpr (sizeof(T) == 8) {
-    return v * (g.dc[g.ax.n + jy] * r.hi);
+    return v * (d[j] * r.hi);
   } else {
-    const float2 fy = __ldg(g.dcx2 + jy);
-    const float ph = fy.x * r.hi;
-    const float pe = fmaf(fy.x, r.hi, -ph) + fmaf(fy.x, r.lo, fy.y * r.hi);
+    const float2 f = __ldg(g.dcx2 + j);
+    const float ph = f.x * r.hi;
+    const float pe = fmaf(f.x, r.hi, -ph) + fmaf(f.x, r.lo, f.y * r.hi);
     return fmaf(v, ph, v * pe);
   }
+}
+
+// an element of the density: its deconvolved value, with a NaN / Inf recorded
+template <typename T>
+__device__ __forceinline__ cx_t<T> pad_value(const Geo<T>& g, const double* d, const YRef<T>& r, int j, T v) {
+  if (!isfinite(v) && *(volatile int*)g.nonfinite == 0) atomicOr(g.nonfinite, 1);
+  return cmk<cx_t<T>>(deconv<T>(g, d, r, j, v), (T)0);
 }
 
 template <typename T>
@@ -127,14 +142,15 @@ struct PadY : PolicyBase {
   const T* rho;
   __host__ __device__ long long nlines() const { return (long long)g.ax.n * g.az.n; }
   __device__ Ref ref(long long L) const { return y_ref<T>(g, L); }
+  __device__ void begin() const {
+    if (blockIdx.x == 0 && threadIdx.x < 2) g.counters[threadIdx.x] = 0;
+  }
   __device__ C load(const Ref& r, int i) const {
     const int jy = g.ay.grid_of(i);
-    const T v = __ldg(rho + r.grid + (long long)jy * g.ax.n);
-    if (!isfinite(v) && *(volatile int*)g.nonfinite == 0) atomicOr(g.nonfinite, 1);
-    return cmk<C>(deconv<T>(g, r, jy, v), (T)0);
+    return pad_value<T>(g, g.dc + g.ax.n, r, jy, __ldg(rho + (r.grid + jy * g.ax.n)));
   }
   __device__ void store(const Ref& r, int i, C v, Acc&) const {
-    if (g.in_yr(i)) g.fine[r.fine + (long long)i * g.ax.nf] = v;
+    if (g.in_yr(i)) g.fine[r.fine + i * g.ax.nf] = v;
   }
 };
 
@@ -151,16 +167,78 @@ struct CropY : PolicyBase {
   __device__ Ref ref(long long L) const { return y_ref<T>(g, L); }
   __device__ C load(const Ref& r, int i) const {
     if (!g.in_yr(i)) return cmk<C>((T)0, (T)0);
-    return __ldg(g.fine + r.fine + (long long)i * g.ax.nf);
+    return __ldg(g.fine + (r.fine + i * g.ax.nf));
   }
   __device__ void store(const Ref& r, int i, C v, Acc&) const {
     const int jy = g.ay.grid_of(i);
-    const T val = deconv<T>(g, r, jy, v.x);
-    T* at = phi + r.grid + (long long)jy * g.ax.n;
+    const T val = deconv<T>(g, g.dc + g.ax.n, r, jy, v.x);
+    T* at = phi + (r.grid + jy * g.ax.n);
     if (ACC)
       *at += val;
     else
       *at = val;
+  }
+};
+
+// 2D: x first and last, as rows of the density and the potential; y in between, storing or reading
+// only the y lines of the range.  (A pass's rounding noise is white along its own axis and follows
+// the spectrum along the axes transformed before it, and the 2D symbol grows like |k|^2 / |k|: with
+// y first the x noise of the rows near k_y = 0 met the symbol of a dipole tilted towards x, and the
+// error of a 256^2 density grew from 2.3e-6 to 3.9e-6.)
+template <typename T>
+__device__ __forceinline__ YRef<T> x_ref(const Geo<T>& g, long long L) {
+  return line_ref<T>((int)L * g.ax.n, g.ay.fine_of((int)L) * g.ax.nf, g.dc[g.ax.n + (int)L] * g.dc[g.ax.n + g.ay.n]);
+}
+
+template <typename T>
+struct PadX2 : PolicyBase {
+  using C = cx_t<T>;
+  using Ref = YRef<T>;
+  static constexpr bool kBlockIn = true, kStrided = false;
+  Geo<T> g;
+  const T* rho;
+  __host__ __device__ long long nlines() const { return g.ay.n; }
+  __device__ Ref ref(long long L) const { return x_ref<T>(g, L); }
+  __device__ void begin() const {
+    if (blockIdx.x == 0 && threadIdx.x < 2) g.counters[threadIdx.x] = 0;
+  }
+  __device__ C load(const Ref& r, int i) const {
+    const int jx = g.ax.grid_of(i);
+    return pad_value<T>(g, g.dc, r, jx, __ldg(rho + (r.grid + jx)));
+  }
+  __device__ void store(const Ref& r, int i, C v, Acc&) const { g.fine[r.fine + i] = v; }
+};
+
+template <typename T, bool FWD>
+struct ColY2 : PolicyBase {
+  using C = cx_t<T>;
+  using Ref = int;  // the column
+  static constexpr bool kBlockIn = FWD, kBlockOut = !FWD;
+  Geo<T> g;
+  __host__ __device__ long long nlines() const { return g.ax.nf; }
+  __device__ Ref ref(long long L) const { return (int)L; }
+  __device__ C load(Ref r, int i) const {
+    if (!FWD && !g.in_yr(i)) return cmk<C>((T)0, (T)0);
+    return __ldg(g.fine + (i * g.ax.nf + r));
+  }
+  __device__ void store(Ref r, int i, C v, Acc&) const {
+    if (!FWD || g.in_yr(i)) g.fine[i * g.ax.nf + r] = v;
+  }
+};
+
+template <typename T>
+struct CropX2 : PolicyBase {
+  using C = cx_t<T>;
+  using Ref = YRef<T>;
+  static constexpr bool kBlockOut = true, kStrided = false;
+  Geo<T> g;
+  T* phi;
+  __host__ __device__ long long nlines() const { return g.ay.n; }
+  __device__ Ref ref(long long L) const { return x_ref<T>(g, L); }
+  __device__ C load(const Ref& r, int i) const { return __ldg(g.fine + (r.fine + i)); }
+  __device__ void store(const Ref& r, int i, C v, Acc&) const {
+    const int jx = g.ax.grid_of(i);
+    phi[r.grid + jx] = deconv<T>(g, g.dc, r, jx, v.x);
   }
 };
 
@@ -169,19 +247,20 @@ struct CropY : PolicyBase {
 template <typename T, bool FWD>
 struct RowX : PolicyBase {
   using C = cx_t<T>;
-  using Ref = long long;  // fine-grid offset of the row
+  using Ref = int;  // fine-grid offset of the row
   static constexpr bool kBlockIn = FWD, kBlockOut = !FWD;
   Geo<T> g;
   __host__ __device__ long long nlines() const { return (long long)g.nyr * g.az.n; }
   static constexpr bool kStrided = false;
   __device__ Ref ref(long long L) const {
-    return g.fidx(g.az.fine_of((int)(L / g.nyr)), g.yr_line((int)(L % g.nyr)), 0);
+    const int q = (int)((unsigned)L / (unsigned)g.nyr);
+    return g.fidx(g.az.fine_of(q), g.yr_line((int)L - q * g.nyr), 0);
   }
   __device__ C load(Ref r, int i) const {
-    if (FWD) return __ldg(g.fine + r + g.ax.grid_of(i));
+    if (FWD) return __ldg(g.fine + (r + g.ax.grid_of(i)));
     // x lines outside the taps' range were neither written by the spread nor transformed
     if (!g.in_xr(i)) return cmk<C>((T)0, (T)0);
-    return __ldg(g.fine + r + i);
+    return __ldg(g.fine + (r + i));
   }
   __device__ void store(Ref r, int i, C v, Acc&) const {
     if (!FWD)
@@ -195,15 +274,16 @@ struct RowX : PolicyBase {
 template <typename T, bool FWD>
 struct ColZ : PolicyBase {
   using C = cx_t<T>;
-  using Ref = long long;  // the column's (y, x) offset
+  using Ref = int;  // the column's (y, x) offset
   static constexpr bool kBlockIn = FWD, kBlockOut = !FWD;
   Geo<T> g;
   __host__ __device__ long long nlines() const { return (long long)g.nxr * g.nyr; }
   __device__ Ref ref(long long L) const {
-    return (long long)g.yr_line((int)(L / g.nxr)) * g.ax.nf + g.xr_line((int)(L % g.nxr));
+    const int q = (int)((unsigned)L / (unsigned)g.nxr);
+    return g.yr_line(q) * g.ax.nf + g.xr_line((int)L - q * g.nxr);
   }
-  __device__ C load(Ref r, int i) const { return __ldg(g.fine + (long long)i * g.ay.nf * g.ax.nf + r); }
-  __device__ void store(Ref r, int i, C v, Acc&) const { g.fine[(long long)i * g.ay.nf * g.ax.nf + r] = v; }
+  __device__ C load(Ref r, int i) const { return __ldg(g.fine + (i * g.sz + r)); }
+  __device__ void store(Ref r, int i, C v, Acc&) const { g.fine[i * g.sz + r] = v; }
 };
 
 // The smooth symbol of the split algorithm (Eq. 3.9) at the fine grid's modes,
@@ -241,7 +321,7 @@ struct SmoothSymbol {
 // transform sums the two modes).
 template <typename T>
 struct ZRef {
-  long long col;  // the column's (y, x) offset
+  int col;        // the column's (y, x) offset
   T kx, ky;       // the column's x and y wavenumbers
   T em;           // e^{-(kx^2 + ky^2)/k0^2} - 1
   T w;            // 1 or 2
@@ -257,12 +337,12 @@ struct SmoothZ : PolicyBase {
   SmoothSymbol<T> sy;
   __host__ __device__ long long nlines() const { return (long long)g.ax.nf * g.nyr; }
   __device__ Ref ref(long long L) const {
-    const int lx = (int)(L % g.ax.nf), ly = (int)(L / g.ax.nf);
+    const int ly = (int)((unsigned)L / (unsigned)g.ax.nf), lx = (int)L - ly * g.ax.nf;
     const bool twice = ly > 0 && 2 * ly < g.ay.nf;
-    return Ref{(long long)ly * g.ax.nf + lx, sy.k_of(0, lx, g.ax.nf), sy.k_of(1, ly, g.ay.nf),
+    return Ref{ly * g.ax.nf + lx, sy.k_of(0, lx, g.ax.nf), sy.k_of(1, ly, g.ay.nf),
                sy.join(sy.em1[lx], sy.em1[g.ax.nf + ly]), (T)(twice ? 2 : 1), twice && 2 * lx == g.ax.nf};
   }
-  __device__ C load(const Ref& r, int i) const { return __ldg(g.fine + (long long)i * g.ay.nf * g.ax.nf + r.col); }
+  __device__ C load(const Ref& r, int i) const { return __ldg(g.fine + (i * g.sz + r.col)); }
   __device__ C apply(const Ref& r, int i, C v) const {
     const T kz = sy.k_of(2, i, g.az.nf);
     const T em = sy.join(r.em, __ldg(sy.em1 + g.ax.nf + g.ay.nf + i));
@@ -272,7 +352,7 @@ struct SmoothZ : PolicyBase {
     return cscale(v, p);
   }
   __device__ void store(const Ref& r, int i, C v, Acc&) const {
-    g.fine[(long long)i * g.ay.nf * g.ax.nf + r.col] = v;
+    g.fine[i * g.sz + r.col] = v;
   }
 };
 
@@ -288,6 +368,8 @@ Geo<T> geo_of(Plan& p, bool unit = false) {
   g.xlo = unit ? 0 : p.xr[0];
   g.nxr = unit ? p.nf[0] : p.xr[1];
   g.nonfinite = p.d_nonfinite;
+  g.sz = p.nf[0] * p.nf[1];
+  g.counters = p.d_counter;
   g.dc = static_cast<const double*>(unit ? p.d_ones : p.d_deconv);
   g.dcx2 = static_cast<const float2*>(unit ? p.d_ones_x2 : p.d_deconv_x2);
   g.fine = static_cast<cx_t<T>*>(p.d_fine);
@@ -304,9 +386,9 @@ struct Precise : P {
 template <typename T, int DIR, int HI, typename P>
 int pass(Plan& p, int n, const P& pol, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
-    if (p.precise_nufft) return dispatch_policy<T, DIR, 16, HI>(n, Precise<P>{pol}, twiddles(p, n), s);
+    if (p.precise_nufft) return dispatch_policy<T, DIR, 16, HI>(p, n, Precise<P>{pol}, s);
   }
-  return dispatch_policy<T, DIR, 16, HI>(n, pol, twiddles(p, n), s);
+  return dispatch_policy<T, DIR, 16, HI>(p, n, pol, s);
 }
 
 }  // namespace
@@ -314,30 +396,40 @@ int pass(Plan& p, int n, const P& pol, cudaStream_t s) {
 template <typename T>
 int nufft_forward_fft(Plan& p, const T* rho, cudaStream_t s) {
   const Geo<T> g = geo_of<T>(p);
-  DDI_TRY((pass<T, -1, 2048>(p, p.nf[1], PadY<T>{{}, g, rho}, s)));
-  p.mark("pad_fft_y", s);
-  DDI_TRY((pass<T, -1, 2048>(p, p.nf[0], RowX<T, true>{{}, g}, s)));
-  p.mark("fft_x_fwd", s);
-  if (p.dim == 3) {
-    DDI_TRY((pass<T, -1, 1024>(p, p.nf[2], ColZ<T, true>{{}, g}, s)));
-    p.mark("fft_z_fwd", s);
+  if (p.dim == 2) {
+    DDI_TRY((pass<T, -1, 2048>(p, p.nf[0], PadX2<T>{{}, g, rho}, s)));
+    p.mark("pad_fft_x", s);
+    DDI_TRY((pass<T, -1, 2048>(p, p.nf[1], ColY2<T, true>{{}, g}, s)));
+    p.mark("fft_y_fwd", s);
+    return DDI_OK;
   }
+  DDI_TRY((pass<T, -1, 1024>(p, p.nf[1], PadY<T>{{}, g, rho}, s)));
+  p.mark("pad_fft_y", s);
+  DDI_TRY((pass<T, -1, 1024>(p, p.nf[0], RowX<T, true>{{}, g}, s)));
+  p.mark("fft_x_fwd", s);
+  DDI_TRY((pass<T, -1, 1024>(p, p.nf[2], ColZ<T, true>{{}, g}, s)));
+  p.mark("fft_z_fwd", s);
   return DDI_OK;
 }
 
 template <typename T>
 int nufft_inverse_fft(Plan& p, T* phi, cudaStream_t s, bool acc) {
   const Geo<T> g = geo_of<T>(p);
-  if (p.dim == 3) {
-    DDI_TRY((pass<T, +1, 1024>(p, p.nf[2], ColZ<T, false>{{}, g}, s)));
-    p.mark("fft_z_inv", s);
+  if (p.dim == 2) {
+    DDI_TRY((pass<T, +1, 2048>(p, p.nf[1], ColY2<T, false>{{}, g}, s)));
+    p.mark("fft_y_inv", s);
+    DDI_TRY((pass<T, +1, 2048>(p, p.nf[0], CropX2<T>{{}, g, phi}, s)));
+    p.mark("fft_x_inv_crop", s);
+    return DDI_OK;
   }
-  DDI_TRY((pass<T, +1, 2048>(p, p.nf[0], RowX<T, false>{{}, g}, s)));
+  DDI_TRY((pass<T, +1, 1024>(p, p.nf[2], ColZ<T, false>{{}, g}, s)));
+  p.mark("fft_z_inv", s);
+  DDI_TRY((pass<T, +1, 1024>(p, p.nf[0], RowX<T, false>{{}, g}, s)));
   p.mark("fft_x_inv", s);
   if (acc)
     DDI_TRY((pass<T, +1, 1024>(p, p.nf[1], CropY<T, true>{{}, g, phi}, s)));
   else
-    DDI_TRY((pass<T, +1, 2048>(p, p.nf[1], CropY<T, false>{{}, g, phi}, s)));
+    DDI_TRY((pass<T, +1, 1024>(p, p.nf[1], CropY<T, false>{{}, g, phi}, s)));
   p.mark(acc ? "fft_y_inv_crop_add" : "fft_y_inv_crop", s);
   return DDI_OK;
 }
@@ -365,15 +457,15 @@ int split_smooth_part(Plan& p, const T* rho, T* phi, cudaStream_t s) {
   sy.inv_k02 = (T)(1.0 / (p.desc.split_k0 * p.desc.split_k0));
   sy.em1 = static_cast<const T*>(p.d_em1);
   sy.scale = (T)(1.0 / ((double)p.nf[0] * (double)p.nf[1] * (double)p.nf[2]));
-  DDI_TRY((dispatch_policy<T, -1, 16, 2048>(p.nf[1], PadY<T>{{}, g, rho}, twiddles(p, p.nf[1]), s)));
+  DDI_TRY((dispatch_policy<T, -1, 16, 1024>(p, p.nf[1], PadY<T>{{}, g, rho}, s)));
   p.mark("smooth_pad_fft_y", s);
-  DDI_TRY((dispatch_policy<T, -1, 16, 2048>(p.nf[0], RowX<T, true>{{}, g}, twiddles(p, p.nf[0]), s)));
+  DDI_TRY((dispatch_policy<T, -1, 16, 1024>(p, p.nf[0], RowX<T, true>{{}, g}, s)));
   p.mark("smooth_fft_x_fwd", s);
-  DDI_TRY((dispatch_policy<T, 0, 16, 1024>(p.nf[2], SmoothZ<T>{{}, g, sy}, twiddles(p, p.nf[2]), s)));
+  DDI_TRY((dispatch_policy<T, 0, 16, 1024>(p, p.nf[2], SmoothZ<T>{{}, g, sy}, s)));
   p.mark("smooth_fft_z_pair", s);
-  DDI_TRY((dispatch_policy<T, +1, 16, 2048>(p.nf[0], RowX<T, false>{{}, g}, twiddles(p, p.nf[0]), s)));
+  DDI_TRY((dispatch_policy<T, +1, 16, 1024>(p, p.nf[0], RowX<T, false>{{}, g}, s)));
   p.mark("smooth_fft_x_inv", s);
-  DDI_TRY((dispatch_policy<T, +1, 16, 2048>(p.nf[1], CropY<T, false>{{}, g, phi}, twiddles(p, p.nf[1]), s)));
+  DDI_TRY((dispatch_policy<T, +1, 16, 1024>(p, p.nf[1], CropY<T, false>{{}, g, phi}, s)));
   p.mark("smooth_fft_y_inv_crop", s);
   return DDI_OK;
 }

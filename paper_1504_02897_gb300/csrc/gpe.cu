@@ -86,6 +86,8 @@ __global__ void k_phase_tables(cx_t<T>* tab, G3 g, double f0, double f1) {
 
 template <typename T>
 __global__ void k_abs2(const cx_t<T>* __restrict__ psi, T* __restrict__ rho, long long total) {
+  chain_release();
+  chain_wait();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     const cx_t<T> v = psi[i];
@@ -121,6 +123,8 @@ __device__ __forceinline__ T expm1t(T a) {
 template <typename T>
 __global__ void k_step_density(const cx_t<T>* __restrict__ psi, T* __restrict__ gout, NonlinParams nl, T dt,
                                long long total) {
+  chain_release();
+  chain_wait();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     const cx_t<T> v = psi[i];
@@ -147,6 +151,8 @@ __global__ void k_step_density(const cx_t<T>* __restrict__ psi, T* __restrict__ 
 template <typename T>
 __global__ void k_nonlinear_general(cx_t<T>* __restrict__ psi, const T* __restrict__ V, const T* __restrict__ phig,
                                     T beta, T lam, T dt, NonlinParams nl, long long total) {
+  chain_release();
+  chain_wait();
   using C = cx_t<T>;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -182,6 +188,8 @@ __global__ void k_nonlinear_general(cx_t<T>* __restrict__ psi, const T* __restri
 template <typename T>
 __global__ void k_nonlinear(cx_t<T>* __restrict__ psi, const T* __restrict__ V, const T* __restrict__ phi, T beta,
                             T lam, T dt, long long total) {
+  chain_release();
+  chain_wait();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     const cx_t<T> v = psi[i];
@@ -335,6 +343,8 @@ template <typename T>
 __global__ void k_adj_a(const cx_t<T>* __restrict__ psi1, const T* __restrict__ V, const T* rho,
                         const T* __restrict__ phi, cx_t<T>* __restrict__ cot, T* __restrict__ grad,
                         T* rout, T beta, T lam, T dt, T dv, long long total) {
+  chain_release();
+  chain_wait();
   using C = cx_t<T>;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -355,6 +365,8 @@ __global__ void k_adj_a(const cx_t<T>* __restrict__ psi1, const T* __restrict__ 
 template <typename T>
 __global__ void k_adj_b(const cx_t<T>* __restrict__ psi1, const T* __restrict__ r, const T* __restrict__ phir,
                         cx_t<T>* __restrict__ cot, T beta, T lam, long long total) {
+  chain_release();
+  chain_wait();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     const T sfield = (T)2 * (beta * r[i] + (phir ? lam * phir[i] : (T)0));
@@ -418,8 +430,7 @@ struct Gpe {
   }
 
   int abs2(const C* a, T* out) {
-    k_abs2<T><<<blocks_for(N), kThreads, 0, s>>>(a, out, N);
-    DDI_LAUNCH_CHECK();
+    DDI_TRY(launch_chain(p, k_abs2<T>, blocks_for(N), kThreads, 0, s, a, out, N));
     return DDI_OK;
   }
 
@@ -507,8 +518,7 @@ struct Gpe {
       } else {
         DDI_CUDA(cudaMemsetAsync(phi, 0, sizeof(T) * N, s));
       }
-      k_nonlinear<T><<<blocks_for(N), kThreads, 0, s>>>(psi, V, phi, (T)beta, (T)lam, (T)dt, N);
-      DDI_LAUNCH_CHECK();
+      DDI_TRY(launch_chain(p, k_nonlinear<T>, blocks_for(N), kThreads, 0, s, psi, V, phi, (T)beta, (T)lam, (T)dt, N));
       const bool more = k + 1 < nsteps;
       DDI_TRY(kinetic(psi, more ? 1 : 0, more ? rho : nullptr));
     }
@@ -522,15 +532,13 @@ struct Gpe {
     DDI_TRY(phase_tables(-0.25 * dt, -0.5 * dt));
     DDI_TRY(kinetic(psi, 0));
     for (int k = 0; k < nsteps; ++k) {
-      k_step_density<T><<<blocks_for(N), kThreads, 0, s>>>(psi, g, nl, (T)dt, N);
-      DDI_LAUNCH_CHECK();
+      DDI_TRY(launch_chain(p, k_step_density<T>, blocks_for(N), kThreads, 0, s, psi, g, nl, (T)dt, N));
       if (lam != 0.0) {
         DDI_TRY(run_ddi<T>(p, g, phi, s));
       } else {
         DDI_CUDA(cudaMemsetAsync(phi, 0, sizeof(T) * N, s));
       }
-      k_nonlinear_general<T><<<blocks_for(N), kThreads, 0, s>>>(psi, V, phi, (T)beta, (T)lam, (T)dt, nl, N);
-      DDI_LAUNCH_CHECK();
+      DDI_TRY(launch_chain(p, k_nonlinear_general<T>, blocks_for(N), kThreads, 0, s, psi, V, phi, (T)beta, (T)lam, (T)dt, nl, N));
       DDI_TRY(kinetic(psi, k + 1 < nsteps ? 1 : 0));
     }
     return DDI_OK;
@@ -607,12 +615,9 @@ struct Gpe {
       DDI_CUDA(cudaMemsetAsync(phi, 0, sizeof(T) * N, s));
     }
     DDI_TRY(kinetic(cot, 1));
-    k_adj_a<T><<<blocks_for(N), kThreads, 0, s>>>(psi1, V, rho, phi, cot, grad, rho, (T)beta, (T)lam, (T)dt,
-                                                  (T)p.dv, N);
-    DDI_LAUNCH_CHECK();
+    DDI_TRY(launch_chain(p, k_adj_a<T>, blocks_for(N), kThreads, 0, s, psi1, V, rho, phi, cot, grad, rho, (T)beta, (T)lam, (T)dt, (T)p.dv, N));
     if (lam != 0.0) DDI_TRY(run_ddi<T>(p, rho, phi, s));
-    k_adj_b<T><<<blocks_for(N), kThreads, 0, s>>>(psi1, rho, lam != 0.0 ? phi : nullptr, cot, (T)beta, (T)lam, N);
-    DDI_LAUNCH_CHECK();
+    DDI_TRY(launch_chain(p, k_adj_b<T>, blocks_for(N), kThreads, 0, s, psi1, rho, lam != 0.0 ? phi : nullptr, cot, (T)beta, (T)lam, N));
     return kinetic(cot, 1);
   }
 

@@ -39,14 +39,14 @@ struct GpePolicy : PolicyBase {
 template <typename T, bool RHO>
 struct GridX : GpePolicy {
   using C = cx_t<T>;
-  using Ref = long long;
+  using Ref = int;  // grids hold < 2^31 points
   C* data;
   T* rho;
   GridDims3 d;
   __host__ __device__ long long nlines() const { return (long long)d.n[1] * d.n[2]; }
   static constexpr bool kStrided = false;
-  __device__ Ref ref(long long L) const { return L * d.n[0]; }
-  __device__ C load(Ref r, int i) const { return __ldg(data + r + i); }
+  __device__ Ref ref(long long L) const { return (int)L * d.n[0]; }
+  __device__ C load(Ref r, int i) const { return __ldg(data + (r + i)); }
   __device__ void store(Ref r, int i, C v, Acc&) const {
     data[r + i] = v;
     if (RHO) rho[r + i] = v.x * v.x + v.y * v.y;
@@ -57,16 +57,17 @@ struct GridX : GpePolicy {
 template <typename T>
 struct GridLines : GpePolicy {
   using C = cx_t<T>;
-  using Ref = long long;
+  using Ref = int;  // grids hold < 2^31 points
   C* data;
   GridDims3 d;
   int axis;
   __host__ __device__ long long nlines() const { return (long long)d.n[0] * (axis == 1 ? d.n[2] : d.n[1]); }
   __device__ Ref ref(long long L) const {
-    if (axis == 2) return L;
-    return (L / d.n[0]) * ((long long)d.n[0] * d.n[1]) + L % d.n[0];
+    if (axis == 2) return (int)L;
+    const int q = (int)((unsigned)L / (unsigned)d.n[0]);
+    return q * d.n[0] * d.n[1] + ((int)L - q * d.n[0]);
   }
-  __device__ long long at(Ref r, int i) const { return r + (long long)i * (axis == 1 ? d.n[0] : (long long)d.n[0] * d.n[1]); }
+  __device__ int at(Ref r, int i) const { return r + i * (axis == 1 ? d.n[0] : d.n[0] * d.n[1]); }
   __device__ C load(Ref r, int i) const { return __ldg(data + at(r, i)); }
   __device__ void store(Ref r, int i, C v, Acc&) const { data[at(r, i)] = v; }
 };
@@ -75,7 +76,7 @@ struct GridLines : GpePolicy {
 // per-axis tables of e - 1, combined as (1+A)(1+B)(1+C) - 1 = P + C + C P with P = A + B + A B
 template <typename T>
 struct KineticRef {
-  long long off;
+  int off;
   cx_t<T> P;  // the other axes' factor minus 1
 };
 template <typename T>
@@ -90,7 +91,7 @@ struct KineticPair : GridLines<T> {
     const C A = tab[x];
     if (this->axis == 1) return Ref{GridLines<T>::ref(L), A};
     const C B = tab[this->d.n[0] + (int)(L / this->d.n[0])];
-    return Ref{L, cadd(cadd(A, B), cmul(A, B))};
+    return Ref{(int)L, cadd(cadd(A, B), cmul(A, B))};
   }
   __device__ C load(const Ref& r, int i) const { return GridLines<T>::load(r.off, i); }
   __device__ C apply(const Ref& r, int i, C v) const {
@@ -115,7 +116,7 @@ struct GfSkip {
 template <typename T>
 struct GfRhsX : GpePolicy {
   using C = cx_t<T>;
-  using Ref = long long;
+  using Ref = int;  // grids hold < 2^31 points
   const C *phi, *cur;
   C* out;
   const T *V, *rho, *dip;
@@ -125,7 +126,7 @@ struct GfRhsX : GpePolicy {
   __host__ __device__ long long nlines() const { return (long long)d.n[1] * d.n[2]; }
   __device__ bool skip() const { return sk.done(); }
   static constexpr bool kStrided = false;
-  __device__ Ref ref(long long L) const { return L * d.n[0]; }
+  __device__ Ref ref(long long L) const { return (int)L * d.n[0]; }
   __device__ C load(Ref r, int i) const {
     const T w = V[r + i] + beta * rho[r + i] + (dip ? lam * dip[r + i] : (T)0);
     const T f = alpha - w;
@@ -145,7 +146,7 @@ struct GfLines : GridLines<T> {
 // precision: the fixed point's own tolerance is the plan's)
 template <typename T>
 struct GfSolveRef {
-  long long off;
+  int off;
   T m2;
 };
 template <typename T>
@@ -181,7 +182,7 @@ struct GfSolvePair : GridLines<T> {
 template <typename T>
 struct GfChangeX : GpePolicy {
   using C = cx_t<T>;
-  using Ref = long long;
+  using Ref = int;  // grids hold < 2^31 points
   struct Acc {
     T m;
   };
@@ -193,8 +194,8 @@ struct GfChangeX : GpePolicy {
   __host__ __device__ long long nlines() const { return (long long)d.n[1] * d.n[2]; }
   __device__ bool skip() const { return sk.done(); }
   static constexpr bool kStrided = false;
-  __device__ Ref ref(long long L) const { return L * d.n[0]; }
-  __device__ C load(Ref r, int i) const { return __ldg(data + r + i); }
+  __device__ Ref ref(long long L) const { return (int)L * d.n[0]; }
+  __device__ C load(Ref r, int i) const { return __ldg(data + (r + i)); }
   __device__ void store(Ref r, int i, C v, Acc& a) const {
     data[r + i] = v;
     const C y = cur[r + i];
@@ -225,7 +226,7 @@ struct GfChangeX : GpePolicy {
 
 template <typename T, int DIR, typename P>
 int grid_pass(const Plan& p, int axis, const P& pol, cudaStream_t s) {
-  return dispatch_policy<T, DIR, 8, 1024>(p.n[axis], pol, twiddles(p, p.n[axis]), s);
+  return dispatch_policy<T, DIR, 8, 1024>(p, p.n[axis], pol, s);
 }
 GridDims3 grid_dims(const Plan& p) { return GridDims3{{p.n[0], p.n[1], p.n[2]}}; }
 

@@ -98,12 +98,14 @@ __device__ __forceinline__ void load_taps(const T* __restrict__ src, T (&dst)[W]
 // accumulate the psi_y (and psi_z) weighted sums in registers, and the node's value is
 // the psi_x-weighted sum over its lanes (shuffle reduction).
 // (at most 64 registers in FP32, so that 4 CTAs per SM keep enough loads in flight)
-template <typename T, int W, int DIM>
+template <typename T, int W>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
     k_interp(const cx_t<T>* __restrict__ fine, const ushort4* __restrict__ l0, const T* __restrict__ psi,
              const T* __restrict__ scale, cx_t<T>* __restrict__ cout, long long count, GridDims g) {
   using C = cx_t<T>;
   constexpr int XL = W <= 8 ? 8 : 16;
+  chain_release();
+  chain_wait();
   const int lane = threadIdx.x & 31;
   const int rx = lane % XL;
   const long long i0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / XL;
@@ -113,7 +115,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
   const T* ps = psi + i * 3 * W;
   T ky[W], kz[W];
   load_taps<T, W>(ps + W, ky);
-  if (DIM == 3) load_taps<T, W>(ps + 2 * W, kz);
+  load_taps<T, W>(ps + 2 * W, kz);
   const bool on = rx < W;
   const T kx = on ? __ldg(ps + rx) : (T)0;
   const int xx = wrap1(s.x + (on ? rx : 0), g.nf[0]);
@@ -121,28 +123,19 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
 #pragma unroll
   for (int ay = 0; ay < W; ++ay) yoff[ay] = wrap1(s.y + ay, g.nf[1]) * g.nf[0];
   T ar = 0, ai = 0;
-  if (DIM == 3) {
-    const long long plane = (long long)g.nf[1] * g.nf[0];
+  const long long plane = (long long)g.nf[1] * g.nf[0];
 #pragma unroll
-    for (int az = 0; az < W; ++az) {
-      const C* zp = fine + wrap1(s.z + az, g.nf[2]) * plane + xx;
-      T zr = 0, zi = 0;
-#pragma unroll
-      for (int ay = 0; ay < W; ++ay) {
-        const C v = __ldg(zp + yoff[ay]);
-        zr += ky[ay] * v.x;
-        zi += ky[ay] * v.y;
-      }
-      ar += kz[az] * zr;
-      ai += kz[az] * zi;
-    }
-  } else {
+  for (int az = 0; az < W; ++az) {
+    const C* zp = fine + wrap1(s.z + az, g.nf[2]) * plane + xx;
+    T zr = 0, zi = 0;
 #pragma unroll
     for (int ay = 0; ay < W; ++ay) {
-      const C v = __ldg(fine + xx + yoff[ay]);
-      ar += ky[ay] * v.x;
-      ai += ky[ay] * v.y;
+      const C v = __ldg(zp + yoff[ay]);
+      zr += ky[ay] * v.x;
+      zi += ky[ay] * v.y;
     }
+    ar += kz[az] * zr;
+    ai += kz[az] * zi;
   }
   ar *= kx;
   ai *= kx;
@@ -154,6 +147,63 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
   if (rx == 0 && valid) {
     const T sc = scale[i];
     cout[i] = cmk<C>(sc * ar, sc * ai);
+  }
+}
+
+// 2D interpolation: as k_interp, but a lane group walks over nodes and requests the next node's taps
+// and kernel values before it gathers for the current one.  With 64 taps a node the gather kernel was
+// latency-bound: the node's data from memory, then its taps, once per thread (1024^2 143 -> 107 us).
+template <typename T, int W>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
+    k_interp2(const cx_t<T>* __restrict__ fine, const ushort4* __restrict__ l0, const T* __restrict__ psi,
+              const T* __restrict__ scale, cx_t<T>* __restrict__ cout, int count, GridDims g) {
+  using C = cx_t<T>;
+  constexpr int XL = W <= 8 ? 8 : 16;
+  chain_release();
+  chain_wait();
+  const int rx = threadIdx.x % XL;
+  const bool on = rx < W;
+  const int groups = (int)(gridDim.x * blockDim.x) / XL;
+  const int first = (int)(blockIdx.x * blockDim.x + threadIdx.x) / XL;
+  ushort4 sn;
+  T kyn[W], kxn, scn;
+  auto request = [&](int i) {
+    const int q = i < count ? i : count - 1;  // lanes past the end work on a copy of the last node
+    sn = __ldg(l0 + q);
+    const T* ps = psi + (size_t)q * 3 * W;
+    load_taps<T, W>(ps + W, kyn);
+    kxn = on ? __ldg(ps + rx) : (T)0;
+    scn = __ldg(scale + q);
+  };
+  request(first);
+  // every lane of the block makes the same number of turns (the shuffles are of whole warps)
+  const int turns = (count - (int)(blockIdx.x * (blockDim.x / XL)) + groups - 1) / groups;
+  for (int k = 0; k < turns; ++k) {
+    const int i = first + k * groups;
+    const ushort4 s = sn;
+    const T kx = kxn, sc = scn;
+    T ky[W];
+#pragma unroll
+    for (int a = 0; a < W; ++a) ky[a] = kyn[a];
+    const C* at = fine + wrap1(s.x + (on ? rx : 0), g.nf[0]);
+    C v[W];
+#pragma unroll
+    for (int a = 0; a < W; ++a) v[a] = __ldg(at + wrap1(s.y + a, g.nf[1]) * g.nf[0]);
+    if (k + 1 < turns) request(i + groups);
+    T ar = 0, ai = 0;
+#pragma unroll
+    for (int a = 0; a < W; ++a) {
+      ar += ky[a] * v[a].x;
+      ai += ky[a] * v[a].y;
+    }
+    ar *= kx;
+    ai *= kx;
+#pragma unroll
+    for (int o = XL / 2; o > 0; o >>= 1) {
+      ar += __shfl_xor_sync(0xffffffffu, ar, o);
+      ai += __shfl_xor_sync(0xffffffffu, ai, o);
+    }
+    if (rx == 0 && i < count) cout[i] = cmk<C>(sc * ar, sc * ai);
   }
 }
 
@@ -213,6 +263,8 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
   using S = WarpStage<T, W>;
   constexpr int XL = S::XL, RL = S::RL, MR = S::MR;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_release();
+  chain_wait();
   const int TX = a.tile[0], TY = a.tile[1], TZ = a.tile[2];
   const int RS = spread_row_stride(TX);
   const int PSZ = TY * RS;
@@ -397,243 +449,8 @@ __global__ void __launch_bounds__(256)
   fine[((long long)gz * g.nf[1] + gy) * g.nf[0] + gx] = cmk<C>(sr, si);
 }
 
-// ---- 2D column spreading (type 1, FP32 2D; the 3D column spread is in columns.cu) ------------------
-constexpr int kColThreads = 128;  // 4 warps per CTA, each taking units on its own
-
-struct ColArgs {
-  int nf[3];
-  int ncx;
-  const ColUnit* units;
-  int nunits;
-  int* counter;
-  const int2* visits;
-  const float2* c;
-  const float* psi;  // [node][3][w]
-  float2* fine;
-  float2* partial;        // [slot][kColX]
-  const int* unit_slots;  // per unit: the partial slot of each leading, then trailing row
-};
-
-#define DDI_COL_CASES(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15)
-
-// 2D column spread.  A column is kColX cells of x and every y line (the window axis).  Lane
-// (lx, g) holds cell lx of the column for the W rows of the window (row r in register
-// r mod W, as in 3D); the four lane groups g take different visits of one run (the visits
-// with the same first y tap, which all start at the window's first row) and their sums for
-// a row are added by two shuffles, in a fixed order, when the row leaves the window.  Staged
-// per visit: psi_x in a zero-padded row (as in 3D), psi_y rotated so that register k reads
-// its tap at index k and doubled for packed FMAs, c_q and the first y tap.
-template <int W, int NS>
-struct alignas(16) ColStage2 {
-  static constexpr int PY = ((2 * W + 7) / 8) * 8 + 4;   // psi_y rotated, each value twice, padding
-  static constexpr int PX = ((W + 15 + 7) / 8) * 8 + 4;  // psi_x at [8, 8 + W)
-  float py[NS][PY];
-  float px[NS][PX];
-  int4 hd[NS];  // byte offset of px[j][8 - ox]; 0; c_q (two floats)
-  int sz[NS];   // first y tap
-};
-
-template <int W, int NS>
-__global__ void __launch_bounds__(kColThreads) k_spread_col2(ColArgs a) {
-  using S = ColStage2<W, NS>;
-  static_assert(W <= 16 && W % 2 == 0, "rows 0..15 of the window, psi_y read in pairs of taps");
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  S* st = reinterpret_cast<S*>(smem_raw) + warp;
-  const int lx = lane & 7, g = lane >> 3;
-  const int lx4 = 4 * lx;
-  const int nfx = a.nf[0], nfy = a.nf[1];
-  const unsigned st_off = (unsigned)(reinterpret_cast<unsigned char*>(st) - smem_raw);
-  for (int i = lane; i < NS * S::PX; i += 32) (&st->px[0][0])[i] = 0.f;
-  __syncwarp();
-  for (;;) {
-    int u = 0;
-    if (lane == 0) u = atomicAdd(a.counter, 1);
-    u = __shfl_sync(0xffffffffu, u, 0);
-    if (u >= a.nunits) break;
-    const ColUnit U = a.units[u];
-    const int x = U.col * kColX + lx;
-    const int zpart_hi = U.z1 - U.phi;
-    float2 acc[W];
-#pragma unroll
-    for (int k = 0; k < W; ++k) acc[k] = make_float2(0.f, 0.f);
-    int zb = U.z0;
-    // row zb leaves the window: the four groups' sums added ((g0 + g1) + (g2 + g3)), written by
-    // group 0 (direct, or to a partial slot when other units touch the row)
-    auto flush = [&]() {
-      float2 v = make_float2(0.f, 0.f);
-      switch (zb % W) {
-#define DDI_TAKE(R)                          \
-  case R:                                    \
-    if constexpr (R < W) {                   \
-      v = acc[R];                            \
-      acc[R] = make_float2(0.f, 0.f);        \
-    }                                        \
-    break;
-        DDI_COL_CASES(DDI_TAKE)
-#undef DDI_TAKE
-      }
-      v.x += __shfl_xor_sync(0xffffffffu, v.x, 8);
-      v.y += __shfl_xor_sync(0xffffffffu, v.y, 8);
-      v.x += __shfl_xor_sync(0xffffffffu, v.x, 16);
-      v.y += __shfl_xor_sync(0xffffffffu, v.y, 16);
-      if (g == 0) {
-        const int r = zb - U.z0;
-        if (r < U.plo || zb >= zpart_hi) {
-          const int k = r < U.plo ? r : U.plo + (zb - zpart_hi);
-          a.partial[(size_t)__ldg(a.unit_slots + U.slot0 + k) * kColX + lx] = v;
-        } else {
-          __stcs(a.fine + (long long)(zb >= nfy ? zb - nfy : zb) * nfx + x, v);
-        }
-      }
-      ++zb;
-    };
-    for (int kb = U.lo; kb < U.hi; kb += NS) {
-      const int cnt = min(NS, U.hi - kb);
-      bool run_start = false;
-      if (lane < cnt) {
-        const int2 v = a.visits[kb + lane];
-        run_start = (v.y >> 12) & 1;
-        const float* ps = a.psi + (size_t)v.x * 3 * W;
-        {
-          float t[W];
-          load_taps<float, W>(ps, t);
-#pragma unroll
-          for (int k = 0; k < W; ++k) st->px[lane][8 + k] = t[k];
-        }
-        const int sy = v.y >> 13;
-        {
-          float t[W];
-          load_taps<float, W>(ps + W, t);
-          float2* pyr = reinterpret_cast<float2*>(st->py[lane]);
-          const int rot = sy % W;  // tap dy feeds row s + dy, held in register (s + dy) mod W
-#pragma unroll
-          for (int k = 0; k < W; ++k) {
-            const int q = rot + k < W ? rot + k : rot + k - W;
-            pyr[q] = make_float2(t[k], t[k]);
-          }
-        }
-        const float2 cq = __ldg(a.c + v.x);
-        const int ox = (v.y & 63) - 16;
-        const unsigned pxo = st_off + (unsigned)(offsetof(S, px) + (lane * S::PX + 8 - ox) * sizeof(float));
-        st->hd[lane] = make_int4((int)pxo, 0, __float_as_int(cq.x), __float_as_int(cq.y));
-        st->sz[lane] = sy;
-      }
-      // runs of one first y tap (bit j set where staged visit j starts one; visit 0 always
-      // starts the batch's first run)
-      unsigned starts = __ballot_sync(0xffffffffu, run_start) | 1u;
-      __syncwarp();
-      while (starts) {
-        const int j0 = __ffs(starts) - 1;
-        starts &= starts - 1;
-        const int j1 = starts ? __ffs(starts) - 1 : cnt;
-        const int sr = st->sz[j0];
-        while (zb < sr) flush();
-        for (int j = j0 + g; j < j1; j += 4) {
-          const int4 h = st->hd[j];
-          const float wx = *reinterpret_cast<const float*>(smem_raw + h.x + lx4);
-          const float2 cw = make_float2(wx * __int_as_float(h.z), wx * __int_as_float(h.w));
-          const float4* p4 = reinterpret_cast<const float4*>(st->py[j]);
-#pragma unroll
-          for (int k = 0; k < W / 2; ++k) {
-            const float4 q = p4[k];
-            acc[2 * k] = __ffma2_rn(cw, make_float2(q.x, q.y), acc[2 * k]);
-            acc[2 * k + 1] = __ffma2_rn(cw, make_float2(q.z, q.w), acc[2 * k + 1]);
-          }
-        }
-      }
-      __syncwarp();
-    }
-    while (zb < U.z1) flush();
-  }
-}
-
-// 2D rows that several column units touch: eight lanes per entry (one per cell), the entry's
-// partial slots summed in slot order (deterministic), eight loads in flight at a time.
-__global__ void __launch_bounds__(256)
-    k_reduce_col2(const ColRed* __restrict__ red, int nred, const float2* __restrict__ partial,
-                  float2* __restrict__ fine, int nfx) {
-  const int e = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 3);
-  if (e >= nred) return;
-  const int lx = threadIdx.x & 7;
-  const int4 r = __ldg(reinterpret_cast<const int4*>(red) + e);  // col, row, s0, ns
-  const float2* src = partial + (size_t)r.z * kColX + lx;
-  float2 sum = make_float2(0.f, 0.f);
-  int k = 0;
-  for (; k + 8 <= r.w; k += 8) {
-    float2 v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = __ldcs(src + (size_t)(k + q) * kColX);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      sum.x += v[q].x;
-      sum.y += v[q].y;
-    }
-  }
-  for (; k < r.w; ++k) {
-    const float2 v = __ldcs(src + (size_t)k * kColX);
-    sum.x += v.x;
-    sum.y += v.y;
-  }
-  fine[(long long)r.y * nfx + r.x * kColX + lx] = sum;
-}
-
-template <int W, int NS>
-int configure_spread_col2(Plan& p) {
-  constexpr size_t smem = sizeof(ColStage2<W, NS>) * (kColThreads / 32);
-  auto kern = k_spread_col2<W, NS>;
-  {
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lock(mu);
-    cudaFuncAttributes fa;
-    DDI_CUDA(cudaFuncGetAttributes(&fa, kern));
-    if ((size_t)fa.maxDynamicSharedSizeBytes < smem)
-      DDI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  }
-  int per_sm = 0;
-  DDI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kColThreads, smem));
-  int sms = 0;
-  DDI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device));
-  p.spread_smem = smem;
-  p.spread_blocks = std::max(1, std::min(per_sm * sms, (p.ncunits + kColThreads / 32 - 1) / (kColThreads / 32)));
-  return DDI_OK;
-}
-
-template <int W, int NS>
-int launch_spread_col2(Plan& p, cudaStream_t s) {
-  ColArgs a;
-  for (int d = 0; d < 3; ++d) a.nf[d] = p.nf[d];
-  a.ncx = p.nf[0] / kColX;
-  a.units = p.d_cunits;
-  a.nunits = p.ncunits;
-  a.counter = p.d_counter;
-  a.visits = p.d_cvis;
-  a.c = static_cast<const float2*>(p.d_c);
-  a.psi = static_cast<const float*>(p.d_psi);
-  a.fine = static_cast<float2*>(p.d_fine);
-  a.partial = static_cast<float2*>(p.d_cpart);
-  a.unit_slots = p.d_cslots;
-  DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, sizeof(int), s));
-  k_spread_col2<W, NS><<<p.spread_blocks, kColThreads, p.spread_smem, s>>>(a);
-  DDI_LAUNCH_CHECK();
-  p.mark("spread", s);
-  if (p.ncred > 0) {
-    k_reduce_col2<<<(unsigned)((p.ncred + 31) / 32), 256, 0, s>>>(
-        p.d_cred, p.ncred, static_cast<const float2*>(p.d_cpart), static_cast<float2*>(p.d_fine), p.nf[0]);
-    DDI_LAUNCH_CHECK();
-    p.mark("spread_reduce", s);
-  }
-  return DDI_OK;
-}
-
 int spread_col(Plan& p, cudaStream_t s, bool configure) {
-  if (p.dim == 3) return configure ? configure_spread_col3(p) : launch_spread_col3(p, s);
-  switch (p.w) {
-    case 6: return configure ? configure_spread_col2<6, 32>(p) : launch_spread_col2<6, 32>(p, s);
-    case 8: return configure ? configure_spread_col2<8, 32>(p) : launch_spread_col2<8, 32>(p, s);
-  }
-  set_error("column spread: kernel width %d not built", p.w);
-  return DDI_ERR_ARG;
+  return configure ? configure_spread_col(p) : launch_spread_col(p, s);
 }
 
 // ---- launch helpers ----------------------------------------------------------------------------
@@ -642,11 +459,19 @@ int launch_interp(Plan& p, cudaStream_t s) {
   const long long cnt = p.Mh;
   constexpr int XL = W <= 8 ? 8 : 16;
   if (cnt == 0) return DDI_OK;
-  k_interp<T, W, DIM><<<(unsigned)((cnt * XL + 255) / 256), 256, 0, s>>>(
-      static_cast<const cx_t<T>*>(p.d_fine), static_cast<const ushort4*>(p.d_l0), static_cast<const T*>(p.d_psi),
-      static_cast<const T*>(p.d_scale), static_cast<cx_t<T>*>(p.d_c), cnt, dims_of(p));
-  DDI_LAUNCH_CHECK();
-  return DDI_OK;
+  if constexpr (DIM == 2) {
+    // two waves of resident CTAs
+    const long long need = (cnt * XL + 255) / 256, most = 152LL * (sizeof(T) == 4 ? 4 : 2) * 2;
+    return launch_chain(p, k_interp2<T, W>, (unsigned)std::min(need, most), 256, 0, s,
+                        static_cast<const cx_t<T>*>(p.d_fine), static_cast<const ushort4*>(p.d_l0),
+                        static_cast<const T*>(p.d_psi), static_cast<const T*>(p.d_scale),
+                        static_cast<cx_t<T>*>(p.d_c), (int)cnt, dims_of(p));
+  } else {
+    return launch_chain(p, k_interp<T, W>, (unsigned)((cnt * XL + 255) / 256), 256, 0, s,
+                        static_cast<const cx_t<T>*>(p.d_fine), static_cast<const ushort4*>(p.d_l0),
+                        static_cast<const T*>(p.d_psi), static_cast<const T*>(p.d_scale),
+                        static_cast<cx_t<T>*>(p.d_c), cnt, dims_of(p));
+  }
 }
 
 // launch geometry of the spread, fixed per plan (computed once so that applies make no
@@ -693,9 +518,7 @@ int launch_spread(Plan& p, cudaStream_t s) {
   auto kern = k_spread<T, W, DIM>;
   const size_t smem = p.spread_smem;
   const int blocks = p.spread_blocks;
-  DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, sizeof(int), s));
-  kern<<<blocks, kSpreadThreads, smem, s>>>(a);
-  DDI_LAUNCH_CHECK();
+  DDI_TRY(launch_chain(p, kern, (unsigned)blocks, kSpreadThreads, smem, s, a));
   p.mark("spread", s);
   if (p.nsplit > 0) {
     for (int s0 = 0; s0 < p.nsplit; s0 += 65535) {
@@ -755,7 +578,8 @@ int time_spread(Plan& p, cudaStream_t s, int reps, float* ms) {
     set_error("time_spread: %s", cudaGetErrorString(cudaGetLastError()));
     return DDI_ERR_CUDA;
   }
-  auto once = [&]() {
+  auto once = [&]() -> int {
+    DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, sizeof(int), s));
     if (p.spread_kind == DDI_SPREAD_COLUMNS) return spread_col(p, s, false);
     if (p.prec == DDI_FP64) return p.dim == 3 ? launch_spread_w<double, 3>(p, s) : launch_spread_w<double, 2>(p, s);
     return p.dim == 3 ? launch_spread_w<float, 3>(p, s) : launch_spread_w<float, 2>(p, s);
@@ -783,7 +607,7 @@ int time_spread(Plan& p, cudaStream_t s, int reps, float* ms) {
 template <typename T>
 int run_type2(Plan& p, const T* rho, cudaStream_t s) {
   DDI_TRY(nufft_forward_fft<T>(p, rho, s));
-  if (p.col_interp) return launch_interp_col3(p, s);
+  if (p.col_interp) return launch_interp_col(p, s);
   DDI_TRY((p.dim == 3 ? launch_interp_w<T, 3>(p, s) : launch_interp_w<T, 2>(p, s)));
   p.mark("interp", s);
   return DDI_OK;
@@ -801,6 +625,7 @@ int run_type1(Plan& p, T* phi, cudaStream_t s, bool acc = false) {
 
 template <typename T>
 int run_type1_from_c(Plan& p, T* phi, cudaStream_t s) {
+  DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, sizeof(int), s));  // run_ddi: cleared by the forward transform
   return run_type1<T>(p, phi, s);
 }
 

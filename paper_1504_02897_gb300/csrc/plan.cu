@@ -98,7 +98,7 @@ void free_plan(Plan& p) {
                   p.d_deconv_x2, p.d_ones_x2,
                   p.d_partial,
                   p.d_visits, p.d_units, p.d_split, p.d_counter, p.d_psi1, p.d_rho, p.d_phi, p.d_work,
-                  p.d_work2,  p.d_kin,   p.d_red,   p.d_io_in, p.d_io_out, p.d_cvis, p.d_cunits, p.d_cred,
+                  p.d_work2,  p.d_kin,   p.d_red,   p.d_io_in, p.d_io_out, p.d_cunits, p.d_cred,
                   p.d_cslots, p.d_cpart, p.d_nonfinite, p.d_cimage, p.d_cnodes, p.d_cshare,
                   p.d_cnoff, p.d_cnpos, p.d_em1};
   for (void* q : ptrs)
@@ -262,8 +262,7 @@ namespace {
 // window) in one contiguous piece
 bool columns_fit(const Plan& p) {
   if (p.w > 16 || p.nf[0] % kColX != 0 || p.nf[0] < kColX + p.w - 1) return false;
-  if (p.dim == 2) return p.nf[1] >= p.w;
-  return p.nf[1] % kColY == 0 && p.nf[1] >= kColY + p.w - 1 && p.nf[2] >= p.w;
+  return p.nf[1] % kColY == 0 && p.nf[1] >= kColY + p.w - 1 && (p.dim == 2 || p.nf[2] >= p.w);
 }
 }  // namespace
 
@@ -282,31 +281,117 @@ static bool columns_auto3(const Plan& p) {
   return columns_fit(p) && p.Mh >= 2048 && p.desc.tile[0] <= 0 && p.desc.tile[1] <= 0 && p.desc.tile[2] <= 0;
 }
 
-// Frees the spread lists of both schemes (the autotuner switches a 2D plan between them).
-void drop_spread_lists(Plan& p) {
-  p.col_interp = false;
-  for (void** q : {(void**)&p.d_visits, (void**)&p.d_units, (void**)&p.d_split, &p.d_partial, (void**)&p.d_cvis,
-                   (void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart, (void**)&p.d_cimage,
-                   (void**)&p.d_cnodes, &p.d_cshare, (void**)&p.d_cnoff, (void**)&p.d_cnpos})
+// The groups' images and node lists on the device, made there from the visits (gvis: [group][32]
+// node or -1 and packed start), 3D: the runs and counts of each group.  Those lists are needed on
+// the device only while the images are made.
+static int upload_images(Plan& p, const std::vector<int2>& gvis, const std::vector<int>* gruns,
+                         const std::vector<int2>* gcount, cudaStream_t stream) {
+  const size_t ng = gvis.size() / 32;
+  int2 *dv = nullptr, *dc = nullptr;
+  int* dr = nullptr;
+  const size_t kept = p.bytes;
+  int st = upload(p, (void**)&dv, gvis, "column visits", stream);
+  if (st == DDI_OK && gruns) st = upload(p, (void**)&dr, *gruns, "column runs", stream);
+  if (st == DDI_OK && gcount) st = upload(p, (void**)&dc, *gcount, "column groups", stream);
+  p.bytes = kept;
+  if (st == DDI_OK) st = dev_alloc(p, (void**)&p.d_cimage, col_image_bytes(p) * ng, "column group images");
+  if (st == DDI_OK) st = dev_alloc(p, (void**)&p.d_cnodes, sizeof(int) * 32 * ng, "column group nodes");
+  if (st == DDI_OK) st = build_col_images(p, dv, dr, dc, stream);
+  if (st == DDI_OK && cudaStreamSynchronize(stream) != cudaSuccess) {
+    set_error("column group images: %s", cudaGetErrorString(cudaGetLastError()));
+    st = DDI_ERR_CUDA;
+  }
+  cudaFree(dv);
+  cudaFree(dr);
+  cudaFree(dc);
+  return st;
+}
+
+// Block spread lists of an FP32 2D plan: every processed node visits the 8 x 8 blocks its footprint
+// reaches; a block's visits (in node order) are cut into groups of 32 and units of about `chunk`
+// visits.  A block of one unit is written by it; the units of the others write partial slots,
+// contiguous per block in unit order, that a reduce entry sums.  Blocks without visits are written
+// as zeros where a y line of them holds taps.
+static int build_spread_block(Plan& p, cudaStream_t stream) {
+  const int W = p.w, nfx = p.nf[0], nfy = p.nf[1];
+  const int ncx = nfx / kColX, ncy = nfy / kColY, nblk = ncx * ncy;
+  DDI_CUDA(cudaStreamSynchronize(stream));
+  for (void** q : {(void**)&p.d_cunits, (void**)&p.d_cred, &p.d_cpart, (void**)&p.d_cimage, (void**)&p.d_cnodes})
     if (*q) {
       cudaFree(*q);
       *q = nullptr;
     }
   p.bytes -= p.spread_bytes;
   p.spread_bytes = 0;
+  const size_t before = p.bytes;
+  // f(block, packed start) for every block of node i
+  auto for_blocks = [&](int64_t i, auto&& f) {
+    const int x = p.h_l0[i].x, y = p.h_l0[i].y;
+    for (int ty = y & ~(kColY - 1); ty < y + W; ty += kColY)
+      for (int tx = x & ~(kColX - 1); tx < x + W; tx += kColX)
+        f((ty % nfy) / kColY * ncx + (tx % nfx) / kColX, ((y - ty + 16) << 6) | (x - tx + 16));
+  };
+  std::vector<int> start((size_t)nblk + 1, 0);
+  for (int64_t i = 0; i < p.Mh; ++i) for_blocks(i, [&](int b, int) { ++start[b + 1]; });
+  long long total = 0, groups = 0;
+  for (int b = 0; b < nblk; ++b) {
+    total += start[b + 1];
+    groups += (start[b + 1] + 31) / 32;
+  }
+  if (32 * groups > (long long)INT32_MAX - 1 || p.Mh > (int64_t)INT32_MAX) {
+    set_error("%lld block-spread visits exceed the 32-bit visit lists; use fewer quadrature nodes", total);
+    return DDI_ERR_ARG;
+  }
+  // visits per unit: about two units per resident warp, at least two groups, at most 16
+  const int cap = p.desc.chunk > 0 ? p.desc.chunk
+                                   : (int)std::min<long long>(512, std::max<long long>(64, total / 9728 / 32 * 32));
+  const int unit_groups = std::max(1, cap / 32);
+  std::vector<int2> gvis((size_t)groups * 32, make_int2(-1, 0));
+  std::vector<int> fill(nblk);
+  std::vector<ColUnit> units;
+  std::vector<ColRed> red;
+  int g = 0, nslot = 0;
+  for (int b = 0; b < nblk; ++b) {
+    const int n = start[b + 1], ng = (n + 31) / 32;
+    fill[b] = g * 32;
+    if (n == 0) {
+      bool needed = false;
+      for (int r = 0; r < kColY; ++r) {
+        int d = b / ncx * kColY + r - p.yr[0];
+        if (d < 0) d += nfy;
+        needed = needed || d < p.yr[1];
+      }
+      if (needed) units.push_back(ColUnit{b, 0, 0, -1, 0, 0, 0, 0});
+      continue;
+    }
+    const int nu = (ng + unit_groups - 1) / unit_groups;
+    if (nu > 1) red.push_back(ColRed{b, 0, nslot, nu});
+    for (int u = 0; u < nu; ++u)
+      units.push_back(ColUnit{b, g + (int)((long long)ng * u / nu), g + (int)((long long)ng * (u + 1) / nu),
+                              nu > 1 ? nslot++ : -1, 0, 0, 0, 0});
+    g += ng;
+  }
+  for (int64_t i = 0; i < p.Mh; ++i) for_blocks(i, [&](int b, int o) { gvis[fill[b]++] = make_int2((int)i, o); });
+  std::stable_sort(units.begin(), units.end(),
+                   [](const ColUnit& a, const ColUnit& b) { return a.hi - a.lo > b.hi - b.lo; });
+  p.visits = p.pairs = total;
+  p.chunk = cap;
+  p.ngroups = (int)groups;
+  p.ncunits = (int)units.size();
+  p.ncslots = nslot;
+  p.ncred = (int)red.size();
+  // entries of more than 24 slots first: a CTA sums each of them
+  p.ncred_long = (int)(std::stable_partition(red.begin(), red.end(), [](const ColRed& r) { return r.ns > 24; }) -
+                       red.begin());
+  DDI_TRY(upload_images(p, gvis, nullptr, nullptr, stream));
+  DDI_TRY(upload(p, (void**)&p.d_cunits, units, "block units", stream));
+  DDI_TRY(upload(p, (void**)&p.d_cred, red, "block reduce entries", stream));
+  DDI_TRY(dev_alloc(p, &p.d_cpart, p.cx_size() * kColX * kColY * (size_t)std::max(1, nslot), "partial blocks"));
+  p.spread_bytes = p.bytes - before;
+  DDI_CUDA(cudaStreamSynchronize(stream));
+  return configure_kernels(p);
 }
 
-// Column spread lists.  3D: columns of kColX x kColY cells in x-y run the whole z axis (the
-// window axis); 2D: columns of kColX cells in x run the whole y axis.  Every processed node
-// visits the columns its cross-axis taps reach; a column's visits are sorted by the node's
-// first tap along the window axis, then (3D) by z class, then by node.  The visits are cut
-// into units of at most `chunk` visits; unit c writes the planes (2D: rows) [a_c, e_c), a_c =
-// its first visit's first tap, e_c the end of its last footprint extended over the gap to the
-// next unit (at most 64 planes ahead; longer gaps and empty columns get units without visits
-// that only write zeros).  A plane that several units touch (their footprints overlap at unit
-// boundaries, and the last unit of a column wraps onto the first) is a leading or trailing
-// plane of each of them: those go to partial slots and a reduce entry sums them in unit order;
-// every other plane is written by its one unit.  Every fine cell is written once per apply.
 // Visits per unit of a 3D column spread: the fewest units that still keep the device even.
 // Swept over 32 .. 1024 (spread + reduction, us): FP32 (2432 resident warps) 24^3 at 64,
 // 96x64x48 54 at 128 and 256 (60 at 512, 86 at 64), 128^3 101 at 512 (126 at 128), 192^3 277 at
@@ -318,14 +403,22 @@ static int default_col_chunk(int prec, long long visits) {
   return (int)std::min<long long>(512, std::max<long long>(64, c));
 }
 
+// Column spread lists of a 3D plan: columns of kColX x kColY cells in x-y run the whole z axis.
+// Every processed node visits the columns its x and y taps reach; a column's visits are sorted by
+// the node's first z tap, then by z class, then by node.  The visits are cut
+// into units of at most `chunk` visits; unit c writes the planes [a_c, e_c), a_c =
+// its first visit's first tap, e_c the end of its last footprint extended over the gap to the
+// next unit (at most kColPlanes planes together; longer gaps and empty columns get units without visits
+// that only write zeros).  A plane that several units touch (their footprints overlap at unit
+// boundaries, and the last unit of a column wraps onto the first) is a leading or trailing
+// plane of each of them: those go to partial slots and a reduce entry sums them in unit order;
+// every other plane is written by its one unit.  Every fine cell is written once per apply.
 int build_spread_col(Plan& p, cudaStream_t stream) {
-  const bool d3 = p.dim == 3;
-  const int W = p.w, nfx = p.nf[0], nfy = p.nf[1];
-  const int nfz = p.nf[p.dim - 1];  // the window axis: z (3D), y (2D)
-  const int cy_cells = d3 ? kColY : 1;
-  const int ncx = nfx / kColX, ncy = d3 ? nfy / kColY : 1, ncol = ncx * ncy;
+  if (p.dim == 2) return build_spread_block(p, stream);
+  const int W = p.w, nfx = p.nf[0], nfy = p.nf[1], nfz = p.nf[2];
+  const int ncx = nfx / kColX, ncy = nfy / kColY, ncol = ncx * ncy;
   DDI_CUDA(cudaStreamSynchronize(stream));
-  for (void** q : {(void**)&p.d_cvis, (void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart,
+  for (void** q : {(void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart,
                    (void**)&p.d_cimage, (void**)&p.d_cnodes, &p.d_cshare, (void**)&p.d_cnoff, (void**)&p.d_cnpos})
     if (*q) {
       cudaFree(*q);
@@ -341,16 +434,10 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
     if (k < 0) k += nf / B;
     return k + 1;
   };
-  auto yspan = [&](int l, int* first) {  // 2D: the one column row
-    if (d3) return span(l, nfy, kColY, first);
-    *first = 0;
-    return 1;
-  };
-  auto wtap = [&](const ushort4& l) { return d3 ? (int)l.z : (int)l.y; };
   std::vector<int> count(ncol + 1, 0);
   for (int64_t i = 0; i < p.Mh; ++i) {
     int fx, fy;
-    const int kx = span(p.h_l0[i].x, nfx, kColX, &fx), ky = yspan(p.h_l0[i].y, &fy);
+    const int kx = span(p.h_l0[i].x, nfx, kColX, &fx), ky = span(p.h_l0[i].y, nfy, kColY, &fy);
     for (int b = 0; b < ky; ++b)
       for (int a = 0; a < kx; ++a) ++count[((fy + b) % ncy) * ncx + (fx + a) % ncx];
   }
@@ -367,35 +454,39 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
     for (int64_t i = 0; i < p.Mh; ++i) {
       const ushort4 l = p.h_l0[i];
       int fx, fy;
-      const int kx = span(l.x, nfx, kColX, &fx), ky = yspan(l.y, &fy);
+      const int kx = span(l.x, nfx, kColX, &fx), ky = span(l.y, nfy, kColY, &fy);
       for (int b = 0; b < ky; ++b)
         for (int a = 0; a < kx; ++a) {
           const int bx = (fx + a) % ncx, by = (fy + b) % ncy;
-          const int ox = rel_start(l.x, bx * kColX, nfx, W), oy = d3 ? rel_start(l.y, by * kColY, nfy, W) : 0;
-          if (ox < -(W - 1) || ox >= kColX || oy < -(W - 1) || oy >= cy_cells) {
+          const int ox = rel_start(l.x, bx * kColX, nfx, W), oy = rel_start(l.y, by * kColY, nfy, W);
+          if (ox < -(W - 1) || ox >= kColX || oy < -(W - 1) || oy >= kColY) {
             set_error("column spread: footprint offset (%d, %d) outside its column", ox, oy);
             return DDI_ERR_INTERNAL;
           }
-          vis[fill[by * ncx + bx]++] = make_int2((int)i, (wtap(l) << 13) | ((oy + 16) << 6) | (ox + 16));
+          vis[fill[by * ncx + bx]++] = make_int2((int)i, ((int)l.z << 13) | ((oy + 16) << 6) | (ox + 16));
         }
     }
   }
-  // per column: by first window-axis tap, then z class (3D: nodes with the same first tap and
-  // bit-identical psi_z rows, e.g. one quadrature ring; 2D: one class), then node (the visits
-  // are in node order already); bit 12 marks the first visit of each run of one (tap, class)
+  // per column: by first z tap, then z class (nodes with the same first tap and bit-identical
+  // psi_z rows: one quadrature ring), then node; bit 12 marks the first visit of each run of one
+  // (tap, class)
+  std::vector<std::pair<int64_t, int2>> key;  // (first tap, class), visit
   for (int c = 0; c < ncol; ++c) {
     auto b = vis.begin() + start[c], e = vis.begin() + start[c + 1];
-    std::stable_sort(b, e, [&](const int2& u, const int2& v) {
-      const int su = u.y >> 13, sv = v.y >> 13;
-      return su != sv ? su < sv : p.h_zcls[u.x] < p.h_zcls[v.x];
+    key.clear();
+    for (auto it = b; it != e; ++it)
+      key.push_back(std::make_pair(((int64_t)(it->y >> 13) << 32) | (uint32_t)p.h_zcls[it->x], *it));
+    std::sort(key.begin(), key.end(), [](const std::pair<int64_t, int2>& u, const std::pair<int64_t, int2>& v) {
+      return u.first != v.first ? u.first < v.first : u.second.x < v.second.x;
     });
+    for (size_t k = 0; k < key.size(); ++k) b[k] = key[k].second;
     for (auto it = b; it != e; ++it)
       if (it == b || (it->y >> 13) != ((it - 1)->y >> 13) || p.h_zcls[it->x] != p.h_zcls[(it - 1)->x])
         it->y |= 1 << 12;
   }
-  const int cap = p.desc.chunk > 0 ? p.desc.chunk : d3 ? default_col_chunk(p.prec, total) : 256;
-  const int lmax = std::min(d3 ? kColPlanes : 64, nfz);
-  // 3D: the column's visits in groups of at most 32 slots and kColRuns runs (columns.cuh).  A
+  const int cap = p.desc.chunk > 0 ? p.desc.chunk : default_col_chunk(p.prec, total);
+  const int lmax = std::min(kColPlanes, nfz);
+  // the column's visits in groups of at most 32 slots and kColRuns runs (columns.cuh).  A
   // run takes an even number of slots, and is cut only where it is longer than a group or leaves
   // half a group empty: its second part adds psi_z to the window once more
   std::vector<int2> gvis;    // [group][32]: node (-1: none), packed x/y start
@@ -442,8 +533,8 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
     if (b0 == b1) {
       // an empty column is written as zeros, unless none of its x or y lines holds a tap (the
       // NUFFT's passes neither transform nor read those lines)
-      bool in_y = !d3, in_x = false;  // a 2D column holds every y line
-      for (int r = 0; d3 && r < kColY; ++r) {
+      bool in_y = false, in_x = false;
+      for (int r = 0; r < kColY; ++r) {
         int d = (c / ncx) * kColY + r - p.yr[0];
         if (d < 0) d += nfy;
         in_y = in_y || d < p.yr[1];
@@ -460,32 +551,25 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
     }
     // visit chunks and their planes [a, b) (b = last first tap + w)
     std::vector<std::array<int, 4>> ch;  // lo, hi, a, b
-    if (d3) {
-      // whole groups: at most cap visits, a window of kColPlanes and the work of about cap visits.
-      // (kernel issue slots: 6 a visit, 33 a run, 40 a plane, 130 a group, on average 22 a visit; the
-      // sparse columns' few visits spread over all planes, and one unit for such a column ran
-      // for 90 us where the average took 13)
-      const int g0 = (int)gcount.size();
-      add_groups(b0, b1);
-      const int g1 = (int)gcount.size();
-      auto first = [&](int g) { return g < g1 ? gbeg[g] : b1; };
-      for (int k = g0; k < g1;) {
-        const int a = vis[gbeg[k]].y >> 13;
-        int hi = k;
-        long long work = 40 * W;
-        for (; hi < g1; ++hi) {
-          const int end = (vis[first(hi + 1) - 1].y >> 13) + W;
-          work += 130 + 6 * gcount[hi].x + 33 * gcount[hi].y + 40 * (end - std::max(a + W, (vis[gbeg[hi]].y >> 13) + W));
-          if (hi > k && (first(hi + 1) - gbeg[k] > cap || end - a > kColPlanes || work > 22LL * cap)) break;
-        }
-        ch.push_back({{k, hi, a, (vis[first(hi) - 1].y >> 13) + W}});
-        k = hi;
+    // whole groups: at most cap visits, a window of kColPlanes and the work of about cap visits.
+    // (kernel issue slots: 6 a visit, 33 a run, 40 a plane, 130 a group, on average 22 a visit; the
+    // sparse columns' few visits spread over all planes, and one unit for such a column ran
+    // for 90 us where the average took 13)
+    const int g0 = (int)gcount.size();
+    add_groups(b0, b1);
+    const int g1 = (int)gcount.size();
+    auto first = [&](int g) { return g < g1 ? gbeg[g] : b1; };
+    for (int k = g0; k < g1;) {
+      const int a = vis[gbeg[k]].y >> 13;
+      int hi = k;
+      long long work = 40 * W;
+      for (; hi < g1; ++hi) {
+        const int end = (vis[first(hi + 1) - 1].y >> 13) + W;
+        work += 130 + 6 * gcount[hi].x + 33 * gcount[hi].y + 40 * (end - std::max(a + W, (vis[gbeg[hi]].y >> 13) + W));
+        if (hi > k && (first(hi + 1) - gbeg[k] > cap || end - a > kColPlanes || work > 22LL * cap)) break;
       }
-    } else {
-      for (int k = b0; k < b1; k += cap) {
-        const int hi = std::min(b1, k + cap);
-        ch.push_back({{k, hi, vis[k].y >> 13, (vis[hi - 1].y >> 13) + W}});
-      }
+      ch.push_back({{k, hi, a, (vis[first(hi) - 1].y >> 13) + W}});
+      k = hi;
     }
     const int nch = (int)ch.size();
     for (int k = 0; k < nch; ++k) {
@@ -528,34 +612,13 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
       contrib[z].clear();
     }
   }
-  // costliest units first, those without visits last.  3D: the work above.  2D: the four lane
-  // groups share a run (one first y tap), so a run of L visits takes ceil(L / 4) steps; a
-  // unit costs about 4 per step, 3 per run and 5 per row it writes (relative instruction
-  // counts of the kernel's visit step, run start and row flush)
+  // costliest units first, those without visits last
   {
     std::vector<long long> cost(units.size());
     for (size_t u = 0; u < units.size(); ++u) {
       const ColUnit& U = units[u];
-      if (d3) {
-        cost[u] = 40LL * (U.z1 - U.z0);
-        for (int k = U.lo; k < U.hi; ++k) cost[u] += 130 + 6 * gcount[k].x + 33 * gcount[k].y;
-        continue;
-      }
-      long long steps = 0, runs = 0;
-      int len = 0;
-      for (int k = U.lo; k < U.hi; ++k) {
-        if (k > U.lo && ((vis[k].y >> 12) & 1)) {
-          steps += (len + 3) / 4;
-          ++runs;
-          len = 0;
-        }
-        ++len;
-      }
-      if (len > 0) {
-        steps += (len + 3) / 4;
-        ++runs;
-      }
-      cost[u] = 4 * steps + 3 * runs + 5LL * (U.z1 - U.z0);
+      cost[u] = 40LL * (U.z1 - U.z0);
+      for (int k = U.lo; k < U.hi; ++k) cost[u] += 130 + 6 * gcount[k].x + 33 * gcount[k].y;
     }
     std::vector<size_t> ord(units.size());
     std::iota(ord.begin(), ord.end(), (size_t)0);
@@ -566,7 +629,7 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
     std::vector<ColUnit> sorted(units.size());
     for (size_t k = 0; k < ord.size(); ++k) sorted[k] = units[ord[k]];
     units.swap(sorted);
-    if (d3) {  // the kernel's table: the slot of each plane of the window, -1 where the unit alone writes it
+    {  // the kernel's table: the slot of each plane of the window, -1 where the unit alone writes it
       std::vector<int> dest(units.size() * kColPlanes, -1);
       for (size_t u = 0; u < units.size(); ++u) {
         const ColUnit& U = units[u];
@@ -590,69 +653,63 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
   p.chunk = cap;
   p.ncunits = (int)units.size();
   p.ncred = (int)red.size();
-  p.ncred_long = 0;
-  if (d3)  // entries of more than 24 slots first: a CTA sums each of them
-    p.ncred_long = (int)(std::stable_partition(red.begin(), red.end(), [](const ColRed& r) { return r.ns > 24; }) -
-                         red.begin());
+  // entries of more than 24 slots first: a CTA sums each of them
+  p.ncred_long = (int)(std::stable_partition(red.begin(), red.end(), [](const ColRed& r) { return r.ns > 24; }) -
+                       red.begin());
   p.ncslots = nslot;
   p.ncvunits = 0;
   for (const ColUnit& U : units) p.ncvunits += U.lo < U.hi ? 1 : 0;
-  if (d3) {
-    p.ngroups = (int)gcount.size();
-    if (gvis.size() > (size_t)INT32_MAX) {
-      set_error("column spread: work list too long");
-      return DDI_ERR_ARG;
-    }
-    // FP64: the gather kernel costs twice the FP64 operations (64^3: 748 us against 400, 128^3 5.9 ms
-    // against 2.5).  FP32: below 2^18 processed nodes its one launch is the shorter (24^3 10 us
-    // against 17, 96x64x48 with 221184 nodes 55 against 54, 128^3 with 524288 133 against 112)
-    p.col_interp = p.prec == DDI_FP64 || p.Mh >= (1 << 18);
-    // where each node's visits are: their interpolation shares are summed in this order
-    if (p.col_interp) {
-      std::vector<int> noff((size_t)p.Mh + 1, 0), npos((size_t)total);
-      for (const int2& v : gvis)
-        if (v.x >= 0) ++noff[(size_t)v.x + 1];
-      for (size_t i = 0; i < (size_t)p.Mh; ++i) noff[i + 1] += noff[i];
-      {
-        std::vector<int> fill(noff.begin(), noff.end() - 1);
-        for (size_t q = 0; q < gvis.size(); ++q)
-          if (gvis[q].x >= 0) npos[fill[gvis[q].x]++] = (int)q;
-      }
-      DDI_TRY(upload(p, (void**)&p.d_cnoff, noff, "node share ranges", stream));
-      DDI_TRY(upload(p, (void**)&p.d_cnpos, npos, "node shares", stream));
-      DDI_TRY(dev_alloc(p, &p.d_cshare, p.cx_size() * gvis.size(), "visit shares"));
-      DDI_CUDA(cudaStreamSynchronize(stream));  // noff and npos die with this block
-    }
-    // the lists the images are made from are needed on the device only while they are made
-    int2 *dv = nullptr, *dc = nullptr;
-    int* dr = nullptr;
-    const size_t kept = p.bytes;
-    int st = upload(p, (void**)&dv, gvis, "column visits", stream);
-    if (st == DDI_OK) st = upload(p, (void**)&dr, gruns, "column runs", stream);
-    if (st == DDI_OK) st = upload(p, (void**)&dc, gcount, "column groups", stream);
-    p.bytes = kept;
-    if (st == DDI_OK) st = dev_alloc(p, (void**)&p.d_cimage, col_image_bytes(p) * gcount.size(), "column group images");
-    if (st == DDI_OK) st = dev_alloc(p, (void**)&p.d_cnodes, sizeof(int) * 32 * gcount.size(), "column group nodes");
-    if (st == DDI_OK) st = build_col_images(p, dv, dr, dc, stream);
-    if (st == DDI_OK && cudaStreamSynchronize(stream) != cudaSuccess) {
-      set_error("column group images: %s", cudaGetErrorString(cudaGetLastError()));
-      st = DDI_ERR_CUDA;
-    }
-    cudaFree(dv);
-    cudaFree(dr);
-    cudaFree(dc);
-    DDI_TRY(st);
-  } else {
-    DDI_TRY(upload(p, (void**)&p.d_cvis, vis, "column visits", stream));
+  p.ngroups = (int)gcount.size();
+  if (gvis.size() > (size_t)INT32_MAX) {
+    set_error("column spread: work list too long");
+    return DDI_ERR_ARG;
   }
+  // FP64: the gather kernel costs twice the FP64 operations (64^3: 748 us against 400, 128^3 5.9 ms
+  // against 2.5).  FP32: below 2^18 processed nodes its one launch is the shorter (24^3 10 us
+  // against 17, 96x64x48 with 221184 nodes 55 against 54, 128^3 with 524288 133 against 112)
+  p.col_interp = p.prec == DDI_FP64 || p.Mh >= (1 << 18);
+  // where each node's visits are: their interpolation shares are summed in this order
+  if (p.col_interp) {
+    std::vector<int> noff((size_t)p.Mh + 1, 0), npos((size_t)total);
+    for (const int2& v : gvis)
+      if (v.x >= 0) ++noff[(size_t)v.x + 1];
+    for (size_t i = 0; i < (size_t)p.Mh; ++i) noff[i + 1] += noff[i];
+    {
+      std::vector<int> fill(noff.begin(), noff.end() - 1);
+      for (size_t q = 0; q < gvis.size(); ++q)
+        if (gvis[q].x >= 0) npos[fill[gvis[q].x]++] = (int)q;
+    }
+    DDI_TRY(upload(p, (void**)&p.d_cnoff, noff, "node share ranges", stream));
+    DDI_TRY(upload(p, (void**)&p.d_cnpos, npos, "node shares", stream));
+    DDI_TRY(dev_alloc(p, &p.d_cshare, p.cx_size() * gvis.size(), "visit shares"));
+    DDI_CUDA(cudaStreamSynchronize(stream));  // noff and npos die with this block
+  }
+  DDI_TRY(upload_images(p, gvis, &gruns, &gcount, stream));
   DDI_TRY(upload(p, (void**)&p.d_cunits, units, "column units", stream));
   DDI_TRY(upload(p, (void**)&p.d_cred, red, "column reduce entries", stream));
   DDI_TRY(upload(p, (void**)&p.d_cslots, slots, "column slot lists", stream));
-  DDI_TRY(dev_alloc(p, &p.d_cpart, p.cx_size() * kColX * cy_cells * (size_t)std::max(1, nslot),
+  DDI_TRY(dev_alloc(p, &p.d_cpart, p.cx_size() * kColX * kColY * (size_t)std::max(1, nslot),
                     "column partial planes"));
   p.spread_bytes = p.bytes - before;
   DDI_CUDA(cudaStreamSynchronize(stream));
   return configure_kernels(p);
+}
+
+// psi_d at tap t of node i, [node][3][w]: tap t sits at x = t - fr from the node, in fine cells;
+// axes past the plan's hold 1, 0, 0, ..
+template <typename T>
+static __global__ void k_taps(const double* __restrict__ fr, T* __restrict__ psi, long long total, int dim, int w,
+                              double beta) {
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= total) return;
+  const int t = (int)(q % w), a = (int)(q / w % 3);
+  const long long i = q / (3 * w);
+  double v = a < dim ? 0.0 : (t == 0 ? 1.0 : 0.0);
+  if (a < dim) {
+    const double z = ((double)t - fr[i * dim + a]) / (0.5 * (double)w);
+    if (z * z < 1.0) v = exp(beta * (sqrt((1.0 - z) * (1.0 + z)) - 1.0));
+  }
+  psi[q] = (T)v;
 }
 
 int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool gpe, bool batch_item) {
@@ -691,14 +748,10 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
               kColX, kColX, kColY, kColX - 1, kColY - 1);
     return DDI_ERR_ARG;
   }
-  // automatic choice: columns in 3D.  In 2D, a plan on its own takes columns only up to 512^2
-  // fine cells; above that the tile spread measured faster alone (the 2D column's runs of one
-  // first y tap are short there, so three of its four lane groups idle), and its autotuner
-  // times both schemes.  Batch items take columns at every size: they run beside the other
-  // items' kernels, and the 96-density batch measured 13.3 ms with columns against 15.5 ms
-  // with tiles (the faster tiles alone) and 15.2 ms with the size rule
+  // automatic choice: columns where they apply (2D: blocks of 8 x 8 cells, faster
+  // than the tiles at every size, see columns.cu)
   p.batch_item = batch_item;
-  const bool columns2 = p.dim == 2 && columns_apply(p) && (batch_item || (long long)p.nf[0] * p.nf[1] <= 512LL * 512);
+  const bool columns2 = p.dim == 2 && columns_apply(p);
   p.Mh = p.M / 2;  // one node of each (k, -k) pair
   p.spread_kind = d.spread == DDI_SPREAD_COLUMNS || (d.spread == DDI_SPREAD_AUTO && (columns2 || columns_auto3(p)))
                       ? DDI_SPREAD_COLUMNS
@@ -720,7 +773,7 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
   // their first-tap tile (spatial locality of the interpolation reads)
   std::vector<int> l0w(3 * p.Mh, 0);
   std::vector<double> fr(3 * p.Mh, 0.0);
-  std::vector<int64_t> okey(p.Mh);
+  std::vector<std::pair<int64_t, int64_t>> okey(p.Mh);  // key, node
   for (int64_t i = 0; i < p.Mh; ++i) {
     const int64_t q = qs[i];
     for (int a = 0; a < dim; ++a) {
@@ -733,50 +786,25 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
     const int bx = l0w[3 * i] / p.tile[0], by = l0w[3 * i + 1] / p.tile[1], bz = l0w[3 * i + 2] / p.tile[2];
     const int64_t bin = ((int64_t)bz * p.ntile[1] + by) * p.ntile[0] + bx;
     const int64_t key = ((int64_t)l0w[3 * i + 2] * p.nf[1] + l0w[3 * i + 1]) * p.nf[0] + l0w[3 * i];
-    okey[i] = bin * p.fine_points() + key;
+    okey[i] = std::make_pair(bin * p.fine_points() + key, i);
   }
-  std::vector<int64_t> perm(p.Mh);
-  std::iota(perm.begin(), perm.end(), 0);
-  std::stable_sort(perm.begin(), perm.end(), [&](int64_t a, int64_t b) { return okey[a] < okey[b]; });
+  std::sort(okey.begin(), okey.end());
 
   p.order.resize(p.Mh);
   std::vector<ushort4>& l0s = p.h_l0;
   l0s.assign(p.Mh, ushort4{});
-  std::vector<double> psi((size_t)p.Mh * 3 * W, 1.0), scale(p.Mh);
-  const double hw = 0.5 * (double)W;
-  // z classes: nodes whose first z tap and fractional z offset are equal have the same psi_z
-  // row (computed by the same operations), so the column spread can sum them before psi_z
+  std::vector<double> scale(p.Mh), frs((size_t)p.Mh * dim);
+  // z classes: the nodes of one ring have one k_z, so equal first z taps and the same psi_z row
+  // (computed by the same operations), and the column spread can sum them before psi_z
   p.h_zcls.assign(p.Mh, 0);
-  {
-    std::vector<std::pair<std::pair<int, uint64_t>, int64_t>> zk((size_t)p.Mh);
-    for (int64_t i = 0; i < p.Mh; ++i) {
-      uint64_t bits = 0;
-      const double f = dim == 3 ? fr[3 * perm[i] + 2] : 0.0;
-      std::memcpy(&bits, &f, sizeof bits);
-      zk[i] = std::make_pair(std::make_pair(dim == 3 ? l0w[3 * perm[i] + 2] : 0, bits), i);
-    }
-    std::sort(zk.begin(), zk.end());
-    int cls = -1;
-    for (size_t k = 0; k < zk.size(); ++k) {
-      if (k == 0 || zk[k].first != zk[k - 1].first) ++cls;
-      p.h_zcls[zk[k].second] = cls;
-    }
-  }
   for (int64_t i = 0; i < p.Mh; ++i) {
-    const int64_t o = perm[i];
+    const int64_t o = okey[i].second;
     p.order[i] = qs[o];
     l0s[i] = make_ushort4((unsigned short)l0w[3 * o], (unsigned short)l0w[3 * o + 1],
                           (unsigned short)l0w[3 * o + 2], 0);
-    for (int a = 0; a < 3; ++a)
-      for (int t = 0; t < W; ++t) {
-        double v = a < dim ? 0.0 : (t == 0 ? 1.0 : 0.0);
-        if (a < dim) {
-          const double z = ((double)t - fr[3 * o + a]) / hw;
-          if (z * z < 1.0) v = std::exp(p.beta * (std::sqrt((1.0 - z) * (1.0 + z)) - 1.0));
-        }
-        psi[((size_t)i * 3 + a) * W + t] = v;
-      }
+    for (int a = 0; a < dim; ++a) frs[(size_t)dim * i + a] = fr[3 * o + a];
     scale[i] = 2.0 * p.dv * p.quad.W[qs[o]];
+    if (dim == 3) p.h_zcls[i] = (int)(qs[o] / nphi);
   }
 
   // the shortest cyclic range of fine y lines holding every tap (the complement of the
@@ -823,9 +851,28 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
 
   // device memory
   const size_t rs = p.real_size(), cs = p.cx_size();
-  std::vector<float> k1, k2;
+  std::vector<float> k2;
   DDI_TRY(upload(p, &p.d_l0, l0s, "node taps", stream));
-  DDI_TRY(upload_real(p, &p.d_psi, psi, "kernel values", stream, &k1));
+  // kernel values psi_d at the w taps: from the FP64 offsets, in FP64 on the device, rounded once
+  DDI_TRY(dev_alloc(p, &p.d_psi, rs * 3 * W * (size_t)p.Mh, "kernel values"));
+  if (p.Mh > 0) {
+    double* d_fr = nullptr;
+    const size_t kept = p.bytes;
+    DDI_TRY(upload(p, (void**)&d_fr, frs, "node offsets", stream));
+    p.bytes = kept;
+    const long long total = (long long)p.Mh * 3 * W;
+    const unsigned blocks = (unsigned)((total + 255) / 256);
+    if (p.prec == DDI_FP64)
+      k_taps<double><<<blocks, 256, 0, stream>>>(d_fr, static_cast<double*>(p.d_psi), total, dim, W, p.beta);
+    else
+      k_taps<float><<<blocks, 256, 0, stream>>>(d_fr, static_cast<float*>(p.d_psi), total, dim, W, p.beta);
+    const cudaError_t e1 = cudaGetLastError(), e2 = cudaStreamSynchronize(stream);
+    cudaFree(d_fr);
+    if (e1 != cudaSuccess || e2 != cudaSuccess) {
+      set_error("kernel values: %s", cudaGetErrorString(e1 != cudaSuccess ? e1 : e2));
+      return DDI_ERR_CUDA;
+    }
+  }
   DDI_TRY(upload_real(p, &p.d_scale, scale, "node scales", stream, &k2));
   std::vector<NodeDir> dirw;
   if (gpe) {
@@ -837,12 +884,13 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
     }
     DDI_TRY(upload(p, (void**)&p.d_dirw, dirw, "node directions", stream));
   }
-  // deconvolution factors stay FP64 in both precisions; FP32 plans also get the y factors
+  // deconvolution factors stay FP64 in both precisions; FP32 plans also get the y (2D: x) factors
   // as FP32 head + tail pairs (applied so that only the final product is rounded)
   auto pairs = [&](const std::vector<double>& v) {
-    std::vector<float2> out((size_t)p.n[1]);
-    for (int j = 0; j < p.n[1]; ++j) {
-      const double f = v[(size_t)p.n[0] + j];
+    const int axis = dim == 3 ? 1 : 0;
+    std::vector<float2> out((size_t)p.n[axis]);
+    for (int j = 0; j < p.n[axis]; ++j) {
+      const double f = v[(size_t)(axis ? p.n[0] : 0) + j];
       const float hi = (float)f;
       out[j] = make_float2(hi, (float)(f - (double)hi));
     }

@@ -57,3 +57,31 @@ def test_columns_match_tiles(D, prec, tol, n, rule, chunk):
     err = float((a - b).abs().max() / b.abs().max())
     assert err <= TOL[prec], err
     assert torch.equal(a, cols.apply(x))  # fixed summation order
+
+
+@pytest.mark.parametrize("n,rule,chunk,tol", [
+    ((8, 8), (9, 10), 0, 0.0),        # the smallest fine grid: 2 x 2 blocks, footprints wrap
+    ((12, 24), (31, 34), 5, 0.0),     # units of one group, many partial blocks
+    ((48, 16), (64, 66), 70, 1e-4),   # w = 6, ragged
+    ((64, 64), (128, 128), 0, 0.0),
+    ((32, 96), (40, 512), 100000, 0.0),  # one unit per block
+])
+def test_blocks_match_tiles_2d(D, n, rule, chunk, tol):
+    # the type-1 stage of random node values by the 2D block spread and by the tile spread (the same
+    # taps in another order; no symbol in between that would amplify the rounding)
+    import torch
+    lo, ln = tuple(-0.25 * v for v in n), tuple(0.5 * v for v in n)
+    kw = dict(precision=1, nufft_tol=tol, nr=rule[0], nphi=rule[1])
+    blocks = D.Plan(2, n, lo, ln, (0.6, 0.0, 0.8), chunk=chunk, **kw)
+    tiles = D.Plan(2, n, lo, ln, (0.6, 0.0, 0.8), spread=1, **kw)
+    assert blocks.info.spread == 2 and tiles.info.spread == 1
+    # the nodes' processing order depends on the plan's tile: values go by original node index
+    q = {int(v): k for k, v in enumerate(tiles.node_order())}
+    perm = torch.tensor([q[int(v)] for v in blocks.node_order()], device="cuda")
+    g = torch.Generator("cuda").manual_seed(3)
+    c = torch.randn(int(tiles.info.nodes_used), 2, generator=g, device="cuda")
+    c = torch.view_as_complex(c)
+    a, b = blocks.type1(c[perm].contiguous()), tiles.type1(c)
+    err = float((a - b).abs().max() / b.abs().max())
+    assert err <= 1e-6, err
+    assert torch.equal(a, blocks.type1(c[perm].contiguous()))
