@@ -76,8 +76,19 @@ template <typename C> __host__ __device__ __forceinline__ C cmk(decltype(C::x) a
   r.y = b;
   return r;
 }
-template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return cmk<C>(a.x + b.x, a.y + b.y); }
-template <typename C> __device__ __forceinline__ C csub(C a, C b) { return cmk<C>(a.x - b.x, a.y - b.y); }
+// (FP32: both components in one packed instruction, rounded as the scalar operations)
+template <typename C> __device__ __forceinline__ C cadd(C a, C b) {
+  if constexpr (sizeof(C) == 8)
+    return __fadd2_rn(a, b);
+  else
+    return cmk<C>(a.x + b.x, a.y + b.y);
+}
+template <typename C> __device__ __forceinline__ C csub(C a, C b) {
+  if constexpr (sizeof(C) == 8)
+    return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+  else
+    return cmk<C>(a.x - b.x, a.y - b.y);
+}
 template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
   return cmk<C>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
@@ -309,20 +320,21 @@ int make_twiddles(Plan& p, int n);
 
 // ---- the GPE's Fourier passes on the plan's grid (gpe_fft.cuh) ---------------------------------
 // transforms are unnormalised, dir = -1: e^{-2 pi i jk/n}
-template <typename T> int gpe_forward(Plan& p, cx_t<T>* a, cudaStream_t s);  // a <- F a
-// a <- F^{-1} e^{i f |mu|^2} F a for the per-axis tables tab of e^{i f mu_d^2} - 1 (x, y, z); rho,
+template <typename T> int gpe_forward(Plan& p, const cx_t<T>* src, cx_t<T>* a, cudaStream_t s);  // a <- F src
+// a <- F^{-1} e^{i f |mu|^2} F src (src may be a) for the per-axis tables tab of e^{i f mu_d^2} - 1 (x, y, z); rho,
 // if not null, <- |a|^2
-template <typename T> int gpe_kinetic(Plan& p, cx_t<T>* a, const cx_t<T>* tab, T* rho, cudaStream_t s);
+template <typename T>
+int gpe_kinetic(Plan& p, const cx_t<T>* src, cx_t<T>* a, const cx_t<T>* tab, T* rho, cudaStream_t s);
 // one sweep of the gradient flow's fixed point,
-//   out <- F^{-1}[F(phi/dt + (alpha - W) cur) / (1/dt + alpha + |mu|^2/2)], W = V + beta rho + lambda Phi,
+//   out <- F^{-1}[F(phi/dt + (alpha - W) cur) / (1/dt + alpha + |mu|^2/2)],
 // and *change <- max |out - cur|^2 (FP64 bits, cleared by the caller); skipped when prev is not
 // null and the FP64 number at *prev is <= tol2
 template <typename T>
 struct GfSweep {
   const cx_t<T>*phi, *cur;
   cx_t<T>* out;
-  const T *V, *rho, *dip;  // dip may be null
-  T beta, lam, alpha, inv_dt;
+  const T* W;
+  T alpha, inv_dt;
   double inv_dt_alpha, ks[3];
   const unsigned long long* prev;
   double tol2;

@@ -58,7 +58,16 @@ __device__ __forceinline__ C tw_const(C x, int k) {
   const int idx = (k * (16 / R)) & 15;
   const double c = cos16(idx);
   const double s = DIR * sin16(idx);
-  return cmk<C>(mul_const(x.x, c) - mul_const(x.y, s), mul_const(x.x, s) + mul_const(x.y, c));
+  if constexpr (sizeof(C) == 8) {
+    // x c + (i x) s, each product head + tail as mul_const's, both components at once
+    const float ch = (float)c, cl = (float)(c - (double)ch), sh = (float)s, sl = (float)(s - (double)sh);
+    const C y = make_float2(-x.y, x.x);
+    const C p = __ffma2_rn(x, make_float2(ch, ch), __fmul2_rn(x, make_float2(cl, cl)));
+    const C q = __ffma2_rn(y, make_float2(sh, sh), __fmul2_rn(y, make_float2(sl, sl)));
+    return __fadd2_rn(p, q);
+  } else {
+    return cmk<C>(mul_const(x.x, c) - mul_const(x.y, s), mul_const(x.x, s) + mul_const(x.y, c));
+  }
 }
 
 // In-register R-point DFT (natural order in and out), radix-2 decimation in time.
@@ -246,7 +255,8 @@ struct MidStages<C, N, DIR, STOP, STOP, PRECISE> {
 
 template <int N>
 __host__ __device__ constexpr int lines_per_cta_base() {
-  return N <= 16 ? 128 : (N <= 128 ? 2048 / N : 4096 / N);
+  // powers of two, so that a CTA is whole warps and lines stay aligned
+  return N <= 16 ? 128 : N <= 32 ? 64 : N <= 64 ? 32 : N <= 256 ? 16 : N <= 512 ? 8 : N <= 1024 ? 4 : 2;
 }
 
 struct LineGeom {
@@ -367,9 +377,15 @@ __global__ void __launch_bounds__(LPB * Shape<N>::TPL)
 // Forward transform, pol.apply(ref, i, v) on every mode, inverse transform of the same line in one
 // pass: the line crosses global memory once each way instead of twice.  Where the last stage has
 // the first stage's radix (N = 16^k), a thread's modes are the inverse's first inputs and stay in
-// registers; otherwise they cross shared memory once.
+// registers; otherwise they cross shared memory once.  FP32 passes without twiddle tails are held to
+// 64 registers, so that a second 512-thread CTA loads while one transforms (256^3 split 1187 -> 1110
+// us); with the tails that spills (128^3 steps 1345 -> 1429 us).
 template <typename T, int N, int LPB, typename P>
-__global__ void __launch_bounds__(LPB * Shape<N>::TPL)
+constexpr int pair_ctas() {
+  return sizeof(T) == 4 && !P::kPrecise && 1024 / (LPB * Shape<N>::TPL) > 1 ? 1024 / (LPB * Shape<N>::TPL) : 1;
+}
+template <typename T, int N, int LPB, typename P>
+__global__ void __launch_bounds__(LPB * Shape<N>::TPL, pair_ctas<T, N, LPB, P>())
     k_fft_pair(P pol, const cx_t<T>* __restrict__ tw) {
   using C = cx_t<T>;
   using Ref = typename P::Ref;

@@ -70,6 +70,8 @@ __device__ __forceinline__ cx_t<T> expm1_i(T a) {
 template <typename T>
 __global__ void k_phase_tables(cx_t<T>* tab, G3 g, double f0, double f1) {
   const int total = g.n[0] + g.n[1] + g.n[2];
+  chain_release();
+  chain_wait();  // the last pass before may still read the tables
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 2 * total; k += gridDim.x * blockDim.x) {
     const int i = k < total ? k : k - total;
     int d = 0, l = i;
@@ -252,6 +254,18 @@ __global__ void k_red_energy(const cx_t<T>* __restrict__ psi, const T* __restric
   block_sum<4>(v, part + (size_t)blockIdx.x * kRedMax);
 }
 
+// sum |psi|^2
+template <typename T>
+__global__ void k_red_mass(const cx_t<T>* __restrict__ psi, long long total, double* part) {
+  double v[1] = {0};
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const cx_t<T> a = psi[i];
+    v[0] += (double)a.x * a.x + (double)a.y * a.y;
+  }
+  block_sum<1>(v, part + (size_t)blockIdx.x * kRedMax);
+}
+
 // sum |mu|^2 |psihat|^2
 template <typename T>
 __global__ void k_red_kinetic(const cx_t<T>* __restrict__ a, G3 g, double* part) {
@@ -271,18 +285,23 @@ __global__ void k_red_kinetic(const cx_t<T>* __restrict__ a, G3 g, double* part)
   block_sum<1>(v, part + (size_t)blockIdx.x * kRedMax);
 }
 
-// max and -min of W = V + beta |psi|^2 + lambda Phi, and a NaN/Inf flag
+// max and -min of W = V + beta rho + lambda Phi, and a NaN/Inf flag; W takes rho's place, for the
+// gradient flow's sweeps.  In the working precision: the range only sets the fixed point's shift alpha
+// (in FP64 the conversions and operations took 27 us at 96^3)
 template <typename T>
-__global__ void k_red_wrange(const T* __restrict__ V, const T* __restrict__ rho, const T* __restrict__ phi,
-                             double beta, double lam, long long total, double* part) {
-  double v[3] = {-INFINITY, -INFINITY, 0.0};
+__global__ void k_red_wrange(const T* __restrict__ V, T* rho, const T* __restrict__ phi, T beta, T lam,
+                             long long total, double* part) {
+  T hi = -(T)INFINITY, lo = (T)INFINITY;
+  bool bad = false;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    const double w = (double)V[i] + beta * (double)rho[i] + (phi ? lam * (double)phi[i] : 0.0);
-    if (!isfinite(w)) v[2] = 1.0;
-    v[0] = fmax(v[0], w);
-    v[1] = fmax(v[1], -w);
+    const T w = V[i] + beta * rho[i] + (phi ? lam * phi[i] : (T)0);
+    rho[i] = w;
+    bad = bad || !isfinite(w);
+    hi = w > hi ? w : hi;
+    lo = w < lo ? w : lo;
   }
+  double v[3] = {(double)hi, -(double)lo, bad ? 1.0 : 0.0};
   block_max<3>(v, part + (size_t)blockIdx.x * kRedMax);
 }
 
@@ -418,15 +437,13 @@ struct Gpe {
 
   // the two tables of kinetic() for e^{i f0 |mu|^2} and e^{i f1 |mu|^2}
   int phase_tables(double f0, double f1) {
-    k_phase_tables<T><<<8, kThreads, 0, s>>>(static_cast<C*>(p.d_kin), g, f0, f1);
-    DDI_LAUNCH_CHECK();
-    return DDI_OK;
+    return launch_chain(p, k_phase_tables<T>, 8, kThreads, 0, s, static_cast<C*>(p.d_kin), g, f0, f1);
   }
 
-  // a <- F^{-1} e^{i f_k |mu|^2} F a; rho, if not null, <- |a|^2
-  int kinetic(C* a, int k, T* rho = nullptr) {
+  // a <- F^{-1} e^{i f_k |mu|^2} F src (src may be a); rho, if not null, <- |a|^2
+  int kinetic(const C* src, C* a, int k, T* rho = nullptr) {
     const C* tab = static_cast<const C*>(p.d_kin) + (size_t)k * (p.n[0] + p.n[1] + p.n[2]);
-    return gpe_kinetic<T>(p, a, tab, rho, s);
+    return gpe_kinetic<T>(p, src, a, tab, rho, s);
   }
 
   int abs2(const C* a, T* out) {
@@ -457,8 +474,7 @@ struct Gpe {
     double sums[4];
     DDI_TRY(reduce(4, 0, sums));
     C* w = static_cast<C*>(p.d_work2);
-    DDI_CUDA(cudaMemcpyAsync(w, psi, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
-    DDI_TRY(gpe_forward<T>(p, w, s));
+    DDI_TRY(gpe_forward<T>(p, psi, w, s));
     k_red_kinetic<T><<<p.red_blocks, kThreads, 0, s>>>(w, g, p.d_red);
     DDI_LAUNCH_CHECK();
     double kin;
@@ -481,11 +497,11 @@ struct Gpe {
 
   // out <- a / ||a|| (out may be a)
   int normalise(const C* a, C* out, double* mass_out) {
-    k_red_energy<T><<<p.red_blocks, kThreads, 0, s>>>(a, static_cast<const T*>(p.d_rho), nullptr, N, p.d_red);
+    k_red_mass<T><<<p.red_blocks, kThreads, 0, s>>>(a, N, p.d_red);
     DDI_LAUNCH_CHECK();
-    double sums[4];
-    DDI_TRY(reduce(1, 0, sums));
-    const double m = p.dv * sums[0];
+    double sum;
+    DDI_TRY(reduce(1, 0, &sum));
+    const double m = p.dv * sum;
     if (!(m > 0.0) || !std::isfinite(m)) {
       set_error("state has zero or non-finite mass");
       return DDI_ERR_NONFINITE;
@@ -506,12 +522,13 @@ struct Gpe {
     return DDI_OK;
   }
 
-  int step(C* psi, const T* V, double beta, double lam, double dt, int nsteps) {
+  // nsteps Strang steps from src (which may be psi) into psi
+  int step(const C* src, C* psi, const T* V, double beta, double lam, double dt, int nsteps) {
     T* rho = static_cast<T*>(p.d_rho);
     T* phi = static_cast<T*>(p.d_phi);
     // consecutive half kinetic steps merge into one full step between nonlinear steps
     DDI_TRY(phase_tables(-0.25 * dt, -0.5 * dt));
-    DDI_TRY(kinetic(psi, 0, rho));
+    DDI_TRY(kinetic(src, psi, 0, rho));
     for (int k = 0; k < nsteps; ++k) {
       if (lam != 0.0) {
         DDI_TRY(run_ddi<T>(p, rho, phi, s));
@@ -520,7 +537,7 @@ struct Gpe {
       }
       DDI_TRY(launch_chain(p, k_nonlinear<T>, blocks_for(N), kThreads, 0, s, psi, V, phi, (T)beta, (T)lam, (T)dt, N));
       const bool more = k + 1 < nsteps;
-      DDI_TRY(kinetic(psi, more ? 1 : 0, more ? rho : nullptr));
+      DDI_TRY(kinetic(psi, psi, more ? 1 : 0, more ? rho : nullptr));
     }
     return DDI_OK;
   }
@@ -530,7 +547,7 @@ struct Gpe {
     T* g = static_cast<T*>(p.d_rho);
     T* phi = static_cast<T*>(p.d_phi);
     DDI_TRY(phase_tables(-0.25 * dt, -0.5 * dt));
-    DDI_TRY(kinetic(psi, 0));
+    DDI_TRY(kinetic(psi, psi, 0));
     for (int k = 0; k < nsteps; ++k) {
       DDI_TRY(launch_chain(p, k_step_density<T>, blocks_for(N), kThreads, 0, s, psi, g, nl, (T)dt, N));
       if (lam != 0.0) {
@@ -539,7 +556,7 @@ struct Gpe {
         DDI_CUDA(cudaMemsetAsync(phi, 0, sizeof(T) * N, s));
       }
       DDI_TRY(launch_chain(p, k_nonlinear_general<T>, blocks_for(N), kThreads, 0, s, psi, V, phi, (T)beta, (T)lam, (T)dt, nl, N));
-      DDI_TRY(kinetic(psi, k + 1 < nsteps ? 1 : 0));
+      DDI_TRY(kinetic(psi, psi, k + 1 < nsteps ? 1 : 0));
     }
     return DDI_OK;
   }
@@ -564,8 +581,8 @@ struct Gpe {
 
   // nsteps single Strang steps from psi0 into cur (cur != psi0), then J; the forward run alone
   int trap_forward(const C* psi0, C* cur, const T* V, double beta, double lam, double dt, int nsteps, double* J) {
-    DDI_CUDA(cudaMemcpyAsync(cur, psi0, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
-    for (int k = 0; k < nsteps; ++k) DDI_TRY(step(cur, V, beta, lam, dt, 1));
+    if (nsteps == 0) DDI_CUDA(cudaMemcpyAsync(cur, psi0, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
+    for (int k = 0; k < nsteps; ++k) DDI_TRY(step(k ? cur : psi0, cur, V, beta, lam, dt, 1));
     return observable(cur, nullptr, J);
   }
 
@@ -580,11 +597,11 @@ struct Gpe {
     C* seg = work + (size_t)ncp * N;              // [every]: one segment's step inputs
     C* cur = seg + (size_t)every * N;             // the running state
     C* cot = cur + N;                             // the cotangent
-    DDI_CUDA(cudaMemcpyAsync(cur, psi0, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
     for (int k = 0; k < nsteps; ++k) {
-      if (k % every == 0) DDI_CUDA(cudaMemcpyAsync(ckpt + (size_t)(k / every) * N, cur, sizeof(C) * N,
+      const C* from = k ? cur : psi0;
+      if (k % every == 0) DDI_CUDA(cudaMemcpyAsync(ckpt + (size_t)(k / every) * N, from, sizeof(C) * N,
                                                    cudaMemcpyDeviceToDevice, s));
-      DDI_TRY(step(cur, V, beta, lam, dt, 1));
+      DDI_TRY(step(from, cur, V, beta, lam, dt, 1));
     }
     DDI_TRY(observable(cur, cot, J));
     DDI_CUDA(cudaMemsetAsync(grad, 0, sizeof(T) * N, s));
@@ -593,9 +610,7 @@ struct Gpe {
       DDI_CUDA(cudaMemcpyAsync(seg, ckpt + (size_t)c * N, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
       for (int k = k0 + 1; k < k1; ++k) {
         C* prev = seg + (size_t)(k - 1 - k0) * N;
-        C* next = prev + N;
-        DDI_CUDA(cudaMemcpyAsync(next, prev, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
-        DDI_TRY(step(next, V, beta, lam, dt, 1));
+        DDI_TRY(step(prev, prev + N, V, beta, lam, dt, 1));
       }
       for (int k = k1 - 1; k >= k0; --k) DDI_TRY(adjoint(seg + (size_t)(k - k0) * N, cot, grad, V, beta, lam, dt));
     }
@@ -606,19 +621,18 @@ struct Gpe {
     C* psi1 = static_cast<C*>(p.d_psi1);
     T* rho = static_cast<T*>(p.d_rho);
     T* phi = static_cast<T*>(p.d_phi);
-    DDI_CUDA(cudaMemcpyAsync(psi1, psi_in, sizeof(C) * N, cudaMemcpyDeviceToDevice, s));
     DDI_TRY(phase_tables(-0.25 * dt, +0.25 * dt));
-    DDI_TRY(kinetic(psi1, 0, rho));
+    DDI_TRY(kinetic(psi_in, psi1, 0, rho));
     if (lam != 0.0) {
       DDI_TRY(run_ddi<T>(p, rho, phi, s));
     } else {
       DDI_CUDA(cudaMemsetAsync(phi, 0, sizeof(T) * N, s));
     }
-    DDI_TRY(kinetic(cot, 1));
+    DDI_TRY(kinetic(cot, cot, 1));
     DDI_TRY(launch_chain(p, k_adj_a<T>, blocks_for(N), kThreads, 0, s, psi1, V, rho, phi, cot, grad, rho, (T)beta, (T)lam, (T)dt, (T)p.dv, N));
     if (lam != 0.0) DDI_TRY(run_ddi<T>(p, rho, phi, s));
     DDI_TRY(launch_chain(p, k_adj_b<T>, blocks_for(N), kThreads, 0, s, psi1, rho, lam != 0.0 ? phi : nullptr, cot, (T)beta, (T)lam, N));
-    return kinetic(cot, 1);
+    return kinetic(cot, cot, 1);
   }
 
   int ground_state(C* phi0, const T* V, double beta, double lam, double dt, double tol, int rule,
@@ -638,7 +652,8 @@ struct Gpe {
       // W = V + beta |phi|^2 + lambda Phi(|phi|^2) and alpha = (max W + min W) / 2
       DDI_TRY(abs2(phi0, rho));
       if (lam != 0.0) DDI_TRY(run_ddi<T>(p, rho, dip, s));
-      k_red_wrange<T><<<p.red_blocks, kThreads, 0, s>>>(V, rho, lam != 0.0 ? dip : nullptr, beta, lam, N, p.d_red);
+      k_red_wrange<T><<<p.red_blocks, kThreads, 0, s>>>(V, rho, lam != 0.0 ? dip : nullptr, (T)beta, (T)lam, N,
+                                                         p.d_red);
       DDI_LAUNCH_CHECK();
       double wr[3];
       DDI_TRY(reduce(3, 1, wr));
@@ -652,11 +667,7 @@ struct Gpe {
       // first batch is the last step's count (it varies slowly along the flow)
       GfSweep<T> w{};
       w.phi = phi0;
-      w.V = V;
-      w.rho = rho;
-      w.dip = lam != 0.0 ? dip : nullptr;
-      w.beta = (T)beta;
-      w.lam = (T)lam;
+      w.W = rho;  // left there by k_red_wrange
       w.alpha = (T)alpha;
       w.inv_dt = (T)(1.0 / dt);
       w.inv_dt_alpha = 1.0 / dt + alpha;
@@ -764,10 +775,12 @@ int gpe_step(ddi_plan plan, void* psi, const void* V, double beta, double lambda
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (plan->p.prec == DDI_FP64) {
       Gpe<double> g(plan->p, s);
-      return g.step(static_cast<double2*>(psi), static_cast<const double*>(V), beta, lambda, dt, nsteps);
+      return g.step(static_cast<double2*>(psi), static_cast<double2*>(psi), static_cast<const double*>(V), beta, lambda,
+                    dt, nsteps);
     }
     Gpe<float> g(plan->p, s);
-    return g.step(static_cast<float2*>(psi), static_cast<const float*>(V), beta, lambda, dt, nsteps);
+    return g.step(static_cast<float2*>(psi), static_cast<float2*>(psi), static_cast<const float*>(V), beta, lambda, dt,
+                  nsteps);
   });
 }
 

@@ -35,18 +35,19 @@ struct GpePolicy : PolicyBase {
   static constexpr bool kPrecise = true;
 };
 
-// rows along x, in place; RHO: also writes |v|^2 of what it stores
+// rows along x, from src to data (they may be the same); RHO: also writes |v|^2 of what it stores
 template <typename T, bool RHO>
 struct GridX : GpePolicy {
   using C = cx_t<T>;
   using Ref = int;  // grids hold < 2^31 points
+  const C* src;
   C* data;
   T* rho;
   GridDims3 d;
   __host__ __device__ long long nlines() const { return (long long)d.n[1] * d.n[2]; }
   static constexpr bool kStrided = false;
   __device__ Ref ref(long long L) const { return (int)L * d.n[0]; }
-  __device__ C load(Ref r, int i) const { return __ldg(data + (r + i)); }
+  __device__ C load(Ref r, int i) const { return __ldg(src + (r + i)); }
   __device__ void store(Ref r, int i, C v, Acc&) const {
     data[r + i] = v;
     if (RHO) rho[r + i] = v.x * v.x + v.y * v.y;
@@ -112,15 +113,15 @@ struct GfSkip {
   __device__ bool done() const { return prev && __longlong_as_double((long long)*prev) <= tol2; }
 };
 
-// x forward of phi/dt + (alpha - W) cur, W = V + beta rho + lambda Phi
+// x forward of phi/dt + (alpha - W) cur
 template <typename T>
 struct GfRhsX : GpePolicy {
   using C = cx_t<T>;
   using Ref = int;  // grids hold < 2^31 points
   const C *phi, *cur;
   C* out;
-  const T *V, *rho, *dip;
-  T beta, lam, alpha, inv_dt;
+  const T* W;
+  T alpha, inv_dt;
   GridDims3 d;
   GfSkip sk;
   __host__ __device__ long long nlines() const { return (long long)d.n[1] * d.n[2]; }
@@ -128,8 +129,7 @@ struct GfRhsX : GpePolicy {
   static constexpr bool kStrided = false;
   __device__ Ref ref(long long L) const { return (int)L * d.n[0]; }
   __device__ C load(Ref r, int i) const {
-    const T w = V[r + i] + beta * rho[r + i] + (dip ? lam * dip[r + i] : (T)0);
-    const T f = alpha - w;
+    const T f = alpha - __ldg(W + (r + i));
     const C a = phi[r + i], c = cur[r + i];
     return cmk<C>(a.x * inv_dt + f * c.x, a.y * inv_dt + f * c.y);
   }
@@ -233,23 +233,23 @@ GridDims3 grid_dims(const Plan& p) { return GridDims3{{p.n[0], p.n[1], p.n[2]}};
 }  // namespace
 
 template <typename T>
-int gpe_forward(Plan& p, cx_t<T>* a, cudaStream_t s) {
+int gpe_forward(Plan& p, const cx_t<T>* src, cx_t<T>* a, cudaStream_t s) {
   const GridDims3 d = grid_dims(p);
-  DDI_TRY((grid_pass<T, -1>(p, 0, GridX<T, false>{{}, a, nullptr, d}, s)));
+  DDI_TRY((grid_pass<T, -1>(p, 0, GridX<T, false>{{}, src, a, nullptr, d}, s)));
   for (int ax = 1; ax < p.dim; ++ax) DDI_TRY((grid_pass<T, -1>(p, ax, GridLines<T>{{}, a, d, ax}, s)));
   return DDI_OK;
 }
 
 template <typename T>
-int gpe_kinetic(Plan& p, cx_t<T>* a, const cx_t<T>* tab, T* rho, cudaStream_t s) {
+int gpe_kinetic(Plan& p, const cx_t<T>* src, cx_t<T>* a, const cx_t<T>* tab, T* rho, cudaStream_t s) {
   const GridDims3 d = grid_dims(p);
   const int last = p.dim - 1;
-  DDI_TRY((grid_pass<T, -1>(p, 0, GridX<T, false>{{}, a, nullptr, d}, s)));
+  DDI_TRY((grid_pass<T, -1>(p, 0, GridX<T, false>{{}, src, a, nullptr, d}, s)));
   if (last == 2) DDI_TRY((grid_pass<T, -1>(p, 1, GridLines<T>{{}, a, d, 1}, s)));
   DDI_TRY((grid_pass<T, 0>(p, last, KineticPair<T>{{{}, a, d, last}, tab, 1.0 / (double)p.grid_points()}, s)));
   if (last == 2) DDI_TRY((grid_pass<T, +1>(p, 1, GridLines<T>{{}, a, d, 1}, s)));
-  if (rho) return grid_pass<T, +1>(p, 0, GridX<T, true>{{}, a, rho, d}, s);
-  return grid_pass<T, +1>(p, 0, GridX<T, false>{{}, a, nullptr, d}, s);
+  if (rho) return grid_pass<T, +1>(p, 0, GridX<T, true>{{}, a, a, rho, d}, s);
+  return grid_pass<T, +1>(p, 0, GridX<T, false>{{}, a, a, nullptr, d}, s);
 }
 
 template <typename T>
@@ -258,8 +258,7 @@ int gpe_gf_sweep(Plan& p, const GfSweep<T>& w, cudaStream_t s) {
   const int last = p.dim - 1;
   const GfSkip sk{w.prev, w.tol2};
   DDI_TRY((grid_pass<T, -1>(p, 0,
-                            GfRhsX<T>{{}, w.phi, w.cur, w.out, w.V, w.rho, w.dip, w.beta, w.lam, w.alpha, w.inv_dt, d, sk},
-                            s)));
+                            GfRhsX<T>{{}, w.phi, w.cur, w.out, w.W, w.alpha, w.inv_dt, d, sk}, s)));
   if (last == 2) DDI_TRY((grid_pass<T, -1>(p, 1, GfLines<T>{{{}, w.out, d, 1}, sk}, s)));
   DDI_TRY((grid_pass<T, 0>(p, last,
                            GfSolvePair<T>{{{}, w.out, d, last},
