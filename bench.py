@@ -193,10 +193,11 @@ def run_reference(args):
 # fine grid 2N per axis, complex 8 B): each pass moves the data it must read and write
 # once; the padded / cropped passes touch only the block they need.
 def fp64_path_figures(torch, stream, ms, w):
-    """The FP64 path is bound by FP64 arithmetic on this part: its model FLOPs per DDI
-    (interpolation 4 and spread 5 flops per tap, w^3 taps per processed node, plus the six
-    fine-grid FFT passes at 5 n log2 n each) over its time, beside a probed FP64 peak
-    (cuBLAS DGEMM 4096^3, best of 5)."""
+    """The FP64 path is bound by FP64 arithmetic on this part: the model FLOPs of the direct sum
+    over taps (interpolation 4 and spread 5 flops per tap, w^3 taps per processed node, plus
+    the six fine-grid FFT passes at 5 n log2 n each) over its time, beside a probed FP64 peak
+    (cuBLAS DGEMM 4096^3, best of 5).  The path sums a ring's nodes before psi_z and executes
+    about a fifth of those operations, so the fraction can exceed 1."""
     mh = N * 64 * 128 // 2
     taps = mh * w ** 3 * 9
     nf = 2 * N

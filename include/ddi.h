@@ -101,10 +101,10 @@ typedef struct {
                           tiles); DDI_SPREAD_TILES => owner-computes tile planes in shared memory (`tile`,
                           `chunk`); DDI_SPREAD_COLUMNS => columns of the fine grid whose planes along the
                           last axis a warp accumulates in registers: 8 x 8 cells in x-y running along z
-                          (3D), 8 cells in x running along y (2D).  Applies to FP32 plans whose fine grid
-                          is a multiple of 8 in x (3D: and in y) and at least w + 7 cells in x (3D: w + 7
-                          in y and w in z; 2D: w in y), and not to compensated 2D plans; DDI_ERR_ARG
-                          otherwise; `chunk` = visits per work item.  The automatic choice also gives
+                          (3D), 8 cells in x running along y and taken in blocks of 8 x 8 cells (2D).
+                          Applies to FP32 plans whose fine grid is a multiple of 8 in x and y and at least
+                          w + 7 cells in x and y (3D: and w in z), and not to compensated 2D plans;
+                          DDI_ERR_ARG otherwise; `chunk` = visits per work item.  The automatic choice also gives
                           columns to FP64 3D plans of 2048 processed nodes and more whose fine grid
                           fits (at least w + 7 cells in x and y, multiples of 8) and whose `tile` is
                           left at 0 */
