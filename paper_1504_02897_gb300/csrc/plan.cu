@@ -742,10 +742,9 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
   choose_tile(p);
   const int dim = d.dim, W = p.w;
   if (d.spread == DDI_SPREAD_COLUMNS && !columns_apply(p)) {
-    set_error("the column spread needs an FP32 plan whose fine grid is a multiple of %d cells in x (3D: %d x %d in "
-              "x-y) and at least w + %d cells along x (3D: w + %d along y and w along z; 2D: w along y), and no "
-              "compensated arithmetic in 2D",
-              kColX, kColX, kColY, kColX - 1, kColY - 1);
+    set_error("the column spread needs an FP32 plan whose fine grid is a multiple of %d x %d cells in x-y and at least "
+              "w + %d cells along x and y (3D: w along z), and no compensated arithmetic in 2D",
+              kColX, kColY, kColX - 1);
     return DDI_ERR_ARG;
   }
   // automatic choice: columns where they apply (2D: blocks of 8 x 8 cells, faster
