@@ -259,18 +259,6 @@ __host__ __device__ constexpr int lines_per_cta_base() {
   return N <= 16 ? 128 : N <= 32 ? 64 : N <= 64 ? 32 : N <= 256 ? 16 : N <= 512 ? 8 : N <= 1024 ? 4 : 2;
 }
 
-struct LineGeom {
-  long long nlines;
-  long long l1;    // line L -> (L / l1, L % l1)
-  long long s_hi;  // offset of (L / l1)
-  long long s_lo;  // offset of (L % l1)
-  long long se;    // element stride along the line
-};
-
-__device__ __forceinline__ long long line_off(const LineGeom& g, long long L) {
-  return (L / g.l1) * g.s_hi + (L % g.l1) * g.s_lo;
-}
-
 // Generic batched-line FFT: a policy P supplies nlines(), ref(L) (the line's addresses,
 // computed once per line by one thread), load(ref, i) /
 // store(ref, i, v, acc) for element i of the line, skip() (the whole pass is not needed), an

@@ -15,22 +15,21 @@
 // the plan, so the per-axis kernel values psi_d(l - s_q) of every node are built once
 // (FP64 on the host, rounded to the working precision) and read here.
 //
-// Launches (fft_nufft.cu holds the FFT passes):
-//   forward FFT x (pad + deconvolution fused), y, z, pruned to the padded block
-//   3D plans that spread by columns interpolate by columns too (columns.cu) where that is faster;
-//   the others:
-//   k_interp    8 (w <= 8) or 16 lanes per node: f_q = sum over the w^d taps of psi F,
-//               each footprint row read as one contiguous segment; writes
-//               c_q = 2 h^d W_q f_q
-//   k_spread    owner-computes spread over work units (tile, z-plane in 3D; tile in
-//               2D): a warp takes a unit, streams the nodes whose taps reach that plane
-//               (ranges built by the plan) and adds c psi_z psi_y psi_x into its
-//               shared-memory plane with plain read-modify-writes (no other unit owns
-//               those cells).  Every plane is written once; long units are split into
-//               partial planes
-//   k_reduce    sums the partial planes of split units
-//   inverse FFT z, y, x (pruned to the cropped block; x fused with crop, deconvolution
-//               and real part)
+// Launches (fft_nufft.cuh holds the FFT passes, columns.cu the column and block kernels):
+//   forward FFT (3D: y with pad + deconvolution fused, x, z; 2D: x, y), pruned to the padded
+//               block and to the lines that hold taps
+//   interpolation: c_q = 2 h^d W_q f_q, f_q = sum over the w^d taps of psi F.  3D plans that spread
+//               by columns interpolate by columns too where that is faster; the others gather:
+//               k_interp (3D) and k_interp2 (2D), 8 (w <= 8) or 16 lanes per node, each footprint
+//               row read as one contiguous segment
+//   spread      by columns (3D) or blocks (2D), or by tiles: k_spread, owner-computes over work
+//               units (tile, z-plane in 3D; tile in 2D): a warp takes a unit, streams the nodes
+//               whose taps reach that plane (ranges built by the plan) and adds c psi_z psi_y psi_x
+//               into its shared-memory plane with plain read-modify-writes (no other unit owns
+//               those cells).  Every plane is written once; long units are split into partial
+//               planes that k_reduce sums
+//   inverse FFT (3D: z, x, y; 2D: y, x), pruned likewise; the last pass fused with crop,
+//               deconvolution and real part
 #include <algorithm>
 #include <climits>
 #include <cmath>

@@ -4,8 +4,9 @@
 // the quadrature (Sec. 2.1, Eq. DDI-Trun1): the node tables (tables.cpp), for each node
 // of one half of the antipodally closed set its first fine-grid tap, its kernel values
 // psi_d at the w taps of each axis (FP64, rounded once) and its scale 2 h^d W_q, the
-// deconvolution factors, the spread work list (per fine-grid tile, the nodes whose taps
-// reach it, in order of their start relative to the tile, and the work units: one per
+// deconvolution factors, the spread work list (3D columns and 2D blocks: the groups of visits
+// of columns.cuh and the units that take them; tiles: per fine-grid tile, the nodes whose taps
+// reach it, in order of their start relative to the tile, and the work units, one per
 // tile plane, long ones cut into pieces that write partial planes), and all
 // device workspace.  ddi_plan_create is the only call that allocates.
 #include <algorithm>
