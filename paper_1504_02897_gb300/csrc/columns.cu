@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_spread
   const int lx = lane & 7, ly = lane >> 3;
   const int nfx = a.nf[0], nfz = a.nf[2];
   const long long plane = (long long)nfx * a.nf[1];
-  const C* __restrict__ cg = static_cast<const C*>(a.c);
+  const C* cg = static_cast<const C*>(a.c);
   // units are taken from a counter, the first one by position; the next unit's index, entry and
   // first group are requested while the current one is being worked on
   const int nwarps = gridDim.x * (blockDim.x >> 5);
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_spread
     // group images are copied one ahead, node values read one ahead, node indices two ahead
     int nnext = n1;
     C cnext = zero;
-    if (n0 >= 0) cnext = __ldg(cg + n0);
+    if (n0 >= 0) cnext = chain_load(cg + n0);
     // after the last group: one more turn that only writes the planes left up to z1
     for (int gi = U.lo; gi <= U.hi; ++gi) {
       const bool end = gi == U.hi;
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_spread
       if (!end) {
         if (gi + 1 < U.hi) {
           copy_image<I::BYTES>(sm + (buf ^ 1) * I::BYTES, a.image + (size_t)(gi + 1) * I::BYTES, lane);
-          if (nnext >= 0) cnext = __ldg(cg + nnext);
+          if (nnext >= 0) cnext = chain_load(cg + nnext);
           nnext = gi + 2 < U.hi ? __ldg(a.nodes + (size_t)(gi + 2) * 32 + lane) : -1;
         }
         cp_async_commit();
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kColThreads3, 8) k_spread_block(BlockArgs a) {
       copy_image<I::BYTES>(sm, a.image + (size_t)U.lo * I::BYTES, lane);
       const int n0 = __ldg(a.nodes + (size_t)U.lo * 32 + lane);
       if (U.lo + 1 < U.hi) nnext = __ldg(a.nodes + (size_t)(U.lo + 1) * 32 + lane);
-      if (n0 >= 0) cnext = __ldg(a.c + n0);
+      if (n0 >= 0) cnext = chain_load(a.c + n0);
     }
     cp_async_commit();
     for (int gi = U.lo; gi < U.hi; ++gi) {
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kColThreads3, 8) k_spread_block(BlockArgs a) {
       cnext = zero;
       if (gi + 1 < U.hi) {
         copy_image<I::BYTES>(sm + (buf ^ 1) * I::BYTES, a.image + (size_t)(gi + 1) * I::BYTES, lane);
-        if (nnext >= 0) cnext = __ldg(a.c + nnext);
+        if (nnext >= 0) cnext = chain_load(a.c + nnext);
         nnext = gi + 2 < U.hi ? __ldg(a.nodes + (size_t)(gi + 2) * 32 + lane) : -1;
       }
       cp_async_commit();
@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(kColThreads3, 8) k_spread_block(BlockArgs a) {
 // (deterministic); a lane sums two cells, eight loads in flight at a time.
 template <typename T>
 __global__ void __launch_bounds__(256)
-    k_reduce_col3(const ColRed* __restrict__ red, int nred, int nlong, const cx_t<T>* __restrict__ partial,
+    k_reduce_col3(const ColRed* __restrict__ red, int nred, int nlong, const cx_t<T>* partial,
                   cx_t<T>* __restrict__ fine, int nfx, int nfy, int ncx) {
   using C = cx_t<T>;
   __shared__ C sh[7][64];
@@ -567,8 +567,8 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_interp
     const C* col = static_cast<const C*>(a.fine) + (long long)y * nfx + x;
     auto load = [&](int z, C& v0, C& v1) {
       const C* at = col + (z >= nfz ? z - nfz : z) * plane;
-      v0 = ok0 ? __ldg(at) : zero;
-      v1 = ok1 ? __ldg(at + 4 * nfx) : zero;
+      v0 = ok0 ? chain_load(at) : zero;
+      v1 = ok1 ? chain_load(at + 4 * nfx) : zero;
     };
     C r0[W / 2], i0[W / 2], r1[W / 2], i1[W / 2];  // planes 2 q and 2 q + 1 (mod W)
     C p0 = zero, p1 = zero;                          // plane zl, requested ahead
@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_interp
 // c_q = 2 h^d W_q times the sum of the node's shares, in the order of its columns
 template <typename T>
 __global__ void __launch_bounds__(256)
-    k_node_sum3(const int* __restrict__ off, const int* __restrict__ pos, const cx_t<T>* __restrict__ share,
+    k_node_sum3(const int* __restrict__ off, const int* __restrict__ pos, const cx_t<T>* share,
                 const T* __restrict__ scale, cx_t<T>* __restrict__ c, int count) {
   using C = cx_t<T>;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -285,8 +285,18 @@ struct Plan {
 // 1525 -> 1385 us.  Not used inside batches, whose side streams fill the gaps, nor in FP64, whose
 // kernels are long (128^3 6.73 against 6.75 ms; rotating 64^3 steps were slower with it, 2.95
 // against 2.72 ms).
+//
+// Such a kernel is alive while the ones before it still write.  So what an evaluation or a caller writes
+// (the fine grid, node values, shares, partial planes, densities, states, traps, phase tables) is read
+// with coherent loads after chain_wait(): through chain_load() or a pointer that is not __restrict__.
+// ld.global.nc, which __ldg and const __restrict__ parameters give, is defined only for data that
+// nothing writes in the kernel's whole life: it is for the plan's constants (work lists, images, taps,
+// factors, twiddles, and the node scales, which ddi_plan_set_axes writes by an ordinary launch).
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// (a plain load: chain_wait's memory clobber keeps it behind the wait.  As a volatile ld.global.ca,
+// which the compiler cannot schedule, 192^3 took 869 us instead of 852)
+template <typename V> __device__ __forceinline__ V chain_load(const V* p) { return *p; }
 
 // Once per kernel and device: raises the kernel's dynamic shared memory limit to `smem` (the limit
 // belongs to the kernel, shared by every plan and thread: only raised).

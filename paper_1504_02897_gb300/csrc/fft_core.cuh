@@ -260,8 +260,8 @@ __host__ __device__ constexpr int lines_per_cta_base() {
 }
 
 // Generic batched-line FFT: a policy P supplies nlines(), ref(L) (the line's addresses,
-// computed once per line by one thread), load(ref, i) /
-// store(ref, i, v, acc) for element i of the line, skip() (the whole pass is not needed), an
+// computed once per line by one thread), load(ref, i), use(ref, i, v) (what becomes of a loaded
+// value, called after all of a thread's loads) / store(ref, i, v, acc) for element i of the line, skip() (the whole pass is not needed), an
 // accumulator Acc with finish(acc), begin() (once per thread, before the lines), and the constants
 //   kStrided   the lines' elements are strided in memory and neighbouring lines adjacent (else the
 //              element index is fastest)
@@ -281,6 +281,7 @@ struct PolicyBase {
   static constexpr bool kPrecise = false, kBlockIn = false, kBlockOut = false, kStrided = true;
   __device__ bool skip() const { return false; }
   __device__ void begin() const {}
+  template <typename Ref, typename C> __device__ C use(const Ref&, int, C v) const { return v; }
   __device__ void finish(const Acc&) const {}
 };
 
@@ -297,6 +298,9 @@ __device__ __forceinline__ void load_first(const P& pol, const Ref& ref, bool li
     else
       v[r] = live ? pol.load(ref, t + r * (N / R0)) : cmk<C>(0, 0);
   }
+#pragma unroll
+  for (int r = 0; r < R0; ++r)
+    if (!(P::kBlockIn && outside_block(r, R0)) && live) v[r] = pol.use(ref, t + r * (N / R0), v[r]);
 }
 // last stage: butterfly j's outputs are elements j + r NSL
 template <int N, int RL, int NSL, typename C, typename P, typename Ref>

@@ -27,8 +27,8 @@
 // symbol, inverse.
 // Grid positions that are not read are never written in the same evaluation, so no
 // zero-fill of the fine grid is needed.  Each CTA reads its own lines before it writes
-// them and no other CTA touches them, so the in-place passes may load through the
-// read-only data cache.
+// them and no other CTA of the pass touches them; the kernel before may still be writing them when
+// the pass starts, so they are read coherently (chain_load, common.cuh).
 #pragma once
 #include "fft_core.cuh"
 
@@ -126,7 +126,9 @@ __device__ __forceinline__ T deconv(const Geo<T>& g, const double* d, const YRef
   }
 }
 
-// an element of the density: its deconvolved value, with a NaN / Inf recorded
+// an element of the density: its deconvolved value, with a NaN / Inf recorded (a policy's use(), after
+// the loads: no load passes the atomic, and with each element loaded and recorded in turn the 256^3
+// pads took 121 us each instead of 93)
 template <typename T>
 __device__ __forceinline__ cx_t<T> pad_value(const Geo<T>& g, const double* d, const YRef<T>& r, int j, T v) {
   if (!isfinite(v) && *(volatile int*)g.nonfinite == 0) atomicOr(g.nonfinite, 1);
@@ -146,8 +148,10 @@ struct PadY : PolicyBase {
     if (blockIdx.x == 0 && threadIdx.x < 2) g.counters[threadIdx.x] = 0;
   }
   __device__ C load(const Ref& r, int i) const {
-    const int jy = g.ay.grid_of(i);
-    return pad_value<T>(g, g.dc + g.ax.n, r, jy, __ldg(rho + (r.grid + jy * g.ax.n)));
+    return cmk<C>(chain_load(rho + (r.grid + g.ay.grid_of(i) * g.ax.n)), (T)0);
+  }
+  __device__ C use(const Ref& r, int i, C v) const {
+    return pad_value<T>(g, g.dc + g.ax.n, r, g.ay.grid_of(i), v.x);
   }
   __device__ void store(const Ref& r, int i, C v, Acc&) const {
     if (g.in_yr(i)) g.fine[r.fine + i * g.ax.nf] = v;
@@ -167,7 +171,7 @@ struct CropY : PolicyBase {
   __device__ Ref ref(long long L) const { return y_ref<T>(g, L); }
   __device__ C load(const Ref& r, int i) const {
     if (!g.in_yr(i)) return cmk<C>((T)0, (T)0);
-    return __ldg(g.fine + (r.fine + i * g.ax.nf));
+    return chain_load(g.fine + (r.fine + i * g.ax.nf));
   }
   __device__ void store(const Ref& r, int i, C v, Acc&) const {
     const int jy = g.ay.grid_of(i);
@@ -202,10 +206,8 @@ struct PadX2 : PolicyBase {
   __device__ void begin() const {
     if (blockIdx.x == 0 && threadIdx.x < 2) g.counters[threadIdx.x] = 0;
   }
-  __device__ C load(const Ref& r, int i) const {
-    const int jx = g.ax.grid_of(i);
-    return pad_value<T>(g, g.dc, r, jx, __ldg(rho + (r.grid + jx)));
-  }
+  __device__ C load(const Ref& r, int i) const { return cmk<C>(chain_load(rho + (r.grid + g.ax.grid_of(i))), (T)0); }
+  __device__ C use(const Ref& r, int i, C v) const { return pad_value<T>(g, g.dc, r, g.ax.grid_of(i), v.x); }
   __device__ void store(const Ref& r, int i, C v, Acc&) const { g.fine[r.fine + i] = v; }
 };
 
@@ -219,7 +221,7 @@ struct ColY2 : PolicyBase {
   __device__ Ref ref(long long L) const { return (int)L; }
   __device__ C load(Ref r, int i) const {
     if (!FWD && !g.in_yr(i)) return cmk<C>((T)0, (T)0);
-    return __ldg(g.fine + (i * g.ax.nf + r));
+    return chain_load(g.fine + (i * g.ax.nf + r));
   }
   __device__ void store(Ref r, int i, C v, Acc&) const {
     if (!FWD || g.in_yr(i)) g.fine[i * g.ax.nf + r] = v;
@@ -235,7 +237,7 @@ struct CropX2 : PolicyBase {
   T* phi;
   __host__ __device__ long long nlines() const { return g.ay.n; }
   __device__ Ref ref(long long L) const { return x_ref<T>(g, L); }
-  __device__ C load(const Ref& r, int i) const { return __ldg(g.fine + (r.fine + i)); }
+  __device__ C load(const Ref& r, int i) const { return chain_load(g.fine + (r.fine + i)); }
   __device__ void store(const Ref& r, int i, C v, Acc&) const {
     const int jx = g.ax.grid_of(i);
     phi[r.grid + jx] = deconv<T>(g, g.dc, r, jx, v.x);
@@ -257,10 +259,10 @@ struct RowX : PolicyBase {
     return g.fidx(g.az.fine_of(q), g.yr_line((int)L - q * g.nyr), 0);
   }
   __device__ C load(Ref r, int i) const {
-    if (FWD) return __ldg(g.fine + (r + g.ax.grid_of(i)));
+    if (FWD) return chain_load(g.fine + (r + g.ax.grid_of(i)));
     // x lines outside the taps' range were neither written by the spread nor transformed
     if (!g.in_xr(i)) return cmk<C>((T)0, (T)0);
-    return __ldg(g.fine + (r + i));
+    return chain_load(g.fine + (r + i));
   }
   __device__ void store(Ref r, int i, C v, Acc&) const {
     if (!FWD)
@@ -282,7 +284,7 @@ struct ColZ : PolicyBase {
     const int q = (int)((unsigned)L / (unsigned)g.nxr);
     return g.yr_line(q) * g.ax.nf + g.xr_line((int)L - q * g.nxr);
   }
-  __device__ C load(Ref r, int i) const { return __ldg(g.fine + (i * g.sz + r)); }
+  __device__ C load(Ref r, int i) const { return chain_load(g.fine + (i * g.sz + r)); }
   __device__ void store(Ref r, int i, C v, Acc&) const { g.fine[i * g.sz + r] = v; }
 };
 
@@ -342,7 +344,7 @@ struct SmoothZ : PolicyBase {
     return Ref{ly * g.ax.nf + lx, sy.k_of(0, lx, g.ax.nf), sy.k_of(1, ly, g.ay.nf),
                sy.join(sy.em1[lx], sy.em1[g.ax.nf + ly]), (T)(twice ? 2 : 1), twice && 2 * lx == g.ax.nf};
   }
-  __device__ C load(const Ref& r, int i) const { return __ldg(g.fine + (i * g.sz + r.col)); }
+  __device__ C load(const Ref& r, int i) const { return chain_load(g.fine + (i * g.sz + r.col)); }
   __device__ C apply(const Ref& r, int i, C v) const {
     const T kz = sy.k_of(2, i, g.az.nf);
     const T em = sy.join(r.em, __ldg(sy.em1 + g.ax.nf + g.ay.nf + i));

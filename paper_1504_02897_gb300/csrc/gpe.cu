@@ -87,7 +87,7 @@ __global__ void k_phase_tables(cx_t<T>* tab, G3 g, double f0, double f1) {
 }
 
 template <typename T>
-__global__ void k_abs2(const cx_t<T>* __restrict__ psi, T* __restrict__ rho, long long total) {
+__global__ void k_abs2(const cx_t<T>* psi, T* __restrict__ rho, long long total) {
   chain_release();
   chain_wait();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -123,7 +123,7 @@ __device__ __forceinline__ T expm1t(T a) {
 
 // g(phi) = int_0^dt h(phi, tau) d tau, the density whose DDI is G / lambda
 template <typename T>
-__global__ void k_step_density(const cx_t<T>* __restrict__ psi, T* __restrict__ gout, NonlinParams nl, T dt,
+__global__ void k_step_density(const cx_t<T>* psi, T* __restrict__ gout, NonlinParams nl, T dt,
                                long long total) {
   chain_release();
   chain_wait();
@@ -151,7 +151,7 @@ __global__ void k_step_density(const cx_t<T>* __restrict__ psi, T* __restrict__ 
 
 // psi <- psi exp(-i [dt V + H(phi) + lambda Phi_g]) exp(-F(phi)), phi = |psi|^2
 template <typename T>
-__global__ void k_nonlinear_general(cx_t<T>* __restrict__ psi, const T* __restrict__ V, const T* __restrict__ phig,
+__global__ void k_nonlinear_general(cx_t<T>* __restrict__ psi, const T* V, const T* phig,
                                     T beta, T lam, T dt, NonlinParams nl, long long total) {
   chain_release();
   chain_wait();
@@ -188,7 +188,7 @@ __global__ void k_nonlinear_general(cx_t<T>* __restrict__ psi, const T* __restri
 
 // psi <- psi exp(-i dt (V + beta |psi|^2 + lambda Phi)) (Case I of Eq. tssp2)
 template <typename T>
-__global__ void k_nonlinear(cx_t<T>* __restrict__ psi, const T* __restrict__ V, const T* __restrict__ phi, T beta,
+__global__ void k_nonlinear(cx_t<T>* __restrict__ psi, const T* V, const T* phi, T beta,
                             T lam, T dt, long long total) {
   chain_release();
   chain_wait();
@@ -359,8 +359,8 @@ __global__ void k_scale(const cx_t<T>* a, cx_t<T>* b, T s, long long total) {
 //   e = exp(-i dt theta); r = Re(conj(-i dt psi1 e) g2); grad += dv r;
 //   cot <- conj(e) g2; rout <- r
 template <typename T>
-__global__ void k_adj_a(const cx_t<T>* __restrict__ psi1, const T* __restrict__ V, const T* rho,
-                        const T* __restrict__ phi, cx_t<T>* __restrict__ cot, T* __restrict__ grad,
+__global__ void k_adj_a(const cx_t<T>* psi1, const T* V, const T* rho,
+                        const T* phi, cx_t<T>* __restrict__ cot, T* __restrict__ grad,
                         T* rout, T beta, T lam, T dt, T dv, long long total) {
   chain_release();
   chain_wait();
@@ -382,7 +382,7 @@ __global__ void k_adj_a(const cx_t<T>* __restrict__ psi1, const T* __restrict__ 
 
 // adjoint, part B: cot += 2 psi1 (beta r + lambda Phi_r)
 template <typename T>
-__global__ void k_adj_b(const cx_t<T>* __restrict__ psi1, const T* __restrict__ r, const T* __restrict__ phir,
+__global__ void k_adj_b(const cx_t<T>* psi1, const T* r, const T* phir,
                         cx_t<T>* __restrict__ cot, T beta, T lam, long long total) {
   chain_release();
   chain_wait();

@@ -47,7 +47,7 @@ struct GridX : GpePolicy {
   __host__ __device__ long long nlines() const { return (long long)d.n[1] * d.n[2]; }
   static constexpr bool kStrided = false;
   __device__ Ref ref(long long L) const { return (int)L * d.n[0]; }
-  __device__ C load(Ref r, int i) const { return __ldg(src + (r + i)); }
+  __device__ C load(Ref r, int i) const { return chain_load(src + (r + i)); }
   __device__ void store(Ref r, int i, C v, Acc&) const {
     data[r + i] = v;
     if (RHO) rho[r + i] = v.x * v.x + v.y * v.y;
@@ -69,7 +69,7 @@ struct GridLines : GpePolicy {
     return q * d.n[0] * d.n[1] + ((int)L - q * d.n[0]);
   }
   __device__ int at(Ref r, int i) const { return r + i * (axis == 1 ? d.n[0] : d.n[0] * d.n[1]); }
-  __device__ C load(Ref r, int i) const { return __ldg(data + at(r, i)); }
+  __device__ C load(Ref r, int i) const { return chain_load(data + at(r, i)); }
   __device__ void store(Ref r, int i, C v, Acc&) const { data[at(r, i)] = v; }
 };
 
@@ -96,7 +96,7 @@ struct KineticPair : GridLines<T> {
   }
   __device__ C load(const Ref& r, int i) const { return GridLines<T>::load(r.off, i); }
   __device__ C apply(const Ref& r, int i, C v) const {
-    const C Z = __ldg(tab + this->d.n[0] + (this->axis == 2 ? this->d.n[1] : 0) + i);
+    const C Z = chain_load(tab + this->d.n[0] + (this->axis == 2 ? this->d.n[1] : 0) + i);
     const C E = cadd(cadd(r.P, Z), cmul(Z, r.P));
     const C o = cadd(v, cmul(v, E));
     return cmk<C>(scale_const(o.x, inv_n), scale_const(o.y, inv_n));
@@ -129,7 +129,7 @@ struct GfRhsX : GpePolicy {
   static constexpr bool kStrided = false;
   __device__ Ref ref(long long L) const { return (int)L * d.n[0]; }
   __device__ C load(Ref r, int i) const {
-    const T f = alpha - __ldg(W + (r + i));
+    const T f = alpha - chain_load(W + (r + i));
     const C a = phi[r + i], c = cur[r + i];
     return cmk<C>(a.x * inv_dt + f * c.x, a.y * inv_dt + f * c.y);
   }
@@ -195,7 +195,7 @@ struct GfChangeX : GpePolicy {
   __device__ bool skip() const { return sk.done(); }
   static constexpr bool kStrided = false;
   __device__ Ref ref(long long L) const { return (int)L * d.n[0]; }
-  __device__ C load(Ref r, int i) const { return __ldg(data + (r + i)); }
+  __device__ C load(Ref r, int i) const { return chain_load(data + (r + i)); }
   __device__ void store(Ref r, int i, C v, Acc& a) const {
     data[r + i] = v;
     const C y = cur[r + i];

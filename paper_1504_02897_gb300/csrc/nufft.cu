@@ -99,7 +99,7 @@ __device__ __forceinline__ void load_taps(const T* __restrict__ src, T (&dst)[W]
 // (at most 64 registers in FP32, so that 4 CTAs per SM keep enough loads in flight)
 template <typename T, int W>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
-    k_interp(const cx_t<T>* __restrict__ fine, const ushort4* __restrict__ l0, const T* __restrict__ psi,
+    k_interp(const cx_t<T>* fine, const ushort4* __restrict__ l0, const T* __restrict__ psi,
              const T* __restrict__ scale, cx_t<T>* __restrict__ cout, long long count, GridDims g) {
   using C = cx_t<T>;
   constexpr int XL = W <= 8 ? 8 : 16;
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
     T zr = 0, zi = 0;
 #pragma unroll
     for (int ay = 0; ay < W; ++ay) {
-      const C v = __ldg(zp + yoff[ay]);
+      const C v = chain_load(zp + yoff[ay]);
       zr += ky[ay] * v.x;
       zi += ky[ay] * v.y;
     }
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
 // latency-bound: the node's data from memory, then its taps, once per thread (1024^2 143 -> 107 us).
 template <typename T, int W>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
-    k_interp2(const cx_t<T>* __restrict__ fine, const ushort4* __restrict__ l0, const T* __restrict__ psi,
+    k_interp2(const cx_t<T>* fine, const ushort4* __restrict__ l0, const T* __restrict__ psi,
               const T* __restrict__ scale, cx_t<T>* __restrict__ cout, int count, GridDims g) {
   using C = cx_t<T>;
   constexpr int XL = W <= 8 ? 8 : 16;
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
     const C* at = fine + wrap1(s.x + (on ? rx : 0), g.nf[0]);
     C v[W];
 #pragma unroll
-    for (int a = 0; a < W; ++a) v[a] = __ldg(at + wrap1(s.y + a, g.nf[1]) * g.nf[0]);
+    for (int a = 0; a < W; ++a) v[a] = chain_load(at + wrap1(s.y + a, g.nf[1]) * g.nf[0]);
     if (k + 1 < turns) request(i + groups);
     T ar = 0, ai = 0;
 #pragma unroll
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
   const bool wrx = a.ntile[0] == 1, wry = a.ntile[1] == 1, wrz = DIM == 3 && a.ntile[2] == 1;
   const bool wrap = wrx || wry;
   const int4* __restrict__ vis = a.visits;
-  const C* __restrict__ cg = static_cast<const C*>(a.c);
+  const C* cg = static_cast<const C*>(a.c);
   const T* __restrict__ psi = static_cast<const T*>(a.psi);
   const int rx = lane % XL, ry = lane / XL;
   const int rxc = rx < W ? rx : W - 1;
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread(SpreadArgs a) {
 // cell), blockIdx.y = split unit - split0, partials summed in slot order (deterministic).
 template <typename T, int DIM>
 __global__ void __launch_bounds__(256)
-    k_reduce(const SplitUnit* __restrict__ split, const cx_t<T>* __restrict__ partial, cx_t<T>* __restrict__ fine,
+    k_reduce(const SplitUnit* __restrict__ split, const cx_t<T>* partial, cx_t<T>* __restrict__ fine,
              GridDims g, int TX, int TY, int TZ, int ntx, int nty, int ntz, int split0) {
   using C = cx_t<T>;
   const int ncell = TX * TY;
@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(256)
   for (; k + 4 <= st.nslots; k += 4) {
     C v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = __ldg(src + (long long)(k + q) * ncell);
+    for (int q = 0; q < 4; ++q) v[q] = chain_load(src + (long long)(k + q) * ncell);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       sr += v[q].x;
@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(256)
     }
   }
   for (; k < st.nslots; ++k) {
-    const C v = __ldg(src + (long long)k * ncell);
+    const C v = chain_load(src + (long long)k * ncell);
     sr += v.x;
     si += v.y;
   }
