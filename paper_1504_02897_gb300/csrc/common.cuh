@@ -190,7 +190,8 @@ struct Plan {
   void* d_deconv = nullptr;   // double [n0 + n1 + n2]: 1/psihat per axis, index j (0..n-1)
   void* d_deconv_x2 = nullptr;  // float2 [n1] (2D: [n0]): the y (x) factors as FP32 head + tail (FP32 plans)
   void* d_ones = nullptr;     // double [n0 + n1 + n2] of ones: the pad and crop of a split plan's smooth part
-  void* d_em1 = nullptr;      // T [nf0 + nf1 + nf2], split plans: e^{-k_d^2/k0^2} - 1 at the fine grid's modes
+  void* d_em1 = nullptr;      // WindowEntry<T> [nf0 + nf1 + nf2], split plans: e^{-k_d^2/k0^2} - 1 at the fine grid's
+                              // modes (window.cuh)
   void* d_ones_x2 = nullptr;  // float2 [n1] of (1, 0)
   void* d_fine = nullptr;     // cx [nf0 nf1 nf2]
   void* d_partial = nullptr;  // cx [nslots * tile cells]

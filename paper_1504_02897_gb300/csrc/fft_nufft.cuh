@@ -31,6 +31,7 @@
 // the pass starts, so they are read coherently (chain_load, common.cuh).
 #pragma once
 #include "fft_core.cuh"
+#include "window.cuh"
 
 namespace ddi {
 namespace {
@@ -292,8 +293,7 @@ struct ColZ : PolicyBase {
 //   p(k) = (1 - e^{-|k|^2/k0^2}) / |k|^2 * (3 (n.k)(m.k) - (n.m) |k|^2),  p(0) = 0,
 // times the inverse transform's 1 / (nf0 nf1 nf2).  Mode l of an axis with nf points is the
 // wavenumber (2 pi / (nf h)) l~ with l~ = l for l < nf/2, else l - nf.  e^{-|k|^2/k0^2} - 1 comes
-// from the plan's per-axis tables of e^{-k_d^2/k0^2} - 1 (FP64-built, rounded once), combined as
-// (1+a)(1+b) - 1 = a + b + a b: no expm1 per mode and no cancellation near k = 0.
+// from the plan's per-axis tables (window.cuh).
 template <typename T>
 struct SmoothSymbol {
   T dk[3];    // 2 pi / (nf_d h_d)
@@ -301,9 +301,8 @@ struct SmoothSymbol {
   T nm;       // n.m
   T inv_k02;  // 1 / k0^2
   T scale;    // 1 / (nf0 nf1 nf2)
-  const T* em1;  // [nf0 + nf1 + nf2]: e^{-k_d^2/k0^2} - 1
+  const WindowEntry<T>* em1;  // [nf0 + nf1 + nf2]: e^{-k_d^2/k0^2} - 1
   __host__ __device__ T k_of(int a, int l, int nf) const { return dk[a] * (T)(l < nf / 2 ? l : l - nf); }
-  __device__ static T join(T a, T b) { return (a + b) + a * b; }
   // em: e^{-|k|^2/k0^2} - 1
   __device__ T operator()(T kx, T ky, T kz, T em) const {
     const T k2 = (kx * kx + ky * ky) + kz * kz;
@@ -325,7 +324,7 @@ template <typename T>
 struct ZRef {
   int col;        // the column's (y, x) offset
   T kx, ky;       // the column's x and y wavenumbers
-  T em;           // e^{-(kx^2 + ky^2)/k0^2} - 1
+  WindowLine<T> em;  // e^{-(kx^2 + ky^2)/k0^2} - 1
   T w;            // 1 or 2
   int nyq;        // x is on its Nyquist line (and the column counts twice)
 };
@@ -342,12 +341,13 @@ struct SmoothZ : PolicyBase {
     const int ly = (int)((unsigned)L / (unsigned)g.ax.nf), lx = (int)L - ly * g.ax.nf;
     const bool twice = ly > 0 && 2 * ly < g.ay.nf;
     return Ref{ly * g.ax.nf + lx, sy.k_of(0, lx, g.ax.nf), sy.k_of(1, ly, g.ay.nf),
-               sy.join(sy.em1[lx], sy.em1[g.ax.nf + ly]), (T)(twice ? 2 : 1), twice && 2 * lx == g.ax.nf};
+               window_line(sy.em1[lx], sy.em1[g.ax.nf + ly]), (T)(twice ? 2 : 1), twice && 2 * lx == g.ax.nf};
   }
   __device__ C load(const Ref& r, int i) const { return chain_load(g.fine + (i * g.sz + r.col)); }
   __device__ C apply(const Ref& r, int i, C v) const {
     const T kz = sy.k_of(2, i, g.az.nf);
-    const T em = sy.join(r.em, __ldg(sy.em1 + g.ax.nf + g.ay.nf + i));
+    const C z = __ldg(reinterpret_cast<const C*>(sy.em1) + g.ax.nf + g.ay.nf + i);
+    const T em = window_join(r.em, WindowEntry<T>{z.x, z.y});
     T p = r.w * sy(r.kx, r.ky, kz, em);
     const bool nz = r.w > (T)1 && 2 * i == g.az.nf;
     if (r.nyq || nz) p = (T)0.5 * (p + r.w * sy(r.nyq ? -r.kx : r.kx, r.ky, nz ? -kz : kz, em));
@@ -457,7 +457,7 @@ int split_smooth_part(Plan& p, const T* rho, T* phi, cudaStream_t s) {
   const double* m = p.desc.axis_m;
   sy.nm = (T)((n[0] * m[0] + n[1] * m[1]) + n[2] * m[2]);
   sy.inv_k02 = (T)(1.0 / (p.desc.split_k0 * p.desc.split_k0));
-  sy.em1 = static_cast<const T*>(p.d_em1);
+  sy.em1 = static_cast<const WindowEntry<T>*>(p.d_em1);
   sy.scale = (T)(1.0 / ((double)p.nf[0] * (double)p.nf[1] * (double)p.nf[2]));
   DDI_TRY((dispatch_policy<T, -1, 16, 1024>(p, p.nf[1], PadY<T>{{}, g, rho}, s)));
   p.mark("smooth_pad_fft_y", s);

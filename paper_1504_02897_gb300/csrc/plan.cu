@@ -19,6 +19,7 @@
 #include <numeric>
 
 #include "common.cuh"
+#include "window.cuh"
 
 namespace ddi {
 
@@ -901,8 +902,8 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
   DDI_TRY(upload(p, &p.d_deconv_x2, dcx2, "deconvolution pairs", stream));
   std::vector<double> ones;
   std::vector<float2> ones2;
-  std::vector<double> em1;
-  std::vector<float> em1f;
+  std::vector<WindowEntry<double>> em1;
+  std::vector<WindowEntry<float>> em1f;
   if (p.split()) {
     ones.assign((size_t)p.n[0] + p.n[1] + p.n[2], 1.0);
     ones2 = pairs(ones);
@@ -911,9 +912,14 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
     for (int a = 0; a < 3; ++a)
       for (int l = 0; l < p.nf[a]; ++l) {
         const double k = (2.0 * M_PI / ((double)p.nf[a] * p.h[a])) * (double)(l < p.nf[a] / 2 ? l : l - p.nf[a]);
-        em1.push_back(std::expm1(-(k * k) / (d.split_k0 * d.split_k0)));
+        const double f = std::expm1(-(k * k) / (d.split_k0 * d.split_k0));
+        if (p.prec == DDI_FP64)
+          em1.push_back(window_entry<double>(f));
+        else
+          em1f.push_back(window_entry<float>(f));
       }
-    DDI_TRY(upload_real(p, &p.d_em1, em1, "window factors", stream, &em1f));
+    DDI_TRY(p.prec == DDI_FP64 ? upload(p, &p.d_em1, em1, "window factors", stream)
+                               : upload(p, &p.d_em1, em1f, "window factors", stream));
   }
   DDI_TRY(dev_alloc(p, (void**)&p.d_counter, 2 * sizeof(int), "unit counters"));
   DDI_TRY(dev_alloc(p, (void**)&p.d_nonfinite, sizeof(int), "non-finite record"));
