@@ -70,7 +70,8 @@ typedef struct {
   double nufft_tol;    /* requested NUFFT tolerance; 0 => 1e-13 (FP64) / 1e-6 (FP32) */
   int tile[3];         /* spread tile (x, y, z) in fine cells, >= w - 1 and dividing 2n (rounded to
                           such a size); 0 => built-in choice; tile[0] < 0 => picked by the
-                          spread-tile autotuner (ddi_tune_spread_tile) when the plan is created */
+                          spread autotuner when the plan is created (plans that spread by columns: the size
+                          of their work items) */
   int chunk;           /* max nodes per spread work item; 0 => built-in choice */
   double split_k0;     /* 3D only.  0 => the quadrature of Eq. DDI-Trun1 on the ball |k| <= kmax.
                           != 0 => the improved split algorithm of Sec. 2.1 (Eq. 3.9) with the window
@@ -136,7 +137,8 @@ typedef struct {
   double kmax;
   int nr, ntheta, nphi;
   size_t device_bytes; /* device memory held by the plan */
-  double spread_tuned_ms; /* spread time of the tile the autotuner picked, in ms; 0 if not tuned */
+  double spread_tuned_ms; /* time of the spread (and, in plans that interpolate by columns, of the interpolation)
+                             with the tile or work items that the autotuner picked, in ms; 0 if not tuned */
   double split_k0;     /* window width k0 of the split algorithm; 0 if the plan does not split */
   int ellipsoid;       /* 1 if the quadrature is the ellipsoidal rule */
   int band[2];         /* split plans: half-widths (x, y) of the band of fine-grid lines the ball's

@@ -11,7 +11,8 @@
 //
 // The autotuner picks the spread tile of a plan by timing the spread (with its
 // partial-plane reduction) for a list of candidate tiles on the plan's own node set and
-// keeping the fastest; for column plans it picks the visits per work unit.  The node positions on the fine grid depend only on the grid, the
+// keeping the fastest; for column plans it picks the visits per work unit, timing the
+// interpolation too where it goes by the same units.  The node positions on the fine grid depend only on the grid, the
 // quadrature sizes and kmax h, not on the box length or the dipole axes, so the result
 // is cached per such shape (and device) for the life of the process.
 #include <algorithm>
@@ -64,7 +65,9 @@ std::vector<std::array<int, 3>> tile_candidates(const Plan& p) {
 }  // namespace
 
 // Column plans have fixed columns; the tuner picks the number of visits per work unit
-// (more units balance the load better, fewer share fewer planes through partial slots).
+// (more units balance the load better, fewer share fewer planes through partial slots).  Timed is what
+// the units drive: the spread and, where the plan interpolates by columns too, the interpolation, which
+// prefers smaller units.  The built-in choice (0) is a candidate, so tuning is never behind it.
 int tune_column_chunk(Plan& p, cudaStream_t s) {
   const std::string key = tune_key_of(p) + " columns";
   std::unique_lock<std::mutex> lock(g_tune_mu);
@@ -77,15 +80,17 @@ int tune_column_chunk(Plan& p, cudaStream_t s) {
     p.tuned_ms = r.ms;
     return DDI_OK;
   }
-  int best = 0;
+  int best = 0, builtin = 0;
   double best_ms = 0.0;
-  for (const int c : {32, 64, 128, 192, 256, 384, 512}) {
+  for (const int c : {0, 32, 64, 128, 192, 256, 384, 512}) {
+    if (c > 0 && c == builtin) continue;
     p.desc.chunk = c;
     DDI_TRY(build_spread_col(p, s));
+    if (c == 0) builtin = p.chunk;
     float ms = 0.f;
     DDI_TRY(time_spread(p, s, 5, &ms));
     if (best == 0 || ms < best_ms) {
-      best = c;
+      best = p.chunk;
       best_ms = ms;
     }
   }

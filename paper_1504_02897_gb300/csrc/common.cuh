@@ -401,7 +401,7 @@ void set_tile(Plan& p, const int want[3]);         // tile rounded as for ddi_pl
 int build_spread(Plan& p, cudaStream_t stream);     // spread lists for the current tile
 int build_spread_col(Plan& p, cudaStream_t stream); // column (2D: block) spread lists for desc.chunk (plan.cu)
 bool columns_apply(const Plan& p);                   // the column spread fits the plan (plan.cu)
-int time_spread(Plan& p, cudaStream_t s, int reps, float* ms);  // best of reps (nufft.cu)
+int time_spread(Plan& p, cudaStream_t s, int reps, float* ms);  // what the lists drive, best of reps (nufft.cu)
 int tune_spread_tile(Plan& p, cudaStream_t s);      // autotuner (batch.cu)
 void destroy_plan(Plan& p);
 void fill_info(const Plan& p, ddi_plan_info* info);

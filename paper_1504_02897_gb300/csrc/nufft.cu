@@ -566,11 +566,13 @@ int configure_kernels(Plan& p) {
   return p.dim == 3 ? configure_spread_w<float, 3>(p, nullptr) : configure_spread_w<float, 2>(p, nullptr);
 }
 
-// Device time of the spread (and its partial-plane reduction) for the plan's current
-// tile: the best of `reps` timed launches after one untimed one, on zeroed node values
-// (the cost depends on the node set and the tile, not on the values).
+// Device time of what the plan's current work lists drive, the spread with its partial-plane
+// reduction and, in plans that interpolate by columns, the interpolation with its node sums:
+// the best of `reps` timed launches after one untimed one (the cost depends on the node set and
+// the lists, not on the values).
 int time_spread(Plan& p, cudaStream_t s, int reps, float* ms) {
   DDI_CUDA(cudaMemsetAsync(p.d_c, 0, p.cx_size() * (size_t)p.Mh, s));
+  if (p.col_interp) DDI_CUDA(cudaMemsetAsync(p.d_fine, 0, p.cx_size() * (size_t)p.fine_points(), s));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     if (e0) cudaEventDestroy(e0);
@@ -578,7 +580,8 @@ int time_spread(Plan& p, cudaStream_t s, int reps, float* ms) {
     return DDI_ERR_CUDA;
   }
   auto once = [&]() -> int {
-    DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, sizeof(int), s));
+    DDI_CUDA(cudaMemsetAsync(p.d_counter, 0, 2 * sizeof(int), s));
+    if (p.col_interp) DDI_TRY(launch_interp_col(p, s));
     if (p.spread_kind == DDI_SPREAD_COLUMNS) return spread_col(p, s, false);
     if (p.prec == DDI_FP64) return p.dim == 3 ? launch_spread_w<double, 3>(p, s) : launch_spread_w<double, 2>(p, s);
     return p.dim == 3 ? launch_spread_w<float, 3>(p, s) : launch_spread_w<float, 2>(p, s);
