@@ -100,15 +100,16 @@ typedef struct {
                           every line, as a plan without split_k0 does */
   int spread;          /* type-1 spreading scheme: 0 => automatic (columns where they apply, else plane
                           tiles); DDI_SPREAD_TILES => owner-computes tile planes in shared memory (`tile`,
-                          `chunk`); DDI_SPREAD_COLUMNS => columns of the fine grid whose planes along the
-                          last axis a warp accumulates in registers: 8 x 8 cells in x-y running along z
-                          (3D), 8 cells in x running along y and taken in blocks of 8 x 8 cells (2D).
-                          Applies to FP32 plans whose fine grid is a multiple of 8 in x and y and at least
-                          w + 7 cells in x and y (3D: and w in z), and not to compensated 2D plans;
-                          DDI_ERR_ARG otherwise; `chunk` = visits per work item.  The automatic choice also gives
-                          columns to FP64 3D plans of 2048 processed nodes and more whose fine grid
-                          fits (at least w + 7 cells in x and y, multiples of 8) and whose `tile` is
-                          left at 0 */
+                          `chunk`); DDI_SPREAD_COLUMNS => 3D: columns of 8 x 8 fine cells in x-y that run along
+                          z, whose planes a warp accumulates in registers; 2D: blocks of 8 x 8 fine cells.
+                          Asking for it applies to FP32 plans whose fine grid is a multiple of 8 in x and y
+                          and at least w + 7 cells in x and y (3D: and w in z), and not to compensated 2D
+                          plans; DDI_ERR_ARG otherwise; `chunk` = visits per work item.  The automatic choice
+                          also gives columns to FP64 3D plans of 2048 processed nodes and more whose fine
+                          grid fits and whose `tile` has no size of the caller's own (0, or < 0: tuned).
+                          `tile` is of no effect in FP32 plans that spread by columns; an FP32 2D plan above
+                          512 x 512 fine cells that gives a tile size (tile[0] or tile[1] > 0) takes tiles
+                          (items of a ddi_batch: blocks) */
   int check_finite;    /* NaN / Inf in rho: the pad pass of every evaluation records them in a device
                           flag of the plan (at no cost for finite input).  0 => ddi_apply stays
                           asynchronous and the flag is read by ddi_plan_check (and by ddi_apply_host,

@@ -749,10 +749,13 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
               kColX, kColY, kColX - 1);
     return DDI_ERR_ARG;
   }
-  // automatic choice: columns where they apply (2D: blocks of 8 x 8 cells, faster
-  // than the tiles at every size, see columns.cu)
+  // automatic choice: columns where they apply (2D: blocks of 8 x 8 cells, faster than the tiles at
+  // every size, see columns.cu; a 2D plan on its own above 512^2 fine cells takes tiles where the caller
+  // gives their size)
   p.batch_item = batch_item;
-  const bool columns2 = p.dim == 2 && columns_apply(p);
+  const bool own_tile = d.tile[0] > 0 || d.tile[1] > 0;
+  const bool columns2 = p.dim == 2 && columns_apply(p) &&
+                        !(own_tile && !batch_item && (long long)p.nf[0] * p.nf[1] > 512LL * 512);
   p.Mh = p.M / 2;  // one node of each (k, -k) pair
   p.spread_kind = d.spread == DDI_SPREAD_COLUMNS || (d.spread == DDI_SPREAD_AUTO && (columns2 || columns_auto3(p)))
                       ? DDI_SPREAD_COLUMNS
