@@ -85,7 +85,9 @@ int tune_column_chunk(Plan& p, cudaStream_t s) {
   for (const int c : {0, 32, 64, 128, 192, 256, 384, 512}) {
     if (c > 0 && c == builtin) continue;
     p.desc.chunk = c;
-    DDI_TRY(build_spread_col(p, s));
+    const int st = build_spread_col(p, s);
+    if (st == DDI_ERR_OOM && best != 0) continue;  // smaller items have longer lists
+    DDI_TRY(st);
     if (c == 0) builtin = p.chunk;
     float ms = 0.f;
     DDI_TRY(time_spread(p, s, 5, &ms));
@@ -267,24 +269,38 @@ int ddi_batch_create(ddi_batch* out, const ddi_plan_desc* descs, int count, int 
       return DDI_ERR_ARG;
     }
     *out = nullptr;
-    ddi_batch_s* b = new (std::nothrow) ddi_batch_s();
-    if (!b) {
-      ddi::set_error("host allocation failed");
-      return DDI_ERR_OOM;
-    }
-    b->flags = flags;
-    if (cudaGetDevice(&b->device) != cudaSuccess) {
-      cudaGetLastError();
-      delete b;
-      ddi::set_error("ddi_batch_create: no current device");
-      return DDI_ERR_CUDA;
-    }
-    try {
-      return build_batch(b, out, descs, count, flags, stream);
-    } catch (...) {
-      free_batch(b);  // the plans and streams built before the failure
-      throw;
-    }
+    auto create = [&](const ddi_plan_desc* ds) -> int {
+      ddi_batch_s* b = new (std::nothrow) ddi_batch_s();
+      if (!b) {
+        ddi::set_error("host allocation failed");
+        return DDI_ERR_OOM;
+      }
+      b->flags = flags;
+      if (cudaGetDevice(&b->device) != cudaSuccess) {
+        cudaGetLastError();
+        delete b;
+        ddi::set_error("ddi_batch_create: no current device");
+        return DDI_ERR_CUDA;
+      }
+      try {
+        return build_batch(b, out, ds, count, flags, stream);
+      } catch (...) {
+        free_batch(b);  // the plans and streams built before the failure
+        throw;
+      }
+    };
+    const int st = create(descs);
+    if (st != DDI_ERR_OOM) return st;
+    // the column lists of some items may have taken the memory that others need: once more with tiles, whose
+    // lists take a tenth, wherever the choice is the library's
+    std::vector<ddi_plan_desc> tiles(descs, descs + count);
+    bool changed = false;
+    for (ddi_plan_desc& d : tiles)
+      if (d.spread == DDI_SPREAD_AUTO && !(d.compensated && d.precision == DDI_FP32)) {
+        d.spread = DDI_SPREAD_TILES;
+        changed = true;
+      }
+    return changed ? create(tiles.data()) : st;
   });
 }
 

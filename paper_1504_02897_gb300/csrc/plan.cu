@@ -283,6 +283,18 @@ static bool columns_auto3(const Plan& p) {
   return columns_fit(p) && p.Mh >= 2048 && p.desc.tile[0] <= 0 && p.desc.tile[1] <= 0 && p.desc.tile[2] <= 0;
 }
 
+// Frees the column (block) lists of a plan, whole or half built.
+static void drop_column_lists(Plan& p) {
+  for (void** q : {(void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart,
+                   (void**)&p.d_cimage, (void**)&p.d_cnodes, &p.d_cshare, (void**)&p.d_cnoff, (void**)&p.d_cnpos})
+    if (*q) {
+      cudaFree(*q);
+      *q = nullptr;
+    }
+  p.bytes -= p.spread_bytes;
+  p.spread_bytes = 0;
+}
+
 // The groups' images and node lists on the device, made there from the visits (gvis: [group][32]
 // node or -1 and packed start), 3D: the runs and counts of each group.  Those lists are needed on
 // the device only while the images are made.
@@ -318,13 +330,7 @@ static int build_spread_block(Plan& p, cudaStream_t stream) {
   const int W = p.w, nfx = p.nf[0], nfy = p.nf[1];
   const int ncx = nfx / kColX, ncy = nfy / kColY, nblk = ncx * ncy;
   DDI_CUDA(cudaStreamSynchronize(stream));
-  for (void** q : {(void**)&p.d_cunits, (void**)&p.d_cred, &p.d_cpart, (void**)&p.d_cimage, (void**)&p.d_cnodes})
-    if (*q) {
-      cudaFree(*q);
-      *q = nullptr;
-    }
-  p.bytes -= p.spread_bytes;
-  p.spread_bytes = 0;
+  drop_column_lists(p);
   const size_t before = p.bytes;
   // f(block, packed start) for every block of node i
   auto for_blocks = [&](int64_t i, auto&& f) {
@@ -415,18 +421,11 @@ static int default_col_chunk(int prec, long long visits) {
 // boundaries, and the last unit of a column wraps onto the first) is a leading or trailing
 // plane of each of them: those go to partial slots and a reduce entry sums them in unit order;
 // every other plane is written by its one unit.  Every fine cell is written once per apply.
-int build_spread_col(Plan& p, cudaStream_t stream) {
-  if (p.dim == 2) return build_spread_block(p, stream);
+static int build_spread_col3(Plan& p, cudaStream_t stream) {
   const int W = p.w, nfx = p.nf[0], nfy = p.nf[1], nfz = p.nf[2];
   const int ncx = nfx / kColX, ncy = nfy / kColY, ncol = ncx * ncy;
   DDI_CUDA(cudaStreamSynchronize(stream));
-  for (void** q : {(void**)&p.d_cunits, (void**)&p.d_cred, (void**)&p.d_cslots, &p.d_cpart,
-                   (void**)&p.d_cimage, (void**)&p.d_cnodes, &p.d_cshare, (void**)&p.d_cnoff, (void**)&p.d_cnpos})
-    if (*q) {
-      cudaFree(*q);
-      *q = nullptr;
-    }
-  p.bytes -= p.spread_bytes;
+  drop_column_lists(p);
   const size_t before = p.bytes;
   // visits: key (column, first window-axis tap) and the packed entry
   auto span = [&](int l, int nf, int B, int* first) {  // blocks of B cells a footprint from l reaches
@@ -697,6 +696,29 @@ int build_spread_col(Plan& p, cudaStream_t stream) {
   return configure_kernels(p);
 }
 
+int build_spread_col(Plan& p, cudaStream_t stream) {
+  const size_t before = p.bytes - p.spread_bytes;
+  const int st = p.dim == 2 ? build_spread_block(p, stream) : build_spread_col3(p, stream);
+  if (st != DDI_OK) {
+    drop_column_lists(p);
+    p.bytes = before;
+  }
+  return st;
+}
+
+// The column lists, and where the automatic choice made the plan a column plan that the device has no room
+// for, or whose visits exceed the 32-bit lists, the tiles' lists instead, which take a tenth of the
+// memory (an image holds about 100 bytes a visit in FP32 and 180 in FP64, and a node has 3.5 to 8
+// visits).  Built last, when everything else the plan needs has been allocated.  Compensated plans have no
+// tile spread to fall back on.
+static int build_columns_or_tiles(Plan& p, cudaStream_t stream) {
+  const int st = build_spread_col(p, stream);
+  if ((st != DDI_ERR_OOM && st != DDI_ERR_ARG) || p.desc.spread != DDI_SPREAD_AUTO || p.col_comp) return st;
+  p.col_interp = false;
+  p.spread_kind = DDI_SPREAD_TILES;
+  return build_spread(p, stream);
+}
+
 // psi_d at tap t of node i, [node][3][w]: tap t sits at x = t - fr from the node, in fine cells;
 // axes past the plan's hold 1, 0, 0, ..
 template <typename T>
@@ -712,6 +734,29 @@ static __global__ void k_taps(const double* __restrict__ fr, T* __restrict__ psi
     if (z * z < 1.0) v = exp(beta * (sqrt((1.0 - z) * (1.0 + z)) - 1.0));
   }
   psi[q] = (T)v;
+}
+
+// The workspace of the GPE's entry points and of ddi_apply_host.
+static int alloc_gpe(Plan& p) {
+  const size_t rs = p.real_size(), cs = p.cx_size();
+  const size_t N = (size_t)p.grid_points();
+  DDI_TRY(dev_alloc(p, &p.d_psi1, cs * N, "gpe psi1"));
+  DDI_TRY(dev_alloc(p, &p.d_rho, rs * N, "gpe rho"));
+  DDI_TRY(dev_alloc(p, &p.d_phi, rs * N, "gpe phi"));
+  DDI_TRY(dev_alloc(p, &p.d_work, cs * N, "gpe work"));
+  DDI_TRY(dev_alloc(p, &p.d_work2, cs * N, "gpe work2"));
+  DDI_TRY(dev_alloc(p, &p.d_kin, cs * 2 * (p.n[0] + p.n[1] + p.n[2]), "kinetic tables"));
+  p.red_blocks = 1024;
+  DDI_TRY(dev_alloc(p, (void**)&p.d_red, sizeof(double) * 16 * (p.red_blocks + 1), "reductions"));
+  if (cudaMallocHost((void**)&p.h_red, sizeof(double) * 64) != cudaSuccess) {
+    cudaGetLastError();
+    set_error("cudaMallocHost failed");
+    return DDI_ERR_OOM;
+  }
+  DDI_TRY(dev_alloc(p, &p.d_io_in, rs * N, "host io in"));
+  DDI_TRY(dev_alloc(p, &p.d_io_out, rs * N, "host io out"));
+  p.gpe_ready = true;
+  return DDI_OK;
 }
 
 int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool gpe, bool batch_item) {
@@ -936,26 +981,8 @@ int create_plan(Plan& p, const ddi_plan_desc* desc_in, cudaStream_t stream, bool
   // the host vectors above die with this frame: finish the uploads first
   DDI_CUDA(cudaStreamSynchronize(stream));
   std::vector<double>().swap(p.quad.dirw);
-  DDI_TRY(p.spread_kind == DDI_SPREAD_COLUMNS ? build_spread_col(p, stream) : build_spread(p, stream));
-  if (!gpe) return DDI_OK;
-  const size_t N = (size_t)p.grid_points();
-  DDI_TRY(dev_alloc(p, &p.d_psi1, cs * N, "gpe psi1"));
-  DDI_TRY(dev_alloc(p, &p.d_rho, rs * N, "gpe rho"));
-  DDI_TRY(dev_alloc(p, &p.d_phi, rs * N, "gpe phi"));
-  DDI_TRY(dev_alloc(p, &p.d_work, cs * N, "gpe work"));
-  DDI_TRY(dev_alloc(p, &p.d_work2, cs * N, "gpe work2"));
-  DDI_TRY(dev_alloc(p, &p.d_kin, cs * 2 * (p.n[0] + p.n[1] + p.n[2]), "kinetic tables"));
-  p.red_blocks = 1024;
-  DDI_TRY(dev_alloc(p, (void**)&p.d_red, sizeof(double) * 16 * (p.red_blocks + 1), "reductions"));
-  if (cudaMallocHost((void**)&p.h_red, sizeof(double) * 64) != cudaSuccess) {
-    cudaGetLastError();
-    set_error("cudaMallocHost failed");
-    return DDI_ERR_OOM;
-  }
-  DDI_TRY(dev_alloc(p, &p.d_io_in, rs * N, "host io in"));
-  DDI_TRY(dev_alloc(p, &p.d_io_out, rs * N, "host io out"));
-  p.gpe_ready = true;
-  return DDI_OK;
+  if (gpe) DDI_TRY(alloc_gpe(p));
+  return p.spread_kind == DDI_SPREAD_COLUMNS ? build_columns_or_tiles(p, stream) : build_spread(p, stream);
 }
 
 namespace {
