@@ -299,13 +299,9 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 // which the compiler cannot schedule, 192^3 took 869 us instead of 852)
 template <typename V> __device__ __forceinline__ V chain_load(const V* p) { return *p; }
 
-// Raises the kernel's dynamic shared memory limit to `smem`, which is a constant of the kernel.  Set before
-// every launch: the limit belongs to the device's context, and a record kept here that it is set would outlive a
-// reset of that context (an attribute call takes less than a launch).
-inline int prepare_kernel(const void* fn, size_t smem) {
-  if (smem > 48 * 1024) DDI_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  return DDI_OK;
-}
+// Once per kernel and device: raises the kernel's dynamic shared memory limit to `smem` (the limit
+// belongs to the kernel, shared by every plan and thread: only raised).
+int prepare_kernel(const void* fn, size_t smem);
 
 template <typename... P, typename... A>
 int launch_chain(const Plan& p, void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,

@@ -1,10 +1,25 @@
 // The FP64-built twiddle tables of the Stockham FFTs (fft_core.cuh).
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <mutex>
 
 #include "common.cuh"
 
 namespace ddi {
+
+int prepare_kernel(const void* fn, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> done;  // (device, kernel) -> limit set
+  int dev = 0;
+  DDI_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = done.find({dev, fn});
+  if (it != done.end() && it->second >= smem) return DDI_OK;
+  if (smem > 48 * 1024) DDI_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  done[{dev, fn}] = smem;
+  return DDI_OK;
+}
 
 int make_twiddles(Plan& p, int n) {
   if (twiddles(p, n)) return DDI_OK;
