@@ -25,8 +25,6 @@
 // 128 registers; 5 CTAs at 96 spill and take 118); 192^3 FP32 564 -> 277 us; 128^3 FP64 27.4 ->
 // 2.6 ms (the FP64 operations above take 2.3 ms at this part's rate).
 #include <algorithm>
-#include <cstring>
-#include <mutex>
 
 #include "columns.cuh"
 
@@ -34,8 +32,6 @@ namespace ddi {
 namespace {
 
 constexpr int kColThreads3 = 128;  // 4 warps per CTA, each taking units on its own
-
-template <typename T> using p2_t = cx_t<T>;
 
 // c + a b per component
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -607,7 +603,16 @@ __global__ void __launch_bounds__(kColThreads3, sizeof(T) == 4 ? 4 : 2) k_interp
         }
         while (zl < sr + W) {
           switch (zslot) {
-#define DDI_PUT3(R)                                                                  case R:                                                                              if constexpr (R < W) {                                                               constexpr int Q = R / 2;                                                           if constexpr (R % 2 == 0)                                                            r0[Q].x = p0.x, i0[Q].x = p0.y, r1[Q].x = p1.x, i1[Q].x = p1.y;                  else                                                                                 r0[Q].y = p0.x, i0[Q].y = p0.y, r1[Q].y = p1.x, i1[Q].y = p1.y;                }                                                                                  break;
+#define DDI_PUT3(R)                                                      \
+  case R:                                                                \
+    if constexpr (R < W) {                                               \
+      constexpr int Q = R / 2;                                           \
+      if constexpr (R % 2 == 0)                                          \
+        r0[Q].x = p0.x, i0[Q].x = p0.y, r1[Q].x = p1.x, i1[Q].x = p1.y;  \
+      else                                                               \
+        r0[Q].y = p0.x, i0[Q].y = p0.y, r1[Q].y = p1.x, i1[Q].y = p1.y;  \
+    }                                                                    \
+    break;
             DDI_COL3_CASES(DDI_PUT3)
 #undef DDI_PUT3
           }

@@ -1,7 +1,8 @@
-// Stockham FFT core shared by the plain axis passes (fft.cu) and the pruned/fused NUFFT
-// passes (fft_nufft.cu): in-register radix-16/8/4/2/3 DFTs, the Stockham stage loop over a
-// padded shared-memory line, and a CTA-level kernel that moves LPB lines between global
-// memory and shared memory through a load/store policy.
+// Stockham FFT core shared by the pruned and fused NUFFT passes (fft_nufft.cuh) and the GPE's
+// passes (gpe_fft.cuh): in-register radix-16/12/8/4/2/3 DFTs, the Stockham stage loop over a
+// padded shared-memory line, and CTA-level kernels that take LPB lines from and to global memory
+// through a load/store policy, one transform a pass (k_fft_policy) or forward and inverse in one
+// (k_fft_pair).
 #pragma once
 #include <cmath>
 
@@ -478,6 +479,7 @@ template <typename T, int N, int DIR, typename P>
 int launch_policy(const Plan& p, const P& pol, cudaStream_t s) {
   constexpr int LPB = lines_per_cta<T, N, P::kStrided>();
   constexpr int threads = LPB * Shape<N>::TPL;
+  static_assert(P::kStrided || threads % 32 == 0, "a CTA of contiguous lines is whole warps");
   const size_t smem = (size_t)LPB * Shape<N>::LS * sizeof(cx_t<T>);
   void (*kern)(P, const cx_t<T>*);
   if constexpr (DIR == 0)

@@ -40,7 +40,6 @@ using namespace fftcore;
 struct Axis {
   int n;   // grid points
   int nf;  // fine points
-  __host__ __device__ bool in_block(int l) const { return l < n / 2 || l >= nf - n / 2; }
   // grid index j (0..n-1) of fine position l in the block
   __host__ __device__ int grid_of(int l) const { return l < n / 2 ? l + n / 2 : l - (nf - n / 2); }
   // fine position of grid index j

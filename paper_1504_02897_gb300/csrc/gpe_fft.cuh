@@ -210,15 +210,11 @@ struct GfChangeX : GpePolicy {
     if (threadIdx.x == 0) top = 0;
     __syncthreads();
     T m = a.m;
-    if (blockDim.x % 32 == 0) {
-      for (int o = 16; o > 0; o >>= 1) {
-        const T q = __shfl_xor_sync(0xffffffffu, m, o);
-        m = q > m ? q : m;
-      }
-      if (threadIdx.x % 32 == 0) atomicMax(&top, (unsigned long long)__double_as_longlong((double)m));
-    } else {
-      atomicMax(&top, (unsigned long long)__double_as_longlong((double)m));
+    for (int o = 16; o > 0; o >>= 1) {  // CTAs of contiguous lines are whole warps (launch_policy)
+      const T q = __shfl_xor_sync(0xffffffffu, m, o);
+      m = q > m ? q : m;
     }
+    if (threadIdx.x % 32 == 0) atomicMax(&top, (unsigned long long)__double_as_longlong((double)m));
     __syncthreads();
     if (threadIdx.x == 0) atomicMax(change, top);
   }

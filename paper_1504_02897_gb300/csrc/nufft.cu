@@ -13,7 +13,7 @@
 //   psi(x) = exp(beta (sqrt(1 - (2x/w)^2) - 1)), |x| < w/2 (x in fine cells),
 // with deconvolution by its Fourier transform psihat(2 pi j'/nf).  The nodes are fixed by
 // the plan, so the per-axis kernel values psi_d(l - s_q) of every node are built once
-// (FP64 on the host, rounded to the working precision) and read here.
+// (k_taps, plan.cu: in FP64, rounded to the working precision) and read here.
 //
 // Launches (fft_nufft.cuh holds the FFT passes, columns.cu the column and block kernels):
 //   forward FFT (3D: y with pad + deconvolution fused, x, z; 2D: x, y), pruned to the padded
@@ -31,11 +31,7 @@
 //   inverse FFT (3D: z, x, y; 2D: y, x), pruned likewise; the last pass fused with crop,
 //               deconvolution and real part
 #include <algorithm>
-#include <climits>
-#include <cmath>
-#include <cstddef>
 #include <mutex>
-#include <utility>
 
 #include "common.cuh"
 

@@ -276,7 +276,8 @@ bool columns_apply(const Plan& p) {
 
 // Whether a plan spreads by columns on its own choice (desc.spread == DDI_SPREAD_AUTO).  FP32:
 // wherever they apply in 3D.  FP64, 3D, without a tile size of the caller's own: from 2048
-// processed nodes up, where there are enough units to fill the device.
+// processed nodes up, where there are enough units to fill the device (whole DDI at 2048 nodes, columns
+// against tiles: 16^3 152 and 1003 us, 32^3 212 and 1051, 48^3 285 and 923).
 static bool columns_auto3(const Plan& p) {
   if (p.dim != 3) return false;
   if (p.prec == DDI_FP32) return columns_apply(p);
@@ -388,7 +389,8 @@ static int build_spread_block(Plan& p, cudaStream_t stream) {
   p.ncunits = (int)units.size();
   p.ncslots = nslot;
   p.ncred = (int)red.size();
-  // entries of more than 24 slots first: a CTA sums each of them
+  // entries of more than 24 slots first: a CTA sums each of them (whole DDI at 512^2 and 1024^2: from 8
+  // slots 104 and 316 us, from 24 105 and 316, from 96 110 and 322)
   p.ncred_long = (int)(std::stable_partition(red.begin(), red.end(), [](const ColRed& r) { return r.ns > 24; }) -
                        red.begin());
   DDI_TRY(upload_images(p, gvis, nullptr, nullptr, stream));
@@ -654,7 +656,8 @@ static int build_spread_col3(Plan& p, cudaStream_t stream) {
   p.chunk = cap;
   p.ncunits = (int)units.size();
   p.ncred = (int)red.size();
-  // entries of more than 24 slots first: a CTA sums each of them
+  // entries of more than 24 slots first: a CTA sums each of them (whole DDI at 128^3 FP32: from 8 slots
+  // 269 us, from 24 270, from 96 275)
   p.ncred_long = (int)(std::stable_partition(red.begin(), red.end(), [](const ColRed& r) { return r.ns > 24; }) -
                        red.begin());
   p.ncslots = nslot;
@@ -666,8 +669,10 @@ static int build_spread_col3(Plan& p, cudaStream_t stream) {
     return DDI_ERR_ARG;
   }
   // FP64: the gather kernel costs twice the FP64 operations (64^3: 748 us against 400, 128^3 5.9 ms
-  // against 2.5).  FP32: below 2^18 processed nodes its one launch is the shorter (24^3 10 us
-  // against 17, 96x64x48 with 221184 nodes 55 against 54, 128^3 with 524288 133 against 112)
+  // against 2.5).  FP32: with few nodes the gather's one launch is the shorter, with many the columns
+  // (whole DDI, gather against columns: 32768 nodes 49 and 53 us, 65536 66 and 68, 102400 85 and 84,
+  // 221184 126 and 118 at 96x64x48 or 148 and 145 at 96^3; 128^3 with 524288, the kernels alone, 133 and
+  // 112).  The line at 2^18 is on the safe side of where they cross
   p.col_interp = p.prec == DDI_FP64 || p.Mh >= (1 << 18);
   // where each node's visits are: their interpolation shares are summed in this order
   if (p.col_interp) {
