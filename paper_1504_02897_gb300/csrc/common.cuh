@@ -282,8 +282,8 @@ struct Plan {
 // holds them until that kernel has completed and its writes are visible.  Every such kernel calls
 // chain_wait() in all its threads before it touches what an evaluation writes (or anything a
 // caller's work on the stream may still use), so completion carries over along the chain.  Saves
-// the launch gap of each of the 9-14 kernels: 24^3 50 -> 40 us, 128^3 304 -> 281 us, four 128^3 steps
-// 1525 -> 1385 us.  Not used inside batches, whose side streams fill the gaps, nor in FP64, whose
+// the launch gap of each of the 9-14 kernels: 24^3 49 -> 36 us, 96x64x48 138 -> 127 us, 128^3 293 -> 270
+// us, 256^3 split 1154 -> 1128 us, four 128^3 steps 1479 -> 1349 us.  Not used inside batches, whose side streams fill the gaps, nor in FP64, whose
 // kernels are long (128^3 6.73 against 6.75 ms; rotating 64^3 steps were slower with it, 2.95
 // against 2.72 ms).
 //
